@@ -51,6 +51,21 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void 
         : "memory");
 }
 
+// A consumer's wait for tile k in slot k % S of the ring.  A group takes every NG-th tile, so
+// the tile before k in that slot, k - S, is another group's, and its load can still be in
+// flight here (loads complete out of order: the group's own last tile, k - NG, can land
+// first).  A wait by parity for tile k would then take the phase before k - S's, which has the
+// parity of k's and is complete, for its own: the group would march a slot that holds no
+// tile yet, and the ring's phases would be lost from there on.  So the phase of tile k - S
+// is waited for first; the one before it is complete, because the load of tile k - S was
+// issued (in order, before that of k - NG) only after tile k - 2 S was marched.
+template <int S> __device__ __forceinline__ bool wait_tile(uint64_t *full, unsigned k)
+{
+    uint64_t *bar = full + k % S;
+    const unsigned phase = (k / S) & 1u;
+    return (k < unsigned(S) || mbar_wait_bounded(bar, phase ^ 1u)) && mbar_wait_bounded(bar, phase);
+}
+
 // thread groups (256 columns each) marching tiles at once; the ring holds one slot more
 template <int L> constexpr int tile_groups() { return L <= 48 ? 3 : 2; }
 template <int L> constexpr unsigned tile_bytes() { return unsigned(L) * 1024u; }
@@ -222,7 +237,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     const int coff = unit * 32 + (((e >> 2) ^ (unit & 7)) << 2) + (e & 3);
     bool bad = false;
     for (unsigned k = grp; k < n_my; k += NG) {
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[k % S], (k / S) & 1u))) {
+        if (!__all_sync(0xffffffffu, wait_tile<S>(full, k))) {
             atomicOr(a.err, ERR_TIMEOUT);
             return;
         }
@@ -461,7 +476,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     float *wi = winv + (grp * 8 + w) * 2 * L;
     bool bad = false;
     for (unsigned k = grp; k < n_my; k += NG) {
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[k % S], (k / S) & 1u))) {
+        if (!__all_sync(0xffffffffu, wait_tile<S>(full, k))) {
             atomicOr(a.err, ERR_TIMEOUT);
             return;
         }

@@ -226,8 +226,8 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
         bulk_wait_all();
         if (!ok) {
             atomicOr(a.err, ERR_TIMEOUT);
-            // let the loads in flight land before the CTA exits
-            for (unsigned j = 0; j < loaded; ++j) mbar_wait_bounded(&full[j % 3], (j / 3) & 1u);
+            // let the loads in flight (the last three at most) land before the CTA exits
+            for (unsigned j = loaded > 3 ? loaded - 3 : 0; j < loaded; ++j) mbar_wait_bounded(&full[j % 3], (j / 3) & 1u);
         }
         return;
     }

@@ -51,19 +51,19 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void 
         : "memory");
 }
 
-// A consumer's wait for tile k in slot k % S of the ring.  A group takes every NG-th tile, so
-// the tile before k in that slot, k - S, is another group's, and its load can still be in
-// flight here (loads complete out of order: the group's own last tile, k - NG, can land
-// first).  A wait by parity for tile k would then take the phase before k - S's, which has the
-// parity of k's and is complete, for its own: the group would march a slot that holds no
-// tile yet, and the ring's phases would be lost from there on.  So the phase of tile k - S
-// is waited for first; the one before it is complete, because the load of tile k - S was
-// issued (in order, before that of k - NG) only after tile k - 2 S was marched.
+// Tile k sits in slot k % S and its load completes a phase of barrier k % 2S: two barriers per
+// slot, taken in turn.  A group takes every NG-th tile, so the tile before k in its slot,
+// k - S, is another group's, and its load can still be in flight when the group waits for
+// tile k (loads complete out of order: the group's own last tile, k - NG, can land first).
+// With one barrier per slot a wait by parity then took the phase before k - S's, which has
+// the parity of k's, for its own, and the group marched a slot that held no tile yet.  The
+// phase before k's on its own barrier is tile k - 2S's, complete because the load of k - S was
+// issued (in order, before that of k - NG) only after tile k - 2S was marched; and tile k + 2S
+// cannot be loaded before tile k is marched.
+template <int S> __device__ __forceinline__ uint64_t *full_bar(uint64_t *full, unsigned k) { return full + k % (2 * S); }
 template <int S> __device__ __forceinline__ bool wait_tile(uint64_t *full, unsigned k)
 {
-    uint64_t *bar = full + k % S;
-    const unsigned phase = (k / S) & 1u;
-    return (k < unsigned(S) || mbar_wait_bounded(bar, phase ^ 1u)) && mbar_wait_bounded(bar, phase);
+    return mbar_wait_bounded(full_bar<S>(full, k), (k / (2 * S)) & 1u);
 }
 
 // thread groups (256 columns each) marching tiles at once; the ring holds one slot more
@@ -77,8 +77,9 @@ template <int L> constexpr int tile_slots()
                ? (196608 / tile_bytes<L>() > 12 ? 12 : int(196608 / tile_bytes<L>()))
                : tile_groups<L>() + 1;
 }
-// barriers (256 B), the velocity-column table, alignment to 1 KB, the ring
-constexpr size_t kTileHeader = 256 + kMaxVel * sizeof(LineCoefT<float>);
+// barriers, the velocity-column table, alignment to 1 KB, the ring
+constexpr size_t kTileBars = 384; // bytes of barriers
+constexpr size_t kTileHeader = kTileBars + kMaxVel * sizeof(LineCoefT<float>);
 template <int L> constexpr size_t tile_smem() { return kTileHeader + 1024 + size_t(tile_slots<L>()) * tile_bytes<L>(); }
 
 // March the periodic line p[0], p[st], ..., p[(L - 1) st] (flow toward +index) in place;
@@ -159,19 +160,17 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     constexpr int NG = tile_groups<L>(), S = tile_slots<L>(), NT = NG * 256;
     constexpr unsigned TB = tile_bytes<L>();
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem); // S: the slot holds its tile
-    uint64_t *done = full + S;                           // S: the tile's group is done with it
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem); // 2S: the slot holds its tile (full_bar)
+    uint64_t *done = full + 2 * S;                           // S: the tile's group is done with it
     uint64_t *marched = done + S;                        // NG: every column of the group's tile is marched
-    LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + 256);
-    static_assert((2 * S + NG) * 8 <= 256, "barriers fit ahead of the table");
+    LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + kTileBars);
+    static_assert((3 * S + NG) * 8 <= int(kTileBars), "barriers fit ahead of the table");
     unsigned char *ring = smem + kTileHeader + ((1024u - ((smem_u32(smem) + unsigned(kTileHeader)) & 1023u)) & 1023u);
     auto slot = [&](unsigned k) { return reinterpret_cast<float *>(ring + size_t(TB) * (k % S)); };
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&done[s], 256);
-        }
+        for (int s = 0; s < 2 * S; ++s) mbar_init(&full[s], 1);
+        for (int s = 0; s < S; ++s) mbar_init(&done[s], 256);
         for (int g = 0; g < NG; ++g) mbar_init(&marched[g], 256);
         fence_barrier_init();
     }
@@ -193,8 +192,9 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         auto load = [&](unsigned k) {
             int u0, o;
             coords(k, u0, o);
-            mbar_arrive_expect_tx(&full[k % S], TB);
-            tma_load_4d(slot(k), &map, &full[k % S], 0, u0, 0, o);
+            uint64_t *bar = full_bar<S>(full, k);
+            mbar_arrive_expect_tx(bar, TB);
+            tma_load_4d(slot(k), &map, bar, 0, u0, 0, o);
         };
         unsigned loaded = 0;
         for (; loaded < unsigned(S) && loaded < n_my; ++loaded) load(loaded);
@@ -216,7 +216,8 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         bulk_wait_all();
         if (!ok) {
             atomicOr(a.err, ERR_TIMEOUT);
-            for (unsigned k = 0; k < loaded; ++k) mbar_wait_bounded(&full[k % S], (k / S) & 1u);
+            // let the loads in flight (the last S at most) land before the CTA exits
+            for (unsigned k = loaded > unsigned(S) ? loaded - S : 0; k < loaded; ++k) wait_tile<S>(full, k);
         }
         return;
     }
@@ -399,9 +400,9 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     constexpr unsigned CB = tile16_codes<L>(), SB = tile16_slot<L, NZ>();
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);
-    uint64_t *done = full + S;
-    LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + 256);
-    static_assert(2 * S * 8 <= 256, "barriers fit ahead of the table");
+    uint64_t *done = full + 2 * S;
+    LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + kTileBars);
+    static_assert(3 * S * 8 <= int(kTileBars), "barriers fit ahead of the table");
     unsigned char *ring = smem + kTileHeader + ((1024u - ((smem_u32(smem) + unsigned(kTileHeader)) & 1023u)) & 1023u);
     auto slot = [&](unsigned k) { return reinterpret_cast<T *>(ring + size_t(SB) * (k % S)); };
     auto sslot = [&](unsigned k) { return reinterpret_cast<float *>(ring + size_t(SB) * (k % S) + CB); };
@@ -409,10 +410,8 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     static_assert(tile16_smem<L, NZ>() <= 227 * 1024, "the tiles and inverse scales fit shared memory");
 
     if (threadIdx.x == 0) {
-        for (int q = 0; q < S; ++q) {
-            mbar_init(&full[q], 1);
-            mbar_init(&done[q], 256);
-        }
+        for (int q = 0; q < 2 * S; ++q) mbar_init(&full[q], 1);
+        for (int q = 0; q < S; ++q) mbar_init(&done[q], 256);
         fence_barrier_init();
     }
     for (int j = threadIdx.x; j < a.nvel; j += blockDim.x) tab[j] = a.table[j];
@@ -434,9 +433,10 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         auto load = [&](unsigned k) {
             int u0, o;
             coords(k, u0, o);
-            mbar_arrive_expect_tx(&full[k % S], CB + unsigned(L) * 4u * unsigned(SX));
-            tma_load_4d(slot(k), &map, &full[k % S], 0, u0, 0, o);
-            tma_load_3d(sslot(k), &smap, &full[k % S], line0(u0), 0, o);
+            uint64_t *bar = full_bar<S>(full, k);
+            mbar_arrive_expect_tx(bar, CB + unsigned(L) * 4u * unsigned(SX));
+            tma_load_4d(slot(k), &map, bar, 0, u0, 0, o);
+            tma_load_3d(sslot(k), &smap, bar, line0(u0), 0, o);
         };
         unsigned loaded = 0;
         for (; loaded < unsigned(S) && loaded < n_my; ++loaded) load(loaded);
@@ -458,7 +458,8 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         bulk_wait_all();
         if (!ok) {
             atomicOr(a.err, ERR_TIMEOUT);
-            for (unsigned k = 0; k < loaded; ++k) mbar_wait_bounded(&full[k % S], (k / S) & 1u);
+            // let the loads in flight (the last S at most) land before the CTA exits
+            for (unsigned k = loaded > unsigned(S) ? loaded - S : 0; k < loaded; ++k) wait_tile<S>(full, k);
         }
         return;
     }

@@ -133,31 +133,10 @@ __device__ __forceinline__ X march_stream(const Lim<X> &lim, unsigned e, unsigne
     // "simple" when c R + R - 1 + LA < L); the rest row by row.
     if (!NEG) {
         constexpr int LA = 2;
-        // window c_{i-2} .. c_{i+2}, donor c_i
-        X cm2, cm1, c0 = s0, cp1 = s1, dcur, dm4m, Fm;
-        const X dm = curv(p2, p1, s0);
-        const X d0 = curv(p1, s0, s1);
-        dm4m = dm4(dm, d0);
-        if (PERIODIC) Fm = sl_mpp5_flux(lim, p3, p2, p1, s0, s1, dm4(curv(p3, p2, p1), dm), dm4m);
-        else Fm = zero;
-        cm2 = p2;
-        cm1 = p1;
-        dcur = d0;
-        auto face = [&](X cp2, T *dst, const float *dsc) {
-            const X dn = curv(c0, cp1, cp2);
-            const X dm4p = dm4(dcur, dn);
-            const X F = sl_mpp5_flux(lim, cm2, cm1, c0, cp1, cp2, dm4m, dm4p);
-            const X out = vadd(c0, vsub(Fm, F));
-            LN::store(dst, out, dsc, rng);
-            sum = vadd(sum, out);
-            cm2 = cm1;
-            cm1 = c0;
-            c0 = cp1;
-            cp1 = cp2;
-            dcur = dn;
-            dm4m = dm4p;
-            Fm = F;
-        };
+        March<X> m(lim);
+        if (PERIODIC) m.start_periodic(p3, p2, p1, s0, s1);
+        else m.start_zero(s0, s1);
+        auto face = [&](X cp2, T *dst, const float *dsc) { LN::store(dst, m.face(cp2), dsc, rng); };
         const int nsimple = (L - LA + 1) / R - 1 > 0 ? (L - LA + 1) / R - 1 : 0;
         for (int c = 0; c < nsimple; ++c) {
             T *cur = slot_ptr(ec + unsigned(c)) + coff;
@@ -183,42 +162,46 @@ __device__ __forceinline__ X march_stream(const Lim<X> &lim, unsigned e, unsigne
                 cp2 = PERIODIC ? (r == L ? s0 : s1) : zero;
             }
             if (!PERIODIC && i == L - 1) {
-                // outer velocity face: nothing crosses it
-                const X out = vadd(c0, Fm);
-                LN::store(row_ptr(i), out, srow_ptr(i), rng);
-                sum = vadd(sum, out);
+                LN::store(row_ptr(i), m.last(), srow_ptr(i), rng); // outer velocity face: nothing crosses it
             } else {
                 face(cp2, row_ptr(i), srow_ptr(i));
             }
             if (i % R == R - 1 || i == L - 1) release(ec + unsigned(i / R));
         }
+        sum = m.sum;
     } else {
         constexpr int LA = 3;
-        // window c_{i-1} .. c_{i+3}, donor c_{i+1}, flux toward -index
-        // curvatures are summed in the marching order (toward -index), as every kernel
-        // that walks a line with a negative Courant number from its far end sums them
+        // window c_{i-1} .. c_{i+3}, donor c_{i+1}, flux toward -index.  Differences and
+        // curvatures are those of a march that walks the line from its far end (downstream
+        // cell minus upstream cell), as every other kernel walks a negative Courant number:
+        // g_k = c_k - c_{k+1}, d_k = g_{k-1} - g_k.
+        const X half = splat<X>(0.5);
         const X s2 = LN::load(row_ptr(2), srow_ptr(2));
-        const X dmn = curv(s0, p1, p2); // d_{-1}
-        const X d0 = curv(s1, s0, p1);
-        const X d1 = curv(s2, s1, s0);
-        X dm4a = dm4(d0, d1);           // limited curvature at face i+1/2
-        X Fm;                            // mass moving left through face i-1/2
-        if (PERIODIC) Fm = sl_mpp5_flux(lim, s2, s1, s0, p1, p2, dm4a, dm4(dmn, d0));
+        X gm = vsub(p1, s0), g0 = vsub(s0, s1), g1 = vsub(s1, s2); // g_{i-1}, g_i, g_{i+1}
+        X hm = vmul(half, gm), h0 = vmul(half, g0);
+        const X dm1 = vsub(vsub(p2, p1), gm), d0 = vsub(gm, g0); // curvatures of cells -1, 0
+        X d1 = vsub(g0, g1);                                     // of cell i + 1
+        X qa = limited_curv(d0, d1);                             // at face i + 1/2
+        X Fm; // mass moving left through face i - 1/2
+        if (PERIODIC) Fm = sl_mpp5_flux(lim, s0, g1, g0, gm, vsub(p2, p1), h0, hm, qa, limited_curv(dm1, d0));
         else Fm = zero;
-        X cm1 = p1, c0 = s0, cp1 = s1, cp2 = s2, d_1 = d1;
+        X c0 = s0, cp1 = s1, cp2 = s2;
         auto face = [&](X cp3, T *dst, const float *dsc) {
-            const X d_2 = curv(cp3, cp2, cp1);
-            const X dm4b = dm4(d_1, d_2); // face i+3/2
-            const X F = sl_mpp5_flux(lim, cp3, cp2, cp1, c0, cm1, dm4b, dm4a);
+            const X g2 = vsub(cp2, cp3), d2 = vsub(g1, g2), h1 = vmul(half, g1);
+            const X qb = limited_curv(d1, d2); // face i + 3/2
+            const X F = sl_mpp5_flux(lim, cp1, g2, g1, g0, gm, h1, h0, qb, qa);
             const X out = vadd(c0, vsub(F, Fm));
             LN::store(dst, out, dsc, rng);
             sum = vadd(sum, out);
-            cm1 = c0;
             c0 = cp1;
             cp1 = cp2;
             cp2 = cp3;
-            d_1 = d_2;
-            dm4a = dm4b;
+            gm = g0;
+            g0 = g1;
+            g1 = g2;
+            h0 = h1;
+            d1 = d2;
+            qa = qb;
             Fm = F;
         };
         const int nsimple = (L - LA + 1) / R - 1 > 0 ? (L - LA + 1) / R - 1 : 0;

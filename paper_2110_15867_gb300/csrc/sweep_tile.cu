@@ -89,38 +89,26 @@ template <int L> constexpr size_t tile_smem() { return kTileHeader + 1024 + size
 // sign).  Returns the sum of the new values.
 // Faces marched per loop iteration: lines up to 32 cells unroll completely; longer lines
 // in blocks of 8 faces, so that the code of a march stays inside the instruction cache.
-template <int L> constexpr int march_unroll() { return L <= 32 ? L : 8; }
+template <int L> constexpr int march_block() { return L <= 32 ? L - 2 : 8; }
 
 template <int L, int DIR>
 __device__ __forceinline__ float march_tile(float *p, int st_rt, const Lim<float> &lim)
 {
     const int st = DIR == 0 ? st_rt : DIR * 256; // rows are 256 floats apart
-    const float a = p[(L - 3) * st], b = p[(L - 2) * st], c = p[(L - 1) * st];
     const float s0 = p[0], s1 = p[st];
-    const float dmm = curv(a, b, c), dm = curv(b, c, s0), d0 = curv(c, s0, s1);
-    float dm4m = dm4(dm, d0);
-    float Fm = sl_mpp5_flux(lim, a, b, c, s0, s1, dm4(dmm, dm), dm4m); // face -1/2, donor c_{-1}
-    float cm2 = b, cm1 = c, c0 = s0, cp1 = s1, dcur = d0, sum = 0.f;
-    auto face = [&](float cp2, float *dst) {
-        const float dn = curv(c0, cp1, cp2);
-        const float dm4p = dm4(dcur, dn);
-        const float F = sl_mpp5_flux(lim, cm2, cm1, c0, cp1, cp2, dm4m, dm4p);
-        const float out = c0 + (Fm - F);
-        *dst = out;
-        sum += out;
-        cm2 = cm1;
-        cm1 = c0;
-        c0 = cp1;
-        cp1 = cp2;
-        dcur = dn;
-        dm4m = dm4p;
-        Fm = F;
-    };
-#pragma unroll march_unroll<L>()
-    for (int i = 0; i < L - 2; ++i) face(p[(i + 2) * st], p + i * st);
-    face(s0, p + (L - 2) * st); // the last two faces take the first two cells' old values
-    face(s1, p + (L - 1) * st);
-    return sum;
+    March<float> m(lim);
+    m.start_periodic(p[(L - 3) * st], p[(L - 2) * st], p[(L - 1) * st], s0, s1);
+    constexpr int B = march_block<L>();
+#pragma unroll 1
+    for (int b = 0; b < (L - 2) / B; ++b, p += B * st)
+#pragma unroll
+        for (int q = 0; q < B; ++q) p[q * st] = m.face(p[(q + 2) * st]);
+    constexpr int R = (L - 2) % B; // faces left before the last two
+#pragma unroll
+    for (int q = 0; q < R; ++q) p[q * st] = m.face(p[(q + 2) * st]);
+    p[R * st] = m.face(s0); // the last two faces take the first two cells' old values
+    p[(R + 1) * st] = m.face(s1);
+    return m.sum;
 }
 
 // The logical 16-byte chunks lane and lane + 32 of a swizzled 1-KB row (chunk j of unit u
@@ -326,32 +314,21 @@ __device__ __forceinline__ float march_tile16(T *p, const float *sp, const float
     const int ss = DIR == 0 ? (st_rt > 0 ? SX : -SX) : DIR * SX; // and SX scales
     const int is = DIR == 0 ? (st_rt > 0 ? 1 : -1) : DIR;     // and 1 inverse scale
     auto get = [&](int i) { return RegCodec<T>::get(p[i * st], sp[i * ss]); };
-    const float a = get(L - 3), b = get(L - 2), c = get(L - 1);
+    auto put = [&](int i, float v) { p[i * st] = RegCodec<T>::put(v, ip[i * is], lcg_next(rng) >> 16); };
     const float s0 = get(0), s1 = get(1);
-    const float dmm = curv(a, b, c), dm = curv(b, c, s0), d0 = curv(c, s0, s1);
-    float dm4m = dm4(dm, d0);
-    float Fm = sl_mpp5_flux(lim, a, b, c, s0, s1, dm4(dmm, dm), dm4m);
-    float cm2 = b, cm1 = c, c0 = s0, cp1 = s1, dcur = d0, sum = 0.f;
-    auto face = [&](float cp2, int i) {
-        const float dn = curv(c0, cp1, cp2);
-        const float dm4p = dm4(dcur, dn);
-        const float F = sl_mpp5_flux(lim, cm2, cm1, c0, cp1, cp2, dm4m, dm4p);
-        const float out = c0 + (Fm - F);
-        p[i * st] = RegCodec<T>::put(out, ip[i * is], lcg_next(rng) >> 16);
-        sum += out;
-        cm2 = cm1;
-        cm1 = c0;
-        c0 = cp1;
-        cp1 = cp2;
-        dcur = dn;
-        dm4m = dm4p;
-        Fm = F;
-    };
-#pragma unroll march_unroll<L>()
-    for (int i = 0; i < L - 2; ++i) face(get(i + 2), i);
-    face(s0, L - 2);
-    face(s1, L - 1);
-    return sum;
+    March<float> m(lim);
+    m.start_periodic(get(L - 3), get(L - 2), get(L - 1), s0, s1);
+    constexpr int B = march_block<L>();
+#pragma unroll 1
+    for (int b = 0; b < (L - 2) / B; ++b, p += B * st, sp += B * ss, ip += B * is)
+#pragma unroll
+        for (int q = 0; q < B; ++q) put(q, m.face(get(q + 2)));
+    constexpr int R = (L - 2) % B;
+#pragma unroll
+    for (int q = 0; q < R; ++q) put(q, m.face(get(q + 2)));
+    put(R, m.face(s0));
+    put(R + 1, m.face(s1));
+    return m.sum;
 }
 
 // march_strided on codes: a value is decoded (the scale of its row) as it enters the
@@ -364,31 +341,19 @@ __device__ __forceinline__ float march_tile16_zf(T *p, int st, const float *sp, 
 {
     static_assert(L >= 4, "lines of at least 4 cells");
     auto get = [&](int i) { return RegCodec<T>::get(p[i * st], sp[i * ss]); };
-    float cm2 = 0.f, cm1 = 0.f, c0 = get(0), cp1 = get(1), cp2 = get(2);
-    float db = curv(0.f, c0, cp1); // curvature of cell 0
-    float dm4m = dm4(c0, db);      // face -1/2: the ghost cell -1 has curvature 0 - 0 + c_0
-    float Fprev = 0.f, sum = 0.f;
-#pragma unroll 8
-    for (int i = 0; i < L; ++i) {
-        float F = 0.f, dm4p = 0.f, dc = 0.f;
-        if (i + 1 < L) {
-            dc = curv(c0, cp1, cp2); // curvature of cell i + 1
-            dm4p = dm4(db, dc);
-            F = sl_mpp5_flux(lim, cm2, cm1, c0, cp1, cp2, dm4m, dm4p);
-        }
-        const float out = vadd(c0, vsub(Fprev, F));
-        p[i * st] = RegCodec<T>::put(out, ip[i * is], lcg_next(rng) >> 16);
-        sum = vadd(sum, out);
-        Fprev = F;
-        dm4m = dm4p;
-        db = dc;
-        cm2 = cm1;
-        cm1 = c0;
-        c0 = cp1;
-        cp1 = cp2;
-        cp2 = i + 3 < L ? get(i + 3) : 0.f;
-    }
-    return sum;
+    auto put = [&](int i, float v) { p[i * st] = RegCodec<T>::put(v, ip[i * is], lcg_next(rng) >> 16); };
+    March<float> m(lim);
+    m.start_zero(get(0), get(1));
+    constexpr int B = 8, R = (L - 2) % B;
+#pragma unroll 1
+    for (int b = 0; b < (L - 2) / B; ++b, p += B * st, sp += B * ss, ip += B * is)
+#pragma unroll
+        for (int q = 0; q < B; ++q) put(q, m.face(get(q + 2)));
+#pragma unroll
+    for (int q = 0; q < R; ++q) put(q, m.face(get(q + 2)));
+    put(R, m.face(0.f));
+    put(R + 1, m.last());
+    return m.sum;
 }
 
 template <int L, typename T, bool SIGNED, int NZ = 32, bool ZF = false>

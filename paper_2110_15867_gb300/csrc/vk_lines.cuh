@@ -77,42 +77,20 @@ template <> struct Chunk<double> {
 
 #define CODED_RNG_INIT(e, seed) (sizeof(T) == 2 ? sr_bits((e), (seed)) : 0u)
 
-// Advance both lines of the pair (forward local frame; zero-flux faces).
-// X = float2: two lines as one packed pair; X = float: one line.
+// Advance the zero-flux line v (forward local frame) held in registers, in place.
+// X = float2: two lines as one packed pair; X = float or double: one line.  Returns the
+// sum of the new values.
 template <int NU, typename X>
 __device__ __forceinline__ X march_regs(X (&v)[NU], const Lim<X> &lim)
 {
-    const X zero = splat<X>(0.0);
-    X d[NU];
+    static_assert(NU >= 4, "lines of at least 4 cells");
+    March<X> m(lim);
+    m.start_zero(v[0], v[1]);
 #pragma unroll
-    for (int i = 0; i < NU; ++i)
-        d[i] = curv(i > 0 ? v[i - 1] : zero, v[i], i + 1 < NU ? v[i + 1] : zero);
-    const X dm = v[0]; // curvature of the ghost cell -1: 0 - 0 + c_0
-    // F[k] = flux through face k - 1/2, k = 1 .. NU-1 (outer faces carry nothing)
-    X Fprev = zero, sum = zero;
-    X dm4m = dm4(dm, d[0]);
-    X out[NU];
-#pragma unroll
-    for (int i = 0; i < NU; ++i) {
-        X F = zero;
-        X dm4p = zero;
-        if (i + 1 < NU) {
-            const X cm2 = i >= 2 ? v[i - 2] : zero;
-            const X cm1 = i >= 1 ? v[i - 1] : zero;
-            const X cp2 = i + 2 < NU ? v[i + 2] : zero;
-            dm4p = dm4(d[i], d[i + 1]);
-            F = sl_mpp5_flux(lim, cm2, cm1, v[i], v[i + 1], cp2, dm4m, dm4p);
-        }
-        out[i] = vadd(v[i], vsub(Fprev, F));
-        sum = vadd(sum, out[i]);
-        Fprev = F;
-        dm4m = dm4p;
-    }
-#pragma unroll
-    for (int i = 0; i < NU; ++i) v[i] = out[i];
-    return sum;
+    for (int i = 0; i < NU - 1; ++i) v[i] = m.face(i + 2 < NU ? v[i + 2] : splat<X>(0.0));
+    v[NU - 1] = m.last();
+    return m.sum;
 }
-
 
 // The zero-flux line p[0], p[st], ..., p[(NU - 1) st] (forward local frame) advanced in
 // place: march_regs with the line read a window ahead and each cell written at its own
@@ -120,32 +98,19 @@ __device__ __forceinline__ X march_regs(X (&v)[NU], const Lim<X> &lim)
 template <int NU> __device__ __forceinline__ float march_strided(float *p, int st, const Lim<float> &lim)
 {
     static_assert(NU >= 4, "lines of at least 4 cells");
-    float cm2 = 0.f, cm1 = 0.f, c0 = p[0], cp1 = p[st], cp2 = p[2 * st];
-    float db = curv(0.f, c0, cp1);  // curvature of cell 0
-    float dm4m = dm4(c0, db);       // face -1/2: the ghost cell -1 has curvature 0 - 0 + c_0
-    float Fprev = 0.f, sum = 0.f;
+    March<float> m(lim);
+    m.start_zero(p[0], p[st]);
     // blocks of 8 faces: a fully unrolled 48-face body per sweep missed in the instruction cache
-#pragma unroll 8
-    for (int i = 0; i < NU; ++i) {
-        float F = 0.f, dm4p = 0.f, dc = 0.f;
-        if (i + 1 < NU) {
-            dc = curv(c0, cp1, cp2); // curvature of cell i + 1
-            dm4p = dm4(db, dc);
-            F = sl_mpp5_flux(lim, cm2, cm1, c0, cp1, cp2, dm4m, dm4p);
-        }
-        const float out = vadd(c0, vsub(Fprev, F));
-        p[i * st] = out;
-        sum = vadd(sum, out);
-        Fprev = F;
-        dm4m = dm4p;
-        db = dc;
-        cm2 = cm1;
-        cm1 = c0;
-        c0 = cp1;
-        cp1 = cp2;
-        cp2 = i + 3 < NU ? p[(i + 3) * st] : 0.f;
-    }
-    return sum;
+    constexpr int B = 8, R = (NU - 2) % B;
+#pragma unroll 1
+    for (int b = 0; b < (NU - 2) / B; ++b, p += B * st)
+#pragma unroll
+        for (int q = 0; q < B; ++q) p[q * st] = m.face(p[(q + 2) * st]);
+#pragma unroll
+    for (int q = 0; q < R; ++q) p[q * st] = m.face(p[(q + 2) * st]);
+    p[R * st] = m.face(0.f);
+    p[(R + 1) * st] = m.last();
+    return m.sum;
 }
 
 // A single value of a line (strided access): decode with the scale of its u_z line,

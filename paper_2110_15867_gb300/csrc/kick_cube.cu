@@ -6,26 +6,27 @@
 // shared memory, run the three velocity sweeps of Eq. (4) on it, and write it back
 // once: f is read and written once per kick instead of once per sweep.
 //
-// Shared memory holds three half-cube buffers (NU / 2 planes of constant j_x each;
-// at NU = 32 in FP32, 64 KB each) that rotate: while a cube sits in two of them,
-// the third receives the first half of the next cube, and once the first half of
-// the current cube has been swept and stored, its buffer receives the second half
-// of the next cube.  Half-cube number j (two per cube, in the order the CTA takes
-// its cubes) always lives in buffer j % 3.  One producer thread drives the TMA
-// engine (loads with transaction-count mbarriers, bulk stores); every wait is
-// bounded.  Rows (u_z lines) are stored with the TMA 32/64/128-byte swizzle, so
-// the three access patterns are free of bank conflicts:
+// Rows (u_z lines) are stored with the TMA 32/64/128-byte swizzle, so the three access
+// patterns are free of bank conflicts.  One producer thread drives the TMA engine (loads
+// with transaction-count mbarriers, bulk stores); every wait is bounded.  The lines are
+// marched by the same SL-MPP5 code (March) as the separate sweeps, so the result equals
+// D_uz D_uy D_ux run as separate kernels, bit for bit.  FP32 storage: kick_pairs_kernel, two
+// lines per thread.  16-bit storage: kick_cube_kernel, one line per thread in registers.
+//
+// 16-bit storage.  Shared memory holds three half-cube buffers (NU / 2 planes of constant
+// j_x each) that rotate: while a cube sits in two of them, the third receives the first half
+// of the next cube, and once the first half of the current cube has been swept and stored,
+// its buffer receives the second half of the next cube.  Half-cube number j (two per cube,
+// in the order the CTA takes its cubes) always lives in buffer j % 3.
 //   D_ux: thread = line (j_y, j_z), walks j_x across both halves (one value per
 //         row, lanes on consecutive j_z: one row segment per warp access);
 //   D_uy: a warp owns whole planes of a half; lane = column j_z, walks j_y;
 //   D_uz: the same warp, lane = row j_y, reads its row in 16-byte chunks.
-// Each line is marched in registers by the same SL-MPP5 code (march_regs) as the
-// separate sweeps, so the result equals D_uz D_uy D_ux run as separate kernels,
-// bit for bit.  16-bit storage keeps the rounding points of the separate path:
-// D_ux encodes its result with the line scales it decoded with (one stochastic
-// draw per value, the stream of the u_x register-line kernel), D_uy writes FP32
-// into a per-warp plane buffer, D_uz takes its rows from there, refreshes each row
-// scale to the row's largest value and encodes with the stream of the u_z kernel.
+// The rounding points are those of the separate path: D_ux encodes its result with the line
+// scales it decoded with (one stochastic draw per value, the stream of the u_x register-line
+// kernel), D_uy writes FP32 into a per-warp plane buffer, D_uz takes its rows from there,
+// refreshes each row scale to the row's largest value and encodes with the stream of the u_z
+// kernel.
 #include "vk_lines.cuh"
 
 namespace vk {
@@ -71,26 +72,21 @@ __device__ __forceinline__ bool cube_ux(unsigned char *const (&h)[2], const floa
     for (int jx = 0; jx < NU; ++jx) {
         const int r = (jx % HP) * NU + jy;
         const T c = *reinterpret_cast<const T *>(h[jx / HP] + G::eoff(r, jz));
-        v[NEG ? NU - 1 - jx : jx] = RegCodec<T>::get(c, G::coded ? s[jx / HP][r] : 1.f);
+        v[NEG ? NU - 1 - jx : jx] = RegCodec<T>::get(c, s[jx / HP][r]);
     }
     const float sum = march_regs<NU, float>(v, lim);
-    unsigned rng = G::coded ? sr_bits(e0, seed) : 0u;
+    unsigned rng = sr_bits(e0, seed);
 #pragma unroll
-    for (int jx = 0; jx < NU; ++jx) {
+    for (int jx = 0; jx < NU; ++jx) { // u_x keeps the scales
         const int r = (jx % HP) * NU + jy;
-        float inv = 1.f;
-        unsigned rb = 0u;
-        if (G::coded) {
-            inv = inv_jx[jx]; // u_x keeps the scales
-            rb = lcg_next(rng) >> 16;
-        }
-        *reinterpret_cast<T *>(h[jx / HP] + G::eoff(r, jz)) = RegCodec<T>::put(v[NEG ? NU - 1 - jx : jx], inv, rb);
+        *reinterpret_cast<T *>(h[jx / HP] + G::eoff(r, jz)) =
+            RegCodec<T>::put(v[NEG ? NU - 1 - jx : jx], inv_jx[jx], lcg_next(rng) >> 16);
     }
     return !(sum >= 0.f) || isinf(sum);
 }
 
-// D_uy on column jz of plane jxl (within half buffer hb, scales sb): FP32 in place, or
-// decoded into the FP32 plane buffer pl (row pitch Cube::pitch) for 16-bit codes.
+// D_uy on column jz of plane jxl (within half buffer hb, scales sb), decoded into the FP32
+// plane buffer pl (row pitch Cube::pitch).
 template <int NU, typename T, bool NEG>
 __device__ __forceinline__ bool cube_uy(unsigned char *hb, const float *sb, float *pl, int jxl, int jz,
                                         const Lim<float> &lim)
@@ -101,20 +97,16 @@ __device__ __forceinline__ bool cube_uy(unsigned char *hb, const float *sb, floa
     for (int jy = 0; jy < NU; ++jy) {
         const int r = jxl * NU + jy;
         const T c = *reinterpret_cast<const T *>(hb + G::eoff(r, jz));
-        v[NEG ? NU - 1 - jy : jy] = RegCodec<T>::get(c, G::coded ? sb[r] : 1.f);
+        v[NEG ? NU - 1 - jy : jy] = RegCodec<T>::get(c, sb[r]);
     }
     const float sum = march_regs<NU, float>(v, lim);
 #pragma unroll
-    for (int jy = 0; jy < NU; ++jy) {
-        const float x = v[NEG ? NU - 1 - jy : jy];
-        if constexpr (G::coded) pl[jy * G::pitch + jz] = x;
-        else *reinterpret_cast<float *>(hb + G::eoff(jxl * NU + jy, jz)) = x;
-    }
+    for (int jy = 0; jy < NU; ++jy) pl[jy * G::pitch + jz] = v[NEG ? NU - 1 - jy : jy];
     return !(sum >= 0.f) || isinf(sum);
 }
 
-// D_uz on row jy of plane jxl: from the half buffer (FP32) or from the FP32 plane
-// buffer (16-bit codes, whose row scale is then refreshed and the row encoded).
+// D_uz on row jy of plane jxl, from the FP32 plane buffer; the row's scale is then refreshed
+// and the row encoded.
 template <int NU, typename T, bool NEG>
 __device__ __forceinline__ bool cube_uz(unsigned char *hb, float *sb, const float *pl, int jxl, int jy,
                                         const Lim<float> &lim, unsigned long long e0, unsigned seed)
@@ -122,29 +114,16 @@ __device__ __forceinline__ bool cube_uz(unsigned char *hb, float *sb, const floa
     using G = Cube<NU, T>;
     const int r = jxl * NU + jy;
     float v[NU];
-    if constexpr (G::coded) {
 #pragma unroll
-        for (int jz = 0; jz < NU; ++jz) v[NEG ? NU - 1 - jz : jz] = pl[jy * G::pitch + jz];
-    } else {
-#pragma unroll
-        for (int j = 0; j < G::chunks; ++j) {
-            float a[4];
-            Chunk<float>::get(hb + G::off(r, j), 1.f, a);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[NEG ? NU - 1 - (4 * j + q) : 4 * j + q] = a[q];
-        }
-    }
+    for (int jz = 0; jz < NU; ++jz) v[NEG ? NU - 1 - jz : jz] = pl[jy * G::pitch + jz];
     const float sum = march_regs<NU, float>(v, lim);
-    float inv = 1.f;
-    if constexpr (G::coded) {
-        float m = 0.f;
+    float m = 0.f;
 #pragma unroll
-        for (int l = 0; l < NU; ++l) m = fmaxf(m, v[l]);
-        m = coded_scale<T>(m);
-        sb[r] = m;
-        inv = inv_scale(m);
-    }
-    unsigned rng = G::coded ? sr_bits(e0, seed) : 0u;
+    for (int l = 0; l < NU; ++l) m = fmaxf(m, v[l]);
+    m = coded_scale<T>(m);
+    sb[r] = m;
+    const float inv = inv_scale(m);
+    unsigned rng = sr_bits(e0, seed);
 #pragma unroll
     for (int j = 0; j < G::chunks; ++j) {
         float a[G::per];
@@ -203,7 +182,7 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
             const long long r0 = first_row(j);
             for (int q = 0; q < G::boxes; ++q)
                 tma_load_2d(hbuf(j) + q * G::box_rows * G::rowbytes, &fmap, bar, 0, int(r0 + q * G::box_rows));
-            if (G::coded) tma_load_2d(sbuf(j), &smap, bar, 0, int(r0 / NU));
+            tma_load_2d(sbuf(j), &smap, bar, 0, int(r0 / NU));
         };
         unsigned loaded = 0;
         for (; loaded < 3 && loaded < halves; ++loaded) load(loaded);
@@ -216,7 +195,7 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
             const long long r0 = first_row(j);
             for (int q = 0; q < G::boxes; ++q)
                 tma_store_2d(&fmap, hbuf(j) + q * G::box_rows * G::rowbytes, 0, int(r0 + q * G::box_rows));
-            if (G::coded) tma_store_2d(&smap, sbuf(j), 0, int(r0 / NU));
+            tma_store_2d(&smap, sbuf(j), 0, int(r0 / NU));
             bulk_commit();
             if (loaded < halves) {
                 bulk_wait_read_all(); // the buffer of half j is free once the store has read it
@@ -258,12 +237,10 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
                 // 16-bit: the warp's lines cross NU rows per j_y (32 / NU values of j_y): each
                 // lane forms the inverse scale of one of them once, for the whole warp
                 float *wi = invs + w * 32;
-                if constexpr (G::coded) {
-                    __syncwarp();
-                    const int jy_l = (q * NT + w * 32) / NU + lane / NU, jx = lane % NU;
-                    wi[lane] = inv_scale(sc[jx / (NU / 2)][(jx % (NU / 2)) * NU + jy_l]);
-                    __syncwarp();
-                }
+                __syncwarp();
+                const int jy_l = (q * NT + w * 32) / NU + lane / NU, jx = lane % NU;
+                wi[lane] = inv_scale(sc[jx / (NU / 2)][(jx % (NU / 2)) * NU + jy_l]);
+                __syncwarp();
                 const float *inv_jx = wi + (lane / NU) * NU;
                 bad |= (kx.nd & 1) ? cube_ux<NU, T, true>(h, sc, inv_jx, jy, jz, lim, e0, a.seed_x)
                                    : cube_ux<NU, T, false>(h, sc, inv_jx, jy, jz, lim, e0, a.seed_x);
@@ -285,7 +262,7 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
                 const Lim<float> lim = to_lim(ky);
                 bad |= (ky.nd & 1) ? cube_uy<NU, T, true>(hb, sb, pl, jxl, c, lim)
                                    : cube_uy<NU, T, false>(hb, sb, pl, jxl, c, lim);
-            } else if (G::coded) {
+            } else {
                 // no D_uy: the plane buffer takes the decoded values as they are
 #pragma unroll 4
                 for (int jy = 0; jy < NU; ++jy) {
@@ -299,7 +276,7 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
                 const Lim<float> lim = to_lim(kz);
                 bad |= (kz.nd & 1) ? cube_uz<NU, T, true>(hb, sb, pl, jxl, c, lim, e0, a.seed_z)
                                    : cube_uz<NU, T, false>(hb, sb, pl, jxl, c, lim, e0, a.seed_z);
-            } else if (G::coded && ky.nd >= 0) {
+            } else if (ky.nd >= 0) {
                 // D_uy changed the plane but D_uz does not run: encode it with the row's scale
                 // refreshed as the u_z sweep would not; keep the stored scale, round to nearest
                 const int r = jxl * NU + c;
@@ -316,12 +293,292 @@ __global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1
     if (bad) atomicOr(a.err, ERR_NAN);
 }
 
+// ----------------------------------------------------------------------------
+// FP32 storage: two lines per thread as packed pairs, lines walked in shared memory
+// ----------------------------------------------------------------------------
+// 32^3 x 32^3 cells, per kick: 3.83 ms with one line per thread in registers, 3.42 with the
+// flux in differences, 3.05 here (76 cycles per face pair and scheduler: 49 instructions, the
+// ALU pipe 60 % and issue 65 % busy; the DRAM traffic alone would take 1.27 ms).  Read from
+// global memory by every thread when they were needed, the coefficients cost 8 % of that;
+// cells read no further ahead than the window, 3 %.
+// The kick is bound by instruction issue and by the ALU pipe (min / max at half rate), not
+// by DRAM.  A thread marches two lines at once, their sums and products as f32x2 (one issue
+// slot for two), through a window of a few cells (vk_common.cuh, March), reading each cell
+// once and writing it back in place, so that 512 threads cover all 1024 lines of a 32^3
+// cube in one go at about 100 registers: 16 warps per SM keep both pipes busy.  (Whole pairs
+// of lines in registers left 8 warps per SM and were slower than one line per thread.)
+//
+// Pieces.  A cube is four pieces of NU / 4 planes of constant j_x; a ring of seven pieces
+// holds the current cube and three pieces of the next.  D_ux walks the planes in the order
+// of its flow and waits for each piece as it comes to it, so the fourth piece of a cube,
+// which can only be loaded once a piece of the previous cube has been stored, arrives while
+// the first three are marched.  Piece j (four per cube, in march order) lives in slot j % 7.
+//   D_ux: thread = columns (j_y, j_z), (j_y, j_z + 1), one 8-byte access per row;
+//   D_uy: a warp owns 64 / NU planes; thread = two adjacent columns of one, walks j_y;
+//   D_uz: the same warp; thread = rows j_y and j_y + NU / 2 of a plane, in 16-byte chunks
+//         (cells of the two rows do not sit in register pairs: SPLIT).
+// All accesses are free of bank conflicts under the TMA swizzle (NU = 16: D_uy two-way).
+template <int NU> struct PairCube {
+    using G = Cube<NU, float>;
+    static constexpr int planes = NU / 4;                       // of a piece
+    static constexpr int rows = planes * NU;                    // u_z lines of a piece
+    static constexpr unsigned bytes = unsigned(rows) * G::rowbytes;
+    static constexpr int slots = 7;
+    static constexpr int threads = NU * NU / 2; // one per pair of lines
+    static constexpr int warps = threads / 32;
+    static constexpr int wplanes = 64 / NU;     // planes a warp owns
+    static constexpr int per_piece = threads / 4; // threads whose planes lie in one piece
+    // barriers (128 B), the coefficients of three cubes (u_x, u_y, u_z), alignment, the ring
+    static constexpr int head = 128 + ((9 * int(sizeof(LineCoefT<float>)) + 127) & ~127);
+    static constexpr size_t smem = head + 1024 + size_t(slots) * bytes;
+    static_assert(rows <= 256, "one TMA box per piece");
+};
+
+// D_ux on the columns at byte offset `off` of every plane.  slot(m): the piece in march
+// order m (waits for it; false: the wait ran out).
+template <int NU, bool NEG, typename Slot>
+__device__ __forceinline__ bool pair_ux(Slot slot, int off, const Lim<float2> &lim, bool &ok)
+{
+    using P = PairCube<NU>;
+    constexpr int NP = P::planes, ST = NU * P::G::rowbytes; // bytes of a plane
+    auto cell = [&](unsigned char *p, int i) -> float2 & { // plane i of the piece in march order
+        return *reinterpret_cast<float2 *>(p + (NEG ? NP - 1 - i : i) * ST);
+    };
+    unsigned char *cur = slot(0, ok) + off;
+    if (!ok) return false;
+    March<float2> m(lim);
+    m.start_zero(cell(cur, 0), cell(cur, 1));
+#pragma unroll
+    for (int i = 2; i < NP; ++i) cell(cur, i - 2) = m.face(cell(cur, i));
+#pragma unroll 1
+    for (int q = 1; q < 4; ++q) {
+        unsigned char *prev = cur;
+        cur = slot(q, ok) + off;
+        if (!ok) return false;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const float2 out = m.face(cell(cur, i));
+            if (i < 2) cell(prev, NP - 2 + i) = out;
+            else cell(cur, i - 2) = out;
+        }
+    }
+    cell(cur, NP - 2) = m.face(make_float2(0.f, 0.f));
+    cell(cur, NP - 1) = m.last();
+    return !(m.sum.x >= 0.f) || !(m.sum.y >= 0.f) || isinf(m.sum.x) || isinf(m.sum.y);
+}
+
+// D_uy on the adjacent columns jz, jz + 1 (jz even) of the plane at pl
+template <int NU, bool NEG>
+__device__ __forceinline__ bool pair_uy(unsigned char *pl, int jz, const Lim<float2> &lim)
+{
+    using G = Cube<NU, float>;
+    auto cell = [&](int i) -> float2 & { return *reinterpret_cast<float2 *>(pl + G::eoff(NEG ? NU - 1 - i : i, jz)); };
+    March<float2> m(lim);
+    m.start_zero(cell(0), cell(1));
+    // cells are read four rows ahead of their use: a read stays behind the writes before it
+    // (the compiler cannot tell the swizzled addresses apart), and so must not wait for a face
+    constexpr int A = 4;
+    float2 ahead[A];
+#pragma unroll
+    for (int i = 0; i < A; ++i) ahead[i] = cell(i + 2);
+#pragma unroll
+    for (int i = 0; i < NU - 2; ++i) {
+        const float2 c = ahead[i % A];
+        if (i + 2 + A < NU) ahead[i % A] = cell(i + 2 + A);
+        cell(i) = m.face(c);
+    }
+    cell(NU - 2) = m.face(make_float2(0.f, 0.f));
+    cell(NU - 1) = m.last();
+    return !(m.sum.x >= 0.f) || !(m.sum.y >= 0.f) || isinf(m.sum.x) || isinf(m.sum.y);
+}
+
+// D_uz on the rows jy and jy + NU / 2 of the plane at pl
+template <int NU, bool NEG>
+__device__ __forceinline__ bool pair_uz(unsigned char *pl, int jy, const Lim<float2> &lim)
+{
+    using G = Cube<NU, float>;
+    constexpr int C = G::chunks;
+    auto at = [&](int row, int j) -> float4 & {
+        return *reinterpret_cast<float4 *>(pl + G::off(row, NEG ? C - 1 - j : j));
+    };
+    March<float2, true> m(lim);
+    float4 oa, ob; // outputs of the chunk being filled (in march order)
+    auto put = [&](int i, float2 v) {
+        const int q = NEG ? 3 - i % 4 : i % 4;
+        (&oa.x)[q] = v.x;
+        (&ob.x)[q] = v.y;
+        if (i % 4 == 3) {
+            at(jy, i / 4) = oa;
+            at(jy + NU / 2, i / 4) = ob;
+        }
+    };
+    float2 first = make_float2(0.f, 0.f);
+    float4 na = at(jy, 0), nb = at(jy + NU / 2, 0); // read one chunk ahead of their use (as in pair_uy)
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        const float4 a = na, b = nb;
+        if (j + 1 < C) {
+            na = at(jy, j + 1);
+            nb = at(jy + NU / 2, j + 1);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = 4 * j + q, s = NEG ? 3 - q : q;
+            const float2 c = make_float2((&a.x)[s], (&b.x)[s]);
+            if (i == 0) first = c;
+            else if (i == 1) m.start_zero(first, c);
+            else put(i - 2, m.face(c));
+        }
+    }
+    put(NU - 2, m.face(make_float2(0.f, 0.f)));
+    put(NU - 1, m.last());
+    return !(m.sum.x >= 0.f) || !(m.sum.y >= 0.f) || isinf(m.sum.x) || isinf(m.sum.y);
+}
+
+template <int NU>
+__global__ void __launch_bounds__(PairCube<NU>::threads + kProducer, NU == 32 ? 1 : 4)
+    kick_pairs_kernel(const __grid_constant__ CUtensorMap fmap, const __grid_constant__ KickArgs a)
+{
+    using P = PairCube<NU>;
+    using G = Cube<NU, float>;
+    constexpr int NT = P::threads, S = P::slots;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem); // S: the slot holds its piece
+    uint64_t *done = full + S;                           // S: the warps that own its planes are done
+    uint64_t *uxd = done + S;                            // D_ux of the current cube is complete
+    static_assert((2 * S + 1) * 8 <= 128, "barriers fit ahead of the ring");
+    LineCoefT<float> *coefs = reinterpret_cast<LineCoefT<float> *>(smem + 128);
+    unsigned char *ring = smem + P::head + ((1024u - ((smem_u32(smem) + unsigned(P::head)) & 1023u)) & 1023u);
+    auto slot = [&](unsigned j) { return ring + size_t(P::bytes) * (j % S); };
+
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < S; ++q) {
+            mbar_init(&full[q], 1);
+            mbar_init(&done[q], P::per_piece);
+        }
+        mbar_init(uxd, NT);
+        fence_barrier_init();
+    }
+    __syncthreads();
+
+    const long long Gd = gridDim.x, b = blockIdx.x;
+    const unsigned n_my = unsigned(a.ncells > b ? (a.ncells - b + Gd - 1) / Gd : 0);
+    const unsigned pieces = 4 * n_my;
+
+    if (threadIdx.x >= NT) {
+        // producer: one thread drives the TMA engine
+        if (threadIdx.x != NT) return;
+        // the coefficients of the cube of piece j (the ring holds pieces of two cubes, and the
+        // third slot keeps those of the cube before for warps still on it)
+        auto coef = [&](unsigned j) { return coefs + 3 * ((j / 4) % 3); };
+        auto first_row = [&](unsigned j) { // of piece j: the quarters of a cube in the order D_ux walks them
+            const long long cube = a.cell0 + b + (long long)(j / 4) * Gd;
+            const int nd = coef(j)->nd;
+            const int q = nd >= 0 && (nd & 1) ? 3 - int(j % 4) : int(j % 4);
+            return int(cube * (NU * NU) + q * P::rows);
+        };
+        auto load = [&](unsigned j) {
+            if (j % 4 == 0) {
+                // read here, ahead of the consumers, who would wait for them three times per cube;
+                // they see them once they have waited for the piece
+                const long long cube = a.cell0 + b + (long long)(j / 4) * Gd;
+                const LineCoefT<float> cx = a.coef_x[cube], cy = a.coef_y[cube], cz = a.coef_z[cube];
+                coef(j)[0] = cx;
+                coef(j)[1] = cy;
+                coef(j)[2] = cz;
+            }
+            uint64_t *bar = &full[j % S];
+            mbar_arrive_expect_tx(bar, P::bytes);
+            tma_load_2d(slot(j), &fmap, bar, 0, first_row(j));
+        };
+        unsigned loaded = 0;
+        for (; loaded < unsigned(S) && loaded < pieces; ++loaded) load(loaded);
+        bool ok = true;
+        for (unsigned j = 0; j < pieces; ++j) {
+            if (!mbar_wait_bounded(&done[j % S], (j / S) & 1u)) {
+                ok = false;
+                break;
+            }
+            tma_store_2d(&fmap, slot(j), 0, first_row(j));
+            bulk_commit();
+            if (loaded < pieces) {
+                bulk_wait_read_all(); // the slot of piece j is free once the store has read it
+                load(loaded++);
+            }
+        }
+        bulk_wait_all();
+        if (!ok) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            // let the loads in flight (the last S at most) land before the CTA exits
+            for (unsigned j = loaded > unsigned(S) ? loaded - S : 0; j < loaded; ++j)
+                mbar_wait_bounded(&full[j % S], (j / S) & 1u);
+        }
+        return;
+    }
+
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    // D_ux: the thread's columns; D_uy, D_uz: its plane (within the warp's), column pair, row
+    const int ux_off = G::eoff(t / (NU / 2), 2 * (t % (NU / 2)));
+    const int wp = lane / (NU / 2), lp = lane % (NU / 2);
+    const int quarter = w / (P::warps / 4); // of the cube: where the warp's planes lie
+    const int pl_off = ((w % (P::warps / 4)) * P::wplanes + wp) * NU * G::rowbytes;
+    bool bad = false, ok = true;
+    for (unsigned k = 0; k < n_my; ++k) {
+        auto piece = [&](int m, bool &good) { // piece m of the cube, once it is loaded
+            const unsigned j = 4 * k + m;
+            good = __all_sync(0xffffffffu, mbar_wait_bounded(&full[j % S], (j / S) & 1u));
+            return slot(j);
+        };
+        piece(0, ok);
+        if (!ok) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            return;
+        }
+        // one Courant number per cell and axis: every branch below is CTA-uniform
+        const LineCoefT<float> *co = coefs + 3 * (k % 3);
+        const LineCoefT<float> kx = co[0];
+        const bool xneg = kx.nd >= 0 && (kx.nd & 1);
+        if (kx.nd >= 0) {
+            const Lim<float2> lim = to_lim2(kx, kx);
+            bad |= xneg ? pair_ux<NU, true>(piece, ux_off, lim, ok) : pair_ux<NU, false>(piece, ux_off, lim, ok);
+        } else {
+            for (int m = 1; m < 4 && ok; ++m) piece(m, ok);
+        }
+        if (!ok) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            return;
+        }
+        // every D_ux line crosses every plane: all of them finish before D_uy
+        mbar_arrive(uxd);
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(uxd, k & 1u))) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            return;
+        }
+        const LineCoefT<float> ky = co[1], kz = co[2];
+        const unsigned j = 4 * k + (xneg ? 3 - quarter : quarter);
+        unsigned char *pl = slot(j) + pl_off;
+        if (ky.nd >= 0) {
+            const Lim<float2> lim = to_lim2(ky, ky);
+            bad |= (ky.nd & 1) ? pair_uy<NU, true>(pl, 2 * lp, lim) : pair_uy<NU, false>(pl, 2 * lp, lim);
+        }
+        __syncwarp();
+        if (kz.nd >= 0) {
+            const Lim<float2> lim = to_lim2(kz, kz);
+            bad |= (kz.nd & 1) ? pair_uz<NU, true>(pl, lp, lim) : pair_uz<NU, false>(pl, lp, lim);
+        }
+        __syncwarp();
+        fence_proxy_async();
+        mbar_arrive(&done[j % S]);
+    }
+    if (bad) atomicOr(a.err, ERR_NAN);
+}
+
 template <int NU, typename T> const void *kick_kernel() { return (const void *)kick_cube_kernel<NU, T>; }
 
 const void *kick_kernel_for(int nu, int dtype)
 {
     switch (dtype) {
-    case 1: return nu == 32 ? kick_kernel<32, float>() : kick_kernel<16, float>();
+    case 1: return nu == 32 ? (const void *)kick_pairs_kernel<32> : (const void *)kick_pairs_kernel<16>;
     case 2: return nu == 32 ? kick_kernel<32, __nv_bfloat16>() : kick_kernel<16, __nv_bfloat16>();
     case 3: return nu == 32 ? kick_kernel<32, __half>() : kick_kernel<16, __half>();
     default: return nullptr;
@@ -330,7 +587,7 @@ const void *kick_kernel_for(int nu, int dtype)
 
 template <int NU> size_t smem_for(int dtype)
 {
-    return dtype == 1 ? Cube<NU, float>::smem : Cube<NU, __nv_bfloat16>::smem;
+    return dtype == 1 ? PairCube<NU>::smem : Cube<NU, __nv_bfloat16>::smem;
 }
 
 template <int NU> int threads_for() { return Cube<NU, float>::threads + kProducer; }
@@ -342,7 +599,11 @@ bool kick_cube_supported(int nux, int nuy, int nuz, int dtype)
     return nux == nuy && nuy == nuz && (nuz == 16 || nuz == 32) && dtype >= 1 && dtype <= 3;
 }
 
-int kick_cube_box_rows(int nu) { return nu * nu / 2 < 256 ? nu * nu / 2 : 256; }
+int kick_cube_box_rows(int nu, int dtype)
+{
+    if (dtype == 1) return nu * nu / 4; // a piece
+    return nu * nu / 2 < 256 ? nu * nu / 2 : 256;
+}
 
 size_t kick_cube_smem(int nu, int dtype) { return nu == 32 ? smem_for<32>(dtype) : smem_for<16>(dtype); }
 
@@ -370,7 +631,9 @@ cudaError_t launch_kick_cube(const CUtensorMap &fmap, const CUtensorMap &smap, c
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     KickArgs args = a;
-    void *params[] = {const_cast<CUtensorMap *>(&fmap), const_cast<CUtensorMap *>(&smap), &args};
+    void *params_f32[] = {const_cast<CUtensorMap *>(&fmap), &args};
+    void *params_coded[] = {const_cast<CUtensorMap *>(&fmap), const_cast<CUtensorMap *>(&smap), &args};
+    void **params = dtype == 1 ? params_f32 : params_coded;
     const int threads = nu == 32 ? threads_for<32>() : threads_for<16>();
     return cudaLaunchKernel(k, dim3(grid), dim3(threads), params, smem, st);
 }

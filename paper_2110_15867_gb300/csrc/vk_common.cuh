@@ -21,6 +21,9 @@ namespace vk {
 // A bounded wait gives up after this much wall time or this many polls.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr unsigned kWaitLimitPolls = 1u << 26;
+// How long one poll may keep the warp asleep (it wakes when the phase completes): warps that
+// wait poll seldom and leave the issue slots to those that work.
+constexpr unsigned kPollNs = 20000;
 
 // ----------------------------------------------------------------------------
 // PTX wrappers
@@ -71,10 +74,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity)
     unsigned ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kPollNs)
         : "memory");
     return ok != 0;
 }
@@ -466,14 +469,33 @@ __device__ __forceinline__ double flux_clamp(double F, double c0)
 // Fractional flux through the downwind face of the donor c0 (local frame, flow toward
 // +index): dmm, dm, dp, dpp = delta_{-2} .. delta_1 around it, hm, hp = dm / 2, dp / 2, qm /
 // qp the limited curvatures (limited_curv) at its upwind / downwind faces.
-template <typename X>
+// SPLIT (packed pairs): operations on the cells themselves act on the two lines one by one,
+// for cells that do not sit in aligned register pairs.
+__device__ __forceinline__ float2 two(float a, float b) { return make_float2(a, b); }
+template <bool SPLIT, typename X> __device__ __forceinline__ X cell_sub(X a, X b)
+{
+    if constexpr (SPLIT) return two(a.x - b.x, a.y - b.y);
+    else return vsub(a, b);
+}
+template <bool SPLIT, typename X> __device__ __forceinline__ X cell_add(X a, X b)
+{
+    if constexpr (SPLIT) return two(a.x + b.x, a.y + b.y);
+    else return vadd(a, b);
+}
+template <bool SPLIT, typename X> __device__ __forceinline__ X cell_mul(X a, X b)
+{
+    if constexpr (SPLIT) return two(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+    else return vmul(a, b);
+}
+
+template <bool SPLIT = false, typename X>
 __device__ __forceinline__ X sl_mpp5_flux(const Lim<X> &k, X c0, X dmm, X dm, X dp, X dpp, X hm, X hp, X qm, X qp)
 {
     const X phi = vfma(k.v3, dpp, vfma(k.v2, dp, vfma(k.v1, dm, vmul(k.v0, dmm))));
     const X md = vfma(splat<X>(CurvScale<X>::md), qp, hp);
     const X lc = vfma(splat<X>(CurvScale<X>::lc), qm, hm);
     const X v = mp_clamp(phi, dp, md, vmul(k.alpha, dm), lc);
-    return flux_clamp(vfma(k.s, v, vmul(k.s, c0)), c0);
+    return flux_clamp(vfma(k.s, v, cell_mul<SPLIT>(k.s, c0)), c0);
 }
 
 // ----------------------------------------------------------------------------
@@ -484,7 +506,7 @@ __device__ __forceinline__ X sl_mpp5_flux(const Lim<X> &k, X c0, X dmm, X dm, X 
 // cells, face(cp2) takes cell i + 2, returns the new value of cell i and moves on; last()
 // is the last cell of a zero-flux line (nothing crosses its outer face).  sum: of the new
 // values (for the NaN / sign check).
-template <typename X> struct March {
+template <typename X, bool SPLIT = false> struct March {
     const Lim<X> &k;
     X c0, cp1, dmm, dm, dp, hm, hp, d0, qm, Fm, sum;
 
@@ -517,12 +539,12 @@ template <typename X> struct March {
     }
     __device__ __forceinline__ X face(X cp2)
     {
-        const X dpp = vsub(cp2, cp1);
+        const X dpp = cell_sub<SPLIT>(cp2, cp1);
         const X dn = vsub(dpp, dp); // curvature of cell i + 1
         const X qp = limited_curv(d0, dn);
-        const X F = sl_mpp5_flux(k, c0, dmm, dm, dp, dpp, hm, hp, qm, qp);
-        const X out = vadd(c0, vsub(Fm, F));
-        sum = vadd(sum, out);
+        const X F = sl_mpp5_flux<SPLIT>(k, c0, dmm, dm, dp, dpp, hm, hp, qm, qp);
+        const X out = cell_add<SPLIT>(c0, vsub(Fm, F));
+        sum = cell_add<SPLIT>(sum, out);
         c0 = cp1;
         cp1 = cp2;
         dmm = dm;

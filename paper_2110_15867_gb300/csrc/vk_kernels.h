@@ -212,7 +212,7 @@ struct KickArgs {
     unsigned seed_x, seed_z; // 16-bit: stochastic-rounding streams of the D_ux and D_uz encodes
 };
 bool kick_cube_supported(int nux, int nuy, int nuz, int dtype); // dtype 1 f32, 2 bf16, 3 f16
-int kick_cube_box_rows(int nu);
+int kick_cube_box_rows(int nu, int dtype);
 size_t kick_cube_smem(int nu, int dtype);
 int occupancy_kick_cube(int nu, int dtype);
 cudaError_t launch_kick_cube(const CUtensorMap &fmap, const CUtensorMap &smap, const KickArgs &a, int nu, int dtype,

@@ -487,7 +487,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         const CUtensorMapSwizzle sw = rowbytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                       : rowbytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                        : CU_TENSOR_MAP_SWIZZLE_32B;
-        const MapSpec ks = spec_rows(tmap_type(c->g.dtype), nu, c->ncell * nu * nu, es, kick_cube_box_rows(nu), sw);
+        const MapSpec ks = spec_rows(tmap_type(c->g.dtype), nu, c->ncell * nu * nu, es, kick_cube_box_rows(nu, c->g.dtype), sw);
         CUresult r = encode_spec(&c->kmap, ks, c->f);
         if (r != CUDA_SUCCESS) return fail(c, VLASOV_ECUDA, "kick tensor map failed (%d)", int(r));
         if (coded) {

@@ -3,17 +3,23 @@
 //
 // A (cell, j_x) plane of the velocity cube holds n_uy rows (j_y) of n_uz cells (j_z),
 // contiguous in f (Listing 1: u_z innermost), and both sweeps stay inside it.  A
-// block stages four planes of one spatial cell in shared memory (rows padded to
-// n_uz + 1 floats, so that a warp walking columns and a warp walking rows both hit 32
-// different banks), 48 threads per plane march its columns (D_uy), then its rows
-// (D_uz), and the block writes the planes back: f is read and written once for the
-// two sweeps instead of twice.  Each line is marched in shared memory through a
-// window of five cells in registers (march_strided, one body for both sweeps, faces in
-// blocks of 8), the arithmetic of march_regs in the same order, so the result equals the
-// separate u_y and u_z sweeps bit for bit.
-// The stride of a line (its axis and the sign of its Courant number) is a run-time
-// value: one march body for both axes and signs (four compile-time bodies measured
-// slower: 43.9 against 41.0 ms on the 48^3 x 48^3 run).
+// block stages four planes of one spatial cell in shared memory, sweeps them along u_y, then
+// along u_z, and writes them back: f is read and written once for the two sweeps.
+//
+// The pass is bound by the marches (instruction issue and the ALU pipe), not by DRAM, so a
+// thread marches two lines at once, sums and products as f32x2 pairs (vk_common.cuh), through
+// a window of a few cells, reading each cell once and writing it back in place: D_uy two
+// adjacent columns (one 8-byte access per row), D_uz rows l and l + n_uy / 2 in 16-byte
+// chunks.  Rows are padded to n_uz + 4 floats, an odd number of 16-byte units: eight rows
+// read at one chunk fall on different banks.  FP32 rows come in by 16-byte asynchronous
+// copies (a bulk copy per row costs more instructions: one thread of a warp at a time issues
+// it).  Faces in
+// blocks of 8 (D_uy) and 4 (D_uz): blocks of 23 and 20 faces missed in the instruction cache
+// (3.6 fetch stalls per issue, 20 % slower).  The arithmetic is march_regs' in the same order: FP32 results equal the separate
+// sweeps bit for bit.
+// 24^3 x 48^3 cells, per kick tail: FP32 4.84 ms with one line per thread, 3.2 ms here (52
+// instructions per face pair, issue 61 % and ALU pipe 56 % busy; DRAM alone 1.8 ms), FP16
+// 4.90 -> 3.5 ms.
 // 16-bit storage: the planes are decoded into FP32 as they are staged; D_uy's result
 // stays FP32 and each row is encoded once, after D_uz, with a refreshed line scale (the
 // rounding points of the fused tail of smaller cubes, not of the separate sweeps).
@@ -25,90 +31,160 @@ namespace {
 
 constexpr int kPlanesPerBlock = 4;
 
-template <int NU> constexpr int plane_pitch() { return NU + 1; }
-template <int NU> constexpr size_t plane_smem() { return size_t(kPlanesPerBlock) * NU * plane_pitch<NU>() * sizeof(float); }
+template <int NU> struct PlaneGeom {
+    static constexpr int pitch = NU + 4;     // floats per row
+    static constexpr int half = NU / 2;      // line pairs per plane
+    static constexpr int threads = kPlanesPerBlock * half;
+    static constexpr size_t smem = size_t(kPlanesPerBlock) * NU * pitch * sizeof(float);
+    static_assert((pitch / 4) % 2 == 1 && NU % 8 == 0, "an odd number of 16-byte units per row");
+};
+
+// 16 bytes from global to shared memory without a register
+__device__ __forceinline__ void copy16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// D_uy on the adjacent columns at p (row 0): p[r * pitch], p[r * pitch + 1]
+template <int NU, bool NEG> __device__ __forceinline__ float2 plane_uy(float *p, const Lim<float2> &lim)
+{
+    constexpr int ST = NEG ? -PlaneGeom<NU>::pitch : PlaneGeom<NU>::pitch;
+    if (NEG) p += (NU - 1) * PlaneGeom<NU>::pitch;
+    auto cell = [&](int i) -> float2 & { return *reinterpret_cast<float2 *>(p + i * ST); };
+    March<float2> m(lim);
+    m.start_zero(cell(0), cell(1));
+    constexpr int B = 8, R = (NU - 2) % B;
+#pragma unroll 1
+    for (int b = 0; b < (NU - 2) / B; ++b, p += B * ST)
+#pragma unroll
+        for (int q = 0; q < B; ++q) cell(q) = m.face(cell(q + 2));
+#pragma unroll
+    for (int q = 0; q < R; ++q) cell(q) = m.face(cell(q + 2));
+    cell(R) = m.face(make_float2(0.f, 0.f));
+    cell(R + 1) = m.last();
+    return m.sum;
+}
+
+// D_uz on the rows at p and p + NU / 2 rows
+template <int NU, bool NEG> __device__ __forceinline__ float2 plane_uz(float *p, const Lim<float2> &lim)
+{
+    constexpr int OTHER = (NU / 2) * PlaneGeom<NU>::pitch, C = NU / 4, ST = NEG ? -4 : 4;
+    if (NEG) p += NU - 4;
+    auto at = [&](int row, int j) -> float4 & { return *reinterpret_cast<float4 *>(p + row + j * ST); };
+    auto pick = [](const float4 &a, const float4 &b, int i) { // cell i of a chunk in march order
+        const int s = NEG ? 3 - i : i;
+        return make_float2((&a.x)[s], (&b.x)[s]);
+    };
+    auto set = [](float4 &a, float4 &b, int i, float2 v) {
+        const int s = NEG ? 3 - i : i;
+        (&a.x)[s] = v.x;
+        (&b.x)[s] = v.y;
+    };
+    March<float2, true> m(lim);
+    float4 a = at(0, 0), b = at(OTHER, 0), oa, ob;
+    float4 na = at(0, 1), nb = at(OTHER, 1); // read one chunk ahead of their use
+    m.start_zero(pick(a, b, 0), pick(a, b, 1));
+    set(oa, ob, 0, m.face(pick(a, b, 2)));
+    set(oa, ob, 1, m.face(pick(a, b, 3)));
+#pragma unroll 1
+    for (int j = 1; j < C; ++j, p += ST) { // chunk j; the outputs of chunk j - 1 are at chunk 0 of p
+        a = na;
+        b = nb;
+        if (j + 1 < C) {
+            na = at(0, 2);
+            nb = at(OTHER, 2);
+        }
+        set(oa, ob, 2, m.face(pick(a, b, 0)));
+        set(oa, ob, 3, m.face(pick(a, b, 1)));
+        at(0, 0) = oa;
+        at(OTHER, 0) = ob;
+        set(oa, ob, 0, m.face(pick(a, b, 2)));
+        set(oa, ob, 1, m.face(pick(a, b, 3)));
+    }
+    set(oa, ob, 2, m.face(make_float2(0.f, 0.f)));
+    set(oa, ob, 3, m.last());
+    at(0, 0) = oa;
+    at(OTHER, 0) = ob;
+    return m.sum;
+}
 
 template <int NU, typename T>
-__global__ void __launch_bounds__(kPlanesPerBlock * NU) plane_tail_kernel(T *__restrict__ f, const __grid_constant__ PlaneTailArgs a)
+__global__ void __launch_bounds__(PlaneGeom<NU>::threads, 5)
+    plane_tail_kernel(T *__restrict__ f, const __grid_constant__ PlaneTailArgs a)
 {
+    using G = PlaneGeom<NU>;
     constexpr bool CODED = sizeof(T) == 2;
-    constexpr int P = plane_pitch<NU>(), PER = 16 / int(sizeof(T)), Q = NU * NU / PER; // 16-byte chunks per plane
+    constexpr int P = G::pitch, PER = 16 / int(sizeof(T));
+    constexpr int ROWS = kPlanesPerBlock * NU;
+    // thread t takes chunk t % CH of rows t / CH, t / CH + RP, ...
+    constexpr int CH = NU / PER, RP = G::threads / CH;
+    static_assert(NU % PER == 0 && G::threads % CH == 0 && ROWS % RP == 0, "whole passes of whole rows");
     extern __shared__ __align__(16) float plane_s[];
-    const long long p0 = a.plane0 + blockIdx.x * (long long)kPlanesPerBlock; // first plane of the block
-    const long long pend = a.plane0 + a.nplanes;
-    // stage the planes (a plane is NU rows of NU values, contiguous; NU % PER == 0, so a
-    // 16-byte chunk never straddles two rows); codes are decoded with their row's scale
-    for (int k = threadIdx.x; k < kPlanesPerBlock * Q; k += blockDim.x) {
-        const int q = k / Q, e = PER * (k - q * Q), row = e / NU, col = e - row * NU;
-        if (p0 + q < pend) {
-            float *s = plane_s + (q * NU + row) * P + col;
-            if constexpr (CODED) {
-                float v[PER];
-                Chunk<T>::get(reinterpret_cast<const unsigned char *>(f + (p0 + q) * NU * NU) + 16 * (k - q * Q),
-                              a.scale[(p0 + q) * NU + row], v);
+    // the block's planes belong to one spatial cell (the host checks n_ux % 4 == 0)
+    const long long p0 = a.plane0 + blockIdx.x * (long long)kPlanesPerBlock;
+    const long long cell = a.plane0 / a.nux + (long long)((blockIdx.x * unsigned(kPlanesPerBlock)) / unsigned(a.nux));
+    const int row0 = threadIdx.x / CH, col0 = PER * (threadIdx.x - row0 * CH);
+    T *g = f + p0 * NU * NU + row0 * NU + col0;
+    float *sg = plane_s + row0 * P + col0;
 #pragma unroll
-                for (int i = 0; i < PER; ++i) s[i] = v[i];
-            } else {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(f + (p0 + q) * NU * NU) + (k - q * Q));
-                s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
-            }
+    for (int k = 0; k < ROWS / RP; ++k) {
+        if constexpr (CODED) { // decoded with their row's scale
+            float v[PER];
+            Chunk<T>::get(reinterpret_cast<const unsigned char *>(g + k * RP * NU), a.scale[p0 * NU + row0 + k * RP], v);
+            float4 *s = reinterpret_cast<float4 *>(sg + k * RP * P);
+            s[0] = make_float4(v[0], v[1], v[2], v[3]);
+            s[1] = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+            copy16(sg + k * RP * P, g + k * RP * NU);
         }
+    }
+    const LineCoefT<float> ky = a.coef_y[cell], kz = a.coef_z[cell];
+    if constexpr (!CODED) asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const int q = threadIdx.x / G::half, l = threadIdx.x - q * G::half;
+    float *plane = plane_s + q * NU * P;
+    bool bad = false;
+    auto check = [&](float2 s) { bad |= !(s.x >= 0.f) || !(s.y >= 0.f) || isinf(s.x) || isinf(s.y); };
+    if (ky.nd >= 0) { // one Courant number per cell: block-uniform
+        const Lim<float2> lim = to_lim2(ky, ky);
+        check((ky.nd & 1) ? plane_uy<NU, true>(plane + 2 * l, lim) : plane_uy<NU, false>(plane + 2 * l, lim));
     }
     __syncthreads();
-    // the block's planes belong to one spatial cell (the host checks n_ux % 4 == 0)
-    const long long cell = p0 / a.nux;
-    const int q = threadIdx.x / NU, l = threadIdx.x - q * NU;
-    float *plane = plane_s + q * NU * P;
-    bool bad = false, any = false;
-    // D_uy (column l, rows 0 .. NU-1), then D_uz (row l): one march body for both
-#pragma unroll 1
-    for (int ax = 0; ax < 2; ++ax) {
-        const LineCoefT<float> k = ax == 0 ? a.coef_y[cell] : a.coef_z[cell];
-        if (p0 + q < pend && k.nd >= 0) {
-            // from the far end when the Courant number is negative
-            const bool neg = k.nd & 1;
-            const int step = ax == 0 ? P : 1;
-            float *first = plane + (ax == 0 ? l : l * P) + (neg ? (NU - 1) * step : 0);
-            const float sum = march_strided<NU>(first, neg ? -step : step, to_lim(k));
-            bad |= !(sum >= 0.f) || isinf(sum);
-            any = true;
-        }
-        __syncthreads();
+    if (kz.nd >= 0) {
+        const Lim<float2> lim = to_lim2(kz, kz);
+        check((kz.nd & 1) ? plane_uz<NU, true>(plane + l * P, lim) : plane_uz<NU, false>(plane + l * P, lim));
     }
     if constexpr (CODED) {
-        // thread l encodes row l (a u_z line) of its plane as the u_z sweep does: the new
-        // scale is the row's largest value; stochastic rounding with the stream that sweep
-        // draws for the line.  A plane neither sweep touched keeps its codes.
-        if (p0 + q < pend && any) {
-            const long long line = (p0 + q) * NU + l;
-            const float *s = plane + l * P;
-            float v[NU], m = 0.f;
+        __syncthreads();
+        // a thread encodes whole rows (u_z lines) as the u_z sweep does: the new scale is the
+        // row's largest value; stochastic rounding with the stream that sweep draws for the
+        // line.  Planes that neither sweep touched keep their codes.
+        if (ky.nd >= 0 || kz.nd >= 0) {
+#pragma unroll 1
+            for (int r = threadIdx.x; r < ROWS; r += G::threads) {
+                const long long line = p0 * NU + r;
+                const float4 *s = reinterpret_cast<const float4 *>(plane_s + r * P);
+                float m = 0.f;
 #pragma unroll
-            for (int j = 0; j < NU; ++j) {
-                v[j] = s[j];
-                m = fmaxf(m, v[j]);
-            }
-            m = coded_scale<T>(m);
-            a.scale[line] = m;
-            const float inv = inv_scale(m);
-            unsigned rng = sr_bits((unsigned long long)line * NU, a.seed);
-            unsigned char *dst = reinterpret_cast<unsigned char *>(f + line * NU);
+                for (int c = 0; c < NU / 4; ++c) m = mx3(mx3(m, s[c].x, s[c].y), s[c].z, s[c].w);
+                m = coded_scale<T>(m);
+                a.scale[line] = m;
+                const float inv = inv_scale(m);
+                unsigned rng = sr_bits((unsigned long long)line * NU, a.seed);
+                unsigned char *dst = reinterpret_cast<unsigned char *>(f + line * NU);
 #pragma unroll
-            for (int c = 0; c < NU / PER; ++c) {
-                float e[PER];
-#pragma unroll
-                for (int i = 0; i < PER; ++i) e[i] = v[PER * c + i];
-                Chunk<T>::put(dst + 16 * c, inv, e, rng);
+                for (int c = 0; c < NU / PER; ++c) {
+                    const float4 x = s[2 * c], y = s[2 * c + 1];
+                    const float e[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+                    Chunk<T>::put(dst + 16 * c, inv, e, rng);
+                }
             }
         }
     } else {
-        for (int k = threadIdx.x; k < kPlanesPerBlock * Q; k += blockDim.x) {
-            const int qq = k / Q, e = 4 * (k - qq * Q), row = e / NU, col = e - row * NU;
-            if (p0 + qq < pend) {
-                const float *s = plane_s + (qq * NU + row) * P + col;
-                reinterpret_cast<float4 *>(f + (p0 + qq) * NU * NU)[k - qq * Q] = make_float4(s[0], s[1], s[2], s[3]);
-            }
-        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < ROWS / RP; ++k)
+            *reinterpret_cast<float4 *>(g + k * RP * NU) = *reinterpret_cast<const float4 *>(sg + k * RP * P);
     }
     if (bad) atomicOr(a.err, ERR_NAN);
 }
@@ -123,9 +199,9 @@ bool plane_tail_supported(int nuy, int nuz, int nux, int dtype)
 template <typename T> static cudaError_t launch_plane_tail_t(T *f, const PlaneTailArgs &a, long long blocks, cudaStream_t st)
 {
     const cudaError_t e = cudaFuncSetAttribute(plane_tail_kernel<48, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(plane_smem<48>()));
+                                               int(PlaneGeom<48>::smem));
     if (e != cudaSuccess) return e;
-    plane_tail_kernel<48, T><<<unsigned(blocks), kPlanesPerBlock * 48, plane_smem<48>(), st>>>(f, a);
+    plane_tail_kernel<48, T><<<unsigned(blocks), PlaneGeom<48>::threads, PlaneGeom<48>::smem, st>>>(f, a);
     return cudaGetLastError();
 }
 

@@ -26,45 +26,11 @@
 // The same tiles serve the u_x sweep of Eq. (4) (ZF): f viewed as [cell][u_x][u_y u_z],
 // zero-flux lines, one Courant number per tile (the cell's), marched through a window of
 // five cells (march_strided, the arithmetic of the other velocity sweeps).
-#include "vk_lines.cuh"
+#include "vk_tiles.cuh"
 
 namespace vk {
 
 namespace {
-
-__device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1, int c2,
-                                            int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void *src, int c0, int c1, int c2, int c3)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
-            reinterpret_cast<uint64_t>(map)),
-        "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-        : "memory");
-}
-
-// Tile k sits in slot k % S and its load completes a phase of barrier k % 2S: two barriers per
-// slot, taken in turn.  A group takes every NG-th tile, so the tile before k in its slot,
-// k - S, is another group's, and its load can still be in flight when the group waits for
-// tile k (loads complete out of order: the group's own last tile, k - NG, can land first).
-// With one barrier per slot a wait by parity then took the phase before k - S's, which has
-// the parity of k's, for its own, and the group marched a slot that held no tile yet.  The
-// phase before k's on its own barrier is tile k - 2S's, complete because the load of k - S was
-// issued (in order, before that of k - NG) only after tile k - 2S was marched; and tile k + 2S
-// cannot be loaded before tile k is marched.
-template <int S> __device__ __forceinline__ uint64_t *full_bar(uint64_t *full, unsigned k) { return full + k % (2 * S); }
-template <int S> __device__ __forceinline__ bool wait_tile(uint64_t *full, unsigned k)
-{
-    return mbar_wait_bounded(full_bar<S>(full, k), (k / (2 * S)) & 1u);
-}
 
 // thread groups (256 columns each) marching tiles at once; the ring holds one slot more
 template <int L> constexpr int tile_groups() { return L <= 48 ? 3 : 2; }
@@ -78,8 +44,6 @@ template <int L> constexpr int tile_slots()
                : tile_groups<L>() + 1;
 }
 // barriers, the velocity-column table, alignment to 1 KB, the ring
-constexpr size_t kTileBars = 384; // bytes of barriers
-constexpr size_t kTileHeader = kTileBars + kMaxVel * sizeof(LineCoefT<float>);
 template <int L> constexpr size_t tile_smem() { return kTileHeader + 1024 + size_t(tile_slots<L>()) * tile_bytes<L>(); }
 
 // March the periodic line p[0], p[st], ..., p[(L - 1) st] (flow toward +index) in place;
@@ -152,7 +116,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     uint64_t *done = full + 2 * S;                           // S: the tile's group is done with it
     uint64_t *marched = done + S;                        // NG: every column of the group's tile is marched
     LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + kTileBars);
-    static_assert((3 * S + NG) * 8 <= int(kTileBars), "barriers fit ahead of the table");
+    static_assert((3 * S + NG) * 8 <= kTileBars, "barriers fit ahead of the table");
     unsigned char *ring = smem + kTileHeader + ((1024u - ((smem_u32(smem) + unsigned(kTileHeader)) & 1023u)) & 1023u);
     auto slot = [&](unsigned k) { return reinterpret_cast<float *>(ring + size_t(TB) * (k % S)); };
 
@@ -180,7 +144,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         auto load = [&](unsigned k) {
             int u0, o;
             coords(k, u0, o);
-            uint64_t *bar = full_bar<S>(full, k);
+            uint64_t *bar = full_bar(full, k, S);
             mbar_arrive_expect_tx(bar, TB);
             tma_load_4d(slot(k), &map, bar, 0, u0, 0, o);
         };
@@ -205,7 +169,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
         if (!ok) {
             atomicOr(a.err, ERR_TIMEOUT);
             // let the loads in flight (the last S at most) land before the CTA exits
-            for (unsigned k = loaded > unsigned(S) ? loaded - S : 0; k < loaded; ++k) wait_tile<S>(full, k);
+            for (unsigned k = loaded > unsigned(S) ? loaded - S : 0; k < loaded; ++k) wait_tile(full, k, S);
         }
         return;
     }
@@ -226,7 +190,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     const int coff = unit * 32 + (((e >> 2) ^ (unit & 7)) << 2) + (e & 3);
     bool bad = false;
     for (unsigned k = grp; k < n_my; k += NG) {
-        if (!__all_sync(0xffffffffu, wait_tile<S>(full, k))) {
+        if (!__all_sync(0xffffffffu, wait_tile(full, k, S))) {
             atomicOr(a.err, ERR_TIMEOUT);
             return;
         }
@@ -274,261 +238,6 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     if (bad) atomicOr(a.err, ERR_NAN);
 }
 
-// ----------------------------------------------------------------------------
-// 16-bit storage (BF16 / FP16 codes, one FP32 scale per u_z line of 32 or 48 cells)
-// ----------------------------------------------------------------------------
-// The same tiles, 512-byte rows of codes (no swizzle) plus the tile's scales (box
-// {8 u_z lines, L rows} for n_uz = 32); a position sweep and a u_x sweep keep every scale.  Each value decodes as
-// code x scale, the line is marched in FP32 and every value is encoded back with
-// stochastic rounding (one stream per column and sweep, one draw per value in march
-// order).  z sweep: warp w takes the columns of one sign of units 2 (w % 4) and
-// 2 (w % 4) + 1 (adjacent 64-byte units fall on disjoint banks).
-// n_uz = 48: a tile's 256 columns fall on 6 or 7 u_z lines, starting anywhere in one; its
-// scale box starts at the line index rounded down to a multiple of 4 (the 16-byte rule of
-// TMA) and spans 12 lines.  n_uz = 32: the 8 lines of the tile exactly.
-template <int NZ> constexpr int tile16_scale_lines() { return NZ == 32 ? 8 : 12; }
-template <int L> constexpr unsigned tile16_codes() { return unsigned(L) * 512u; }
-template <int L, int NZ = 32> constexpr unsigned tile16_slot()
-{
-    return (tile16_codes<L>() + unsigned(L) * 4u * unsigned(tile16_scale_lines<NZ>()) + 127u) & ~127u;
-}
-template <int L, int NZ = 32> constexpr int tile16_slots()
-{
-    return (196608 / tile16_slot<L, NZ>() > 12 ? 12 : int(196608 / tile16_slot<L, NZ>())) > tile_groups<L>() + 1
-               ? (196608 / tile16_slot<L, NZ>() > 12 ? 12 : int(196608 / tile16_slot<L, NZ>()))
-               : tile_groups<L>() + 1;
-}
-// after the ring: per consumer warp, the inverse scales of the (up to two) u_z lines its
-// columns belong to, one per row, formed once per tile instead of once per value
-template <int L> constexpr size_t tile16_inv_bytes() { return size_t(tile_groups<L>()) * 8 * 2 * L * sizeof(float); }
-template <int L, int NZ = 32> constexpr size_t tile16_smem()
-{
-    return kTileHeader + 1024 + size_t(tile16_slots<L, NZ>()) * tile16_slot<L, NZ>() + tile16_inv_bytes<L>();
-}
-
-template <int L, int DIR, typename T, int SX = 8>
-__device__ __forceinline__ float march_tile16(T *p, const float *sp, const float *ip, int st_rt, const Lim<float> &lim,
-                                              unsigned rng)
-{
-    const int st = DIR == 0 ? st_rt : DIR * 256;                // rows are 256 codes apart
-    const int ss = DIR == 0 ? (st_rt > 0 ? SX : -SX) : DIR * SX; // and SX scales
-    const int is = DIR == 0 ? (st_rt > 0 ? 1 : -1) : DIR;     // and 1 inverse scale
-    auto get = [&](int i) { return RegCodec<T>::get(p[i * st], sp[i * ss]); };
-    auto put = [&](int i, float v) { p[i * st] = RegCodec<T>::put(v, ip[i * is], lcg_next(rng) >> 16); };
-    const float s0 = get(0), s1 = get(1);
-    March<float> m(lim);
-    m.start_periodic(get(L - 3), get(L - 2), get(L - 1), s0, s1);
-    constexpr int B = march_block<L>();
-#pragma unroll 1
-    for (int b = 0; b < (L - 2) / B; ++b, p += B * st, sp += B * ss, ip += B * is)
-#pragma unroll
-        for (int q = 0; q < B; ++q) put(q, m.face(get(q + 2)));
-    constexpr int R = (L - 2) % B;
-#pragma unroll
-    for (int q = 0; q < R; ++q) put(q, m.face(get(q + 2)));
-    put(R, m.face(s0));
-    put(R + 1, m.face(s1));
-    return m.sum;
-}
-
-// march_strided on codes: a value is decoded (the scale of its row) as it enters the
-// window and a new value encoded (the inverse scale of its row, one stochastic-rounding
-// draw per cell in walk order) at its own face.  st, ss, is: the strides between rows of
-// codes, scales and inverse scales (negative for a line walked from its far end).
-template <int L, typename T>
-__device__ __forceinline__ float march_tile16_zf(T *p, int st, const float *sp, int ss, const float *ip, int is,
-                                                 const Lim<float> &lim, unsigned rng)
-{
-    static_assert(L >= 4, "lines of at least 4 cells");
-    auto get = [&](int i) { return RegCodec<T>::get(p[i * st], sp[i * ss]); };
-    auto put = [&](int i, float v) { p[i * st] = RegCodec<T>::put(v, ip[i * is], lcg_next(rng) >> 16); };
-    March<float> m(lim);
-    m.start_zero(get(0), get(1));
-    constexpr int B = 8, R = (L - 2) % B;
-#pragma unroll 1
-    for (int b = 0; b < (L - 2) / B; ++b, p += B * st, sp += B * ss, ip += B * is)
-#pragma unroll
-        for (int q = 0; q < B; ++q) put(q, m.face(get(q + 2)));
-#pragma unroll
-    for (int q = 0; q < R; ++q) put(q, m.face(get(q + 2)));
-    put(R, m.face(0.f));
-    put(R + 1, m.last());
-    return m.sum;
-}
-
-template <int L, typename T, bool SIGNED, int NZ = 32, bool ZF = false>
-__global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
-    tile_sweep16_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap smap,
-                        const __grid_constant__ TileArgs a)
-{
-    constexpr int NG = tile_groups<L>(), S = tile16_slots<L, NZ>(), NT = NG * 256, SX = tile16_scale_lines<NZ>();
-    constexpr unsigned CB = tile16_codes<L>(), SB = tile16_slot<L, NZ>();
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem);
-    uint64_t *done = full + 2 * S;
-    LineCoefT<float> *tab = reinterpret_cast<LineCoefT<float> *>(smem + kTileBars);
-    static_assert(3 * S * 8 <= int(kTileBars), "barriers fit ahead of the table");
-    unsigned char *ring = smem + kTileHeader + ((1024u - ((smem_u32(smem) + unsigned(kTileHeader)) & 1023u)) & 1023u);
-    auto slot = [&](unsigned k) { return reinterpret_cast<T *>(ring + size_t(SB) * (k % S)); };
-    auto sslot = [&](unsigned k) { return reinterpret_cast<float *>(ring + size_t(SB) * (k % S) + CB); };
-    float *winv = reinterpret_cast<float *>(ring + size_t(SB) * S);
-    static_assert(tile16_smem<L, NZ>() <= 227 * 1024, "the tiles and inverse scales fit shared memory");
-
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < 2 * S; ++q) mbar_init(&full[q], 1);
-        for (int q = 0; q < S; ++q) mbar_init(&done[q], 256);
-        fence_barrier_init();
-    }
-    for (int j = threadIdx.x; j < a.nvel; j += blockDim.x) tab[j] = a.table[j];
-    __syncthreads();
-
-    const long long G = gridDim.x, b = blockIdx.x;
-    const unsigned n_my = unsigned(a.num_tiles > b ? (a.num_tiles - b + G - 1) / G : 0);
-    auto coords = [&](unsigned k, int &u0, int &o) {
-        const long long t = a.tile0 + b + (long long)k * G;
-        const long long oq = t / a.tiles_inner;
-        u0 = int((t - oq * a.tiles_inner) * 8);
-        o = int(oq);
-    };
-    // first u_z line of the tile's scale box (n_uz = 32: its first line exactly)
-    auto line0 = [&](int u0) { return NZ == 32 ? u0 : int(32ll * u0 / NZ / 4 * 4); };
-
-    if (threadIdx.x >= NT) {
-        if (threadIdx.x != NT) return;
-        auto load = [&](unsigned k) {
-            int u0, o;
-            coords(k, u0, o);
-            uint64_t *bar = full_bar<S>(full, k);
-            mbar_arrive_expect_tx(bar, CB + unsigned(L) * 4u * unsigned(SX));
-            tma_load_4d(slot(k), &map, bar, 0, u0, 0, o);
-            tma_load_3d(sslot(k), &smap, bar, line0(u0), 0, o);
-        };
-        unsigned loaded = 0;
-        for (; loaded < unsigned(S) && loaded < n_my; ++loaded) load(loaded);
-        bool ok = true;
-        for (unsigned k = 0; k < n_my; ++k) {
-            if (!mbar_wait_bounded(&done[k % S], (k / S) & 1u)) {
-                ok = false;
-                break;
-            }
-            int u0, o;
-            coords(k, u0, o);
-            tma_store_4d(&map, slot(k), 0, u0, 0, o); // the scales stay as they are
-            bulk_commit();
-            if (loaded < n_my) {
-                bulk_wait_read_all();
-                load(loaded++);
-            }
-        }
-        bulk_wait_all();
-        if (!ok) {
-            atomicOr(a.err, ERR_TIMEOUT);
-            // let the loads in flight (the last S at most) land before the CTA exits
-            for (unsigned k = loaded > unsigned(S) ? loaded - S : 0; k < loaded; ++k) wait_tile<S>(full, k);
-        }
-        return;
-    }
-
-    const int grp = threadIdx.x >> 8, tid = threadIdx.x & 255, w = tid >> 5, lane = tid & 31;
-    int unit, e;
-    if (a.zperm) {
-        unit = ((w & 3) << 1) + (lane >> 4);
-        e = (w >> 2) * 16 + (lane & 15);
-    } else {
-        unit = w;
-        e = lane;
-    }
-    // this warp's inverse scales: [h][row] for the (up to two) u_z lines of its columns
-    float *wi = winv + (grp * 8 + w) * 2 * L;
-    bool bad = false;
-    for (unsigned k = grp; k < n_my; k += NG) {
-        if (!__all_sync(0xffffffffu, wait_tile<S>(full, k))) {
-            atomicOr(a.err, ERR_TIMEOUT);
-            return;
-        }
-        int u0, o;
-        coords(k, u0, o);
-        const long long inner = 32ll * (u0 + unit) + e;
-        const LineCoefT<float> kc = ZF ? a.cell_coef[o] : tab[(inner / a.vstride) % a.nvel];
-        T *p = slot(k) + unit * 32 + e;
-        // the scale box column of this thread's u_z line, the warp's first such column and
-        // how many the warp spans (n_uz = 32: units are lines, two under zperm)
-        int col, first, nlines;
-        if constexpr (NZ == 32) {
-            col = unit;
-            first = a.zperm ? ((w & 3) << 1) : w;
-            nlines = a.zperm ? 2 : 1;
-        } else {
-            // (no zperm: the warp's 32 columns are contiguous, on one or two lines)
-            const long long x0 = line0(u0), c0 = 32ll * (u0 + w);
-            col = int(inner / NZ - x0);
-            first = int(c0 / NZ - x0);
-            nlines = int((c0 + 31) / NZ - c0 / NZ) + 1;
-        }
-        const float *sp = sslot(k) + col;
-        const float *ip_col = wi + (col - first) * L;
-        __syncwarp(); // every lane is done with the previous tile's inverses
-        for (int idx = lane; idx < nlines * L; idx += 32) {
-            const int h = idx / L, r = idx - h * L;
-            wi[idx] = inv_scale(sslot(k)[r * SX + first + h]);
-        }
-        __syncwarp();
-        if (kc.nd >= 0) {
-            const Lim<float> lim = to_lim(kc);
-            const bool neg = kc.nd & 1;
-            // the column's stream, from the index of its first cell
-            const unsigned rng = sr_bits((unsigned long long)((long long)o * L * a.n_inner + inner), a.seed);
-            float sum;
-            if constexpr (ZF)
-                sum = march_tile16_zf<L, T>(neg ? p + (L - 1) * 256 : p, neg ? -256 : 256, neg ? sp + (L - 1) * SX : sp,
-                                            neg ? -SX : SX, neg ? ip_col + (L - 1) : ip_col, neg ? -1 : 1, lim, rng);
-            else if constexpr (!SIGNED)
-                sum = march_tile16<L, 0, T, SX>(neg ? p + (L - 1) * 256 : p, neg ? sp + (L - 1) * SX : sp,
-                                                neg ? ip_col + (L - 1) : ip_col, neg ? -256 : 256, lim, rng);
-            else if (neg)
-                sum = march_tile16<L, -1, T, SX>(p + (L - 1) * 256, sp + (L - 1) * SX, ip_col + (L - 1), 0, lim, rng);
-            else sum = march_tile16<L, 1, T, SX>(p, sp, ip_col, 0, lim, rng);
-            bad |= !(sum >= 0.f) || isinf(sum);
-        }
-        fence_proxy_async();
-        mbar_arrive(&done[k % S]);
-    }
-    if (bad) atomicOr(a.err, ERR_NAN);
-}
-
-template <int L, typename T, int NZ = 32> const void *tile16_kernel(bool sign)
-{
-    return sign ? (const void *)tile_sweep16_kernel<L, T, true, NZ> : (const void *)tile_sweep16_kernel<L, T, false, NZ>;
-}
-
-template <typename T> const void *tile16_kernel_for(int L, bool sign, int nuz)
-{
-    if (nuz == 48) return L == 48 ? tile16_kernel<48, T, 48>(sign) : nullptr;
-    if (nuz != 32) return nullptr;
-    switch (L) {
-    case 16: return tile16_kernel<16, T>(sign);
-    case 24: return tile16_kernel<24, T>(sign);
-    case 32: return tile16_kernel<32, T>(sign);
-    case 48: return tile16_kernel<48, T>(sign);
-    case 64: return tile16_kernel<64, T>(sign);
-    case 96: return tile16_kernel<96, T>(sign);
-    default: return nullptr;
-    }
-}
-
-size_t tile16_smem_for(int L, int nuz)
-{
-    if (nuz == 48) return tile16_smem<48, 48>();
-    switch (L) {
-    case 16: return tile16_smem<16>();
-    case 24: return tile16_smem<24>();
-    case 32: return tile16_smem<32>();
-    case 48: return tile16_smem<48>();
-    case 64: return tile16_smem<64>();
-    default: return tile16_smem<96>();
-    }
-}
-
 template <int L> const void *tile_kernel(bool moment, bool sign)
 {
     if (sign) return moment ? (const void *)tile_sweep_kernel<L, true, true> : (const void *)tile_sweep_kernel<L, false, true>;
@@ -558,67 +267,41 @@ size_t tile_smem_for(int L)
     }
 }
 
-int tile_threads_for(int L, bool) { return (L <= 48 ? 3 : 2) * 256 + kProducer; }
+int tile_threads_for(int L) { return (L <= 48 ? 3 : 2) * 256 + kProducer; }
 
 // u_x sweeps (zero-flux lines, one direction per tile): lines of 48 cells
-const void *tile_kernel_zf(int L, int dtype, int nuz)
-{
-    if (L != 48) return nullptr;
-    if (dtype == 1) return (const void *)tile_sweep_kernel<48, false, true, true>;
-    if (nuz != 48) return nullptr;
-    if (dtype == 2) return (const void *)tile_sweep16_kernel<48, __nv_bfloat16, true, 48, true>;
-    if (dtype == 3) return (const void *)tile_sweep16_kernel<48, __half, true, 48, true>;
-    return nullptr;
-}
-
-const void *tile_kernel_any(int L, int dtype, bool moment, bool sign, int nuz)
-{
-    if (dtype == 2) return moment ? nullptr : tile16_kernel_for<__nv_bfloat16>(L, sign, nuz);
-    if (dtype == 3) return moment ? nullptr : tile16_kernel_for<__half>(L, sign, nuz);
-    return tile_kernel_for(L, moment, sign);
-}
+const void *tile_kernel_zf(int L) { return L == 48 ? (const void *)tile_sweep_kernel<48, false, true, true> : nullptr; }
 
 } // namespace
 
-bool tile_sweep_supported(int L, long long n_inner, int dtype, int nuz)
-{
-    if (n_inner % 256 != 0 || !tile_kernel_any(L, dtype, false, true, nuz)) return false;
-    return dtype == 1 || ((dtype == 2 || dtype == 3) && n_inner % nuz == 0);
-}
+bool tile_sweep_supported(int L, long long n_inner) { return n_inner % 256 == 0 && tile_kernel_for(L, false) != nullptr; }
 
-bool tile_sweep_zf_supported(int L, long long n_inner, int dtype, int nuz)
-{
-    return n_inner % 256 == 0 && n_inner % nuz == 0 && tile_kernel_zf(L, dtype, nuz) != nullptr;
-}
+bool tile_sweep_zf_supported(int L, long long n_inner) { return n_inner % 256 == 0 && tile_kernel_zf(L) != nullptr; }
 
-int occupancy_tile_sweep(int L, int dtype, bool moment, int nuz)
+int occupancy_tile_sweep(int L, bool moment)
 {
-    const void *k = tile_kernel_any(L, dtype, moment, true, nuz);
+    const void *k = tile_kernel_for(L, moment);
     if (!k) return 0;
-    const size_t smem = dtype == 1 ? tile_smem_for(L) : tile16_smem_for(L, nuz);
+    const size_t smem = tile_smem_for(L);
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, tile_threads_for(L, moment), smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, tile_threads_for(L), smem) != cudaSuccess) return 0;
     return n;
 }
 
-cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const CUtensorMap &smap,
-                              const TileArgs &a, int dtype, int grid, cudaStream_t st)
+cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const TileArgs &a, int grid, cudaStream_t st)
 {
     if (a.num_tiles <= 0 || grid <= 0) return cudaSuccess;
     const bool moment = a.mpart != nullptr, zf = a.cell_coef != nullptr;
-    const void *k = zf ? tile_kernel_zf(a.L, dtype, a.nuz) : tile_kernel_any(a.L, dtype, moment, a.tile_sign != 0, a.nuz);
+    const void *k = zf ? tile_kernel_zf(a.L) : tile_kernel_for(a.L, moment, a.tile_sign != 0);
     if (!k || (!zf && (a.nvel <= 0 || a.vstride <= 0)) || a.nvel > kMaxVel || a.tiles_inner <= 0 || (zf && moment))
         return cudaErrorInvalidValue;
-    if (moment && (dtype != 1 || a.cube % 256 || a.nparts <= 0)) return cudaErrorInvalidValue;
-    if (dtype != 1 && (a.zperm && a.nuz != 32)) return cudaErrorInvalidValue;
-    const size_t smem = dtype == 1 ? tile_smem_for(a.L) : tile16_smem_for(a.L, a.nuz);
+    if (moment && (a.cube % 256 || a.nparts <= 0)) return cudaErrorInvalidValue;
+    const size_t smem = tile_smem_for(a.L);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
-    // FP32: (map, dmap, args); 16-bit: in place (map, smap, args)
-    void *params[] = {const_cast<CUtensorMap *>(&map),
-                      const_cast<CUtensorMap *>(dtype == 1 ? &dmap : &smap), const_cast<TileArgs *>(&a)};
-    return cudaLaunchKernel(k, dim3(grid), dim3(tile_threads_for(a.L, moment)), params, smem, st);
+    void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), const_cast<TileArgs *>(&a)};
+    return cudaLaunchKernel(k, dim3(grid), dim3(tile_threads_for(a.L)), params, smem, st);
 }
 
 } // namespace vk

@@ -245,10 +245,8 @@ struct TileArgs {
     long long tile0, num_tiles;              // tiles [tile0, tile0 + num_tiles), t = outer tiles_inner + block
     long long vstride;                       // column j takes table[(inner / vstride) % nvel]
     int nvel;
-    int nuz;                                 // 16-bit storage: n_uz (32 or 48), the length of a scale's line
     int zperm;                               // z sweep with n_uz = 32: warps grouped by the sign of u_z
     int tile_sign;                           // 1: every warp's columns have one sign of u (else per column)
-    unsigned seed;                           // 16-bit storage: the stochastic-rounding streams of this sweep
     unsigned *err;
     // u_x sweep (zero-flux lines): the Courant numbers per outer index (a cell); null for
     // the position sweeps, which take table[] per column
@@ -259,17 +257,42 @@ struct TileArgs {
     int nparts;
     LineCoefT<float> table[kMaxVel];
 };
-// dtype 1 (FP32), 2 (BF16), 3 (FP16; n_uz = 32 with L up to 96, or n_uz = 48 with L = 48;
-// one scale per u_z line)
-bool tile_sweep_supported(int L, long long n_inner, int dtype, int nuz);
-// the u_x sweep on the same tiles ([cell][u_x][u_y u_z]): lines of 48 cells (16-bit: n_uz = 48)
-bool tile_sweep_zf_supported(int L, long long n_inner, int dtype, int nuz);
-int occupancy_tile_sweep(int L, int dtype, bool moment, int nuz);
-// FP32: tiles loaded through map and stored through dmap (the same map in place).  16-bit:
-// in place through map (codes, box {32, 8, L, 1}, no swizzle) with the scales through smap
-// ([n_outer][L][n_inner / n_uz] floats, box {8, L, 1} for n_uz = 32, {12, L, 1} for 48)
-cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const CUtensorMap &smap,
-                              const TileArgs &a, int dtype, int grid, cudaStream_t st);
+bool tile_sweep_supported(int L, long long n_inner);
+// the u_x sweep on the same tiles ([cell][u_x][u_y u_z]): lines of 48 cells
+bool tile_sweep_zf_supported(int L, long long n_inner);
+int occupancy_tile_sweep(int L, bool moment);
+// tiles loaded through map and stored through dmap (the same map in place)
+cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const TileArgs &a, int grid, cudaStream_t st);
+
+// ----------------------------------------------------------------------------
+// the same on 16-bit storage, two lines per thread (sweep_tile16.cu): position sweeps with
+// |nu| < 1 and u_x sweeps, in place; map views the codes as [n_outer][L][n_inner / 32][32]
+// with box {32, 8, L, 1} (no swizzle), smap the scales as [n_outer][L][n_inner / n_uz] with
+// box {scale_lines, L, 1}
+// ----------------------------------------------------------------------------
+struct Tile16Args {
+    int L, nuz;
+    long long n_inner;
+    unsigned tiles_inner, num_tiles; // tiles_inner = n_inner / 256; num_tiles = n_outer tiles_inner
+    int slots, groups;               // of the ring; thread groups
+    int scale_lines, warp_lines;     // u_z lines of a tile's scale box; most a warp's columns touch
+    int zperm;                       // z sweep: warps grouped by the sign of u_z
+    unsigned slot_bytes;
+    long long vstride;               // column j takes table[(inner / vstride) % nvel]
+    int nvel;
+    unsigned seed;                   // the stochastic-rounding streams of this sweep
+    unsigned *err;
+    const LineCoefT<float> *cell_coef; // u_x sweep: the Courant numbers per outer index (a cell), else null
+    FastDivU32 div_tiles, div_nuz, div_vstride, div_nvel; // set by the launcher
+    LineCoefT<float> table[kMaxVel];
+};
+// fills the sizes of a; false when the shape does not fit these tiles
+// (z: the z sweep, whose sign of u changes inside every u_z line)
+bool tile16_geometry(int L, long long n_inner, long long n_outer, int nuz, bool z, Tile16Args &a);
+int occupancy_tile16(const Tile16Args &a, int dtype, bool zf);
+cudaError_t launch_tile16(const CUtensorMap &map, const CUtensorMap &smap, const Tile16Args &a, int dtype, int grid,
+                          cudaStream_t st);
+
 
 // host launchers (return cudaGetLastError() of the launch); tiles are loaded
 // through map and stored through dmap (the same map for an in-place sweep)

@@ -140,6 +140,7 @@ struct vlasov_ctx {
     CUtensorMap tmap[4], tsmap[4]; // tsmap: 16-bit storage, the scales of a tile
     MapSpec tspec[4];
     int tgrid[4];
+    Tile16Args t16[4]; // 16-bit storage: the sizes of the tiles
     long long ttiles_inner[4], tn_outer[4];
     // the whole kick D_uz D_uy D_ux in one pass (n_ux = n_uy = n_uz = 16 or 32)
     bool can_kick_cube;
@@ -445,33 +446,39 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         long long I = 1, O = 1;
         for (int k = ax + 1; k < 6; ++k) I *= d6[k];
         for (int k = 0; k < ax; ++k) O *= d6[k];
-        // u_x: [cell][u_x][u_y u_z], zero-flux lines of 48 (lines of 16 and 32 take the
-        // one-pass kick or the register lines)
-        const bool ok = ax == 3 ? tile_sweep_zf_supported(int(d6[ax]), I, c->g.dtype, int(c->g.nuz))
-                                : tile_sweep_supported(int(d6[ax]), I, c->g.dtype, int(c->g.nuz));
-        if (!ok || O > 0x7fffffffll || I / 32 > 0x7fffffffll) continue;
-        c->tspec[ax] = spec_tiles(I, d6[ax], O);
+        if (O > 0x7fffffffll || I / 32 > 0x7fffffffll) continue;
+        const int L = int(d6[ax]), nuz = int(c->g.nuz);
+        int occ;
         if (coded) {
-            // codes: 512-byte rows of 32-code units, no swizzle; scales: one per u_z line, a
-            // tile's 8 lines (n_uz = 32) or the 12 from its first line rounded down to a
-            // multiple of 4 (n_uz = 48: the 6 or 7 lines of its 256 columns)
-            const long long nl = I / c->g.nuz;
+            // u_x: [cell][u_x][u_y u_z], zero-flux lines (lines of 16 and 32 take the one-pass kick
+            // or the register lines)
+            if (ax == 3 && reg_lines_supported(L) && L != 48) continue;
+            if (!tile16_geometry(L, I, O, nuz, ax == 2, c->t16[ax])) continue;
+            // codes: 512-byte rows of 32-code units, no swizzle; scales: one per u_z line, those
+            // of a tile's 256 columns
+            const long long nl = I / nuz;
+            c->tspec[ax] = spec_tiles(I, L, O);
             c->tspec[ax].type = tmap_type(c->g.dtype);
-            c->tspec[ax].gstr[0] = 64; c->tspec[ax].gstr[1] = (cuuint64_t)(I * 2); c->tspec[ax].gstr[2] = (cuuint64_t)(I * d6[ax] * 2);
+            c->tspec[ax].gstr[0] = 64; c->tspec[ax].gstr[1] = (cuuint64_t)(I * 2); c->tspec[ax].gstr[2] = (cuuint64_t)(I * L * 2);
             c->tspec[ax].swz = CU_TENSOR_MAP_SWIZZLE_NONE;
             MapSpec ss{};
             ss.type = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
             ss.rank = 3;
-            ss.gdim[0] = (cuuint64_t)nl; ss.gdim[1] = (cuuint64_t)d6[ax]; ss.gdim[2] = (cuuint64_t)O;
-            ss.gstr[0] = (cuuint64_t)(nl * 4); ss.gstr[1] = (cuuint64_t)(nl * d6[ax] * 4);
-            ss.box[0] = c->g.nuz == 32 ? 8 : 12; ss.box[1] = (cuuint32_t)d6[ax]; ss.box[2] = 1;
+            ss.gdim[0] = (cuuint64_t)nl; ss.gdim[1] = (cuuint64_t)L; ss.gdim[2] = (cuuint64_t)O;
+            ss.gstr[0] = (cuuint64_t)(nl * 4); ss.gstr[1] = (cuuint64_t)(nl * L * 4);
+            ss.box[0] = (cuuint32_t)c->t16[ax].scale_lines; ss.box[1] = (cuuint32_t)L; ss.box[2] = 1;
             ss.swz = CU_TENSOR_MAP_SWIZZLE_NONE;
             ss.promo = CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
             if (encode_spec(&c->tsmap[ax], ss, c->scale) != CUDA_SUCCESS) continue;
+            occ = occupancy_tile16(c->t16[ax], c->g.dtype, ax == 3);
+        } else {
+            // u_x: zero-flux lines of 48
+            if (!(ax == 3 ? tile_sweep_zf_supported(L, I) : tile_sweep_supported(L, I))) continue;
+            c->tspec[ax] = spec_tiles(I, L, O);
+            occ = occupancy_tile_sweep(L, ax == 0);
         }
-        if (encode_spec(&c->tmap[ax], c->tspec[ax], c->f) != CUDA_SUCCESS) continue;
-        const int occ = occupancy_tile_sweep(int(d6[ax]), c->g.dtype, ax == 0 && !coded, int(c->g.nuz));
         if (occ <= 0) continue;
+        if (encode_spec(&c->tmap[ax], c->tspec[ax], c->f) != CUDA_SUCCESS) continue;
         c->ttiles_inner[ax] = I / 256;
         c->tn_outer[ax] = O;
         const long long tiles = O * (I / 256);
@@ -816,8 +823,23 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
     for (int j = 0; j < nvel; ++j) numax = fmax(numax, fabs((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx)));
     SweepMaps m;
     int rc;
+    if (numax < 1.0 && c->use_tiles && c->tile_ok[ax] && coded(c)) {
+        // no whole-cell shift: whole lines staged per tile, in place (checked above)
+        Tile16Args A = c->t16[ax];
+        A.num_tiles = unsigned(c->tn_outer[ax] * c->ttiles_inner[ax]);
+        A.vstride = vstride;
+        A.nvel = nvel;
+        A.seed = c->sweeps;
+        A.err = c->d_err;
+        A.cell_coef = nullptr;
+        for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
+        PartTimer t(c, ax, 1);
+        const cudaError_t e = launch_tile16(c->tmap[ax], c->tsmap[ax], A, c->g.dtype, c->tgrid[ax], c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "position sweep launch");
+        return VLASOV_OK;
+    }
     if (numax < 1.0 && c->use_tiles && c->tile_ok[ax]) {
-        // no whole-cell shift: whole lines staged per tile
+        // the same on FP32 storage
         TileArgs A{};
         A.L = (&c->g.nx)[ax];
         A.n_inner = c->ttiles_inner[ax] * 256;
@@ -832,7 +854,6 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         }
         A.vstride = vstride;
         A.nvel = nvel;
-        A.nuz = int(c->g.nuz);
         A.zperm = ax == 2 && c->g.nuz == 32;
         // Tiles have one sign of u when its runs (vstride nvel / 2 columns: u_j < 0 exactly for
         // j < nvel / 2) are whole tiles; the march then takes a fixed direction per tile (D_x,
@@ -844,17 +865,15 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         const int grid = int(A.num_tiles < c->tgrid[ax] ? A.num_tiles : c->tgrid[ax]);
         A.tile_sign = A.zperm || (nvel % 2 == 0 && run % 256 == 0);
         A.err = c->d_err;
-        A.seed = c->sweeps;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
         const long long cube = velocity_cube(c);
-        const bool fm = rho_fused && ax == 0 && !coded(c) && c->fuse_moment && cube % 256 == 0 && moment_buffer(c);
+        const bool fm = rho_fused && ax == 0 && c->fuse_moment && cube % 256 == 0 && moment_buffer(c);
         if (fm) { A.mpart = c->d_mpart; A.cube = cube; A.nparts = int(cube / 256); }
-        if (coded(c)) m.in = m.out = c->tmap[ax]; // 16-bit sweeps run in place (checked above)
-        else if ((rc = sweep_maps(c, c->tmap[ax], c->tspec[ax], src, dst, m))) return rc;
+        if ((rc = sweep_maps(c, c->tmap[ax], c->tspec[ax], src, dst, m))) return rc;
         cudaError_t e;
         {
             PartTimer t(c, ax, 1);
-            e = launch_tile_sweep(m.in, m.out, c->tsmap[ax], A, c->g.dtype, grid, c->stream);
+            e = launch_tile_sweep(m.in, m.out, A, grid, c->stream);
         }
         if (e != cudaSuccess) return cuda_fail(c, e, "position sweep launch");
         if (fm) {
@@ -958,6 +977,19 @@ static bool use_reg_lines(const vlasov_ctx *c, int ax)
 // columns take the coefficients of its cell)
 static int run_tile_ux(vlasov_ctx *c, const void *src, void *dst)
 {
+    if (coded(c)) { // in place (checked by the caller); never on an x-slab
+        Tile16Args A = c->t16[3];
+        A.num_tiles = unsigned(c->tn_outer[3] * c->ttiles_inner[3]);
+        A.vstride = 1;
+        A.nvel = 0;
+        A.seed = c->sweeps;
+        A.err = c->d_err;
+        A.cell_coef = (const LineCoefT<float> *)c->d_coef[0];
+        PartTimer t(c, 3, 1);
+        const cudaError_t e = launch_tile16(c->tmap[3], c->tsmap[3], A, c->g.dtype, c->tgrid[3], c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "u_x tile sweep launch");
+        return VLASOV_OK;
+    }
     TileArgs A{};
     A.L = int(c->g.nux);
     A.n_inner = c->ttiles_inner[3] * 256;
@@ -973,18 +1005,15 @@ static int run_tile_ux(vlasov_ctx *c, const void *src, void *dst)
     if (A.num_tiles <= 0) return VLASOV_OK;
     A.vstride = 1;
     A.nvel = 0;
-    A.nuz = int(c->g.nuz);
     A.tile_sign = 1;
     A.err = c->d_err;
-    A.seed = c->sweeps;
     A.cell_coef = (const LineCoefT<float> *)c->d_coef[0];
     SweepMaps m;
     int rc;
-    if (coded(c)) m.in = m.out = c->tmap[3]; // in place (checked by the caller)
-    else if ((rc = sweep_maps(c, c->tmap[3], c->tspec[3], src, dst, m))) return rc;
+    if ((rc = sweep_maps(c, c->tmap[3], c->tspec[3], src, dst, m))) return rc;
     const int grid = int(A.num_tiles < c->tgrid[3] ? A.num_tiles : c->tgrid[3]);
     PartTimer t(c, 3, 1);
-    const cudaError_t e = launch_tile_sweep(m.in, m.out, c->tsmap[3], A, c->g.dtype, grid, c->stream);
+    const cudaError_t e = launch_tile_sweep(m.in, m.out, A, grid, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "u_x tile sweep launch");
     return VLASOV_OK;
 }

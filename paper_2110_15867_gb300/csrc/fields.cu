@@ -18,54 +18,59 @@ namespace vk {
 // velocity-sweep coefficients
 // ----------------------------------------------------------------------------
 
+// One thread per cell and axis (blockIdx.y): the FP64 chain of a cell (the gradient, the five
+// weights, a division; FP64 runs at 2 lanes per SM and clock) is what a small grid waits
+// for, so its axes run side by side and small grids take small blocks, which spread over
+// more SMs.  8^3 cells: 25 us with one thread per cell walking the three axes in blocks of
+// 256, 8 us here; 64 x 64 x 32: 83 -> 48 us.
+struct CoefAxes {
+    double scale[3]; // nu = scale (8 (phi_+1 - phi_-1) - (phi_+2 - phi_-2)): -dt / (12 h du)
+    int axis[3];
+};
 template <typename C>
-__global__ void velocity_coef_kernel(GridDims g, const float *__restrict__ phi, double dt, int mask,
+__global__ void velocity_coef_kernel(int nx, int ny, int nz, const float *__restrict__ phi, CoefAxes ax,
                                      LineCoefT<C> *cx, LineCoefT<C> *cy, LineCoefT<C> *cz, unsigned *err)
 {
-    const long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int iz = int(c % g.n[2]);
-        const int iy = int((c / g.n[2]) % g.n[1]);
-        const int ix = int(c / ((long long)g.n[2] * g.n[1]));
-        const int idx[3] = {ix, iy, iz};
-        LineCoefT<C> *outs[3] = {cx, cy, cz};
-        for (int d = 0; d < 3; ++d) {
-            if (!(mask & (1 << d))) continue;
-            double v[5];
-            for (int o = -2; o <= 2; ++o) {
-                int q[3] = {idx[0], idx[1], idx[2]};
-                q[d] = (q[d] + o + 2 * g.n[d]) % g.n[d];
-                v[o + 2] = (double)phi[((long long)q[0] * g.n[1] + q[1]) * g.n[2] + q[2]];
-            }
-            const double h = g.L / g.n[d];
-            const double grad = (8.0 * (v[3] - v[1]) - (v[4] - v[0])) / (12.0 * h);
-            const double du = 2.0 * g.V / g.nu[d];
-            const double nu = -grad * dt / du;
-            LineCoefT<C> k = make_line_coef<C>(nu);
-            if (!(fabs(nu) < 1.0)) { // also catches NaN
-                k.nd = -1;
-                atomicOr(err, ERR_CFL);
-            }
-            outs[d][c] = k;
-        }
+    const unsigned ncell = unsigned(nx) * ny * nz; // <= 2^24
+    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= ncell) return;
+    const int d = ax.axis[blockIdx.y];
+    const int st = d == 2 ? 1 : d == 1 ? nz : ny * nz, n = d == 2 ? nz : d == 1 ? ny : nx;
+    const int i = int(c / unsigned(st) % unsigned(n));
+    auto at = [&](int o) { // cell i + o of the periodic line, |o| <= 2 <= n
+        const int q = i + o;
+        return (double)phi[int(c) + (q < 0 ? o + n : q >= n ? o - n : o) * st];
+    };
+    const double nu = ax.scale[blockIdx.y] * (8.0 * (at(1) - at(-1)) - (at(2) - at(-2)));
+    LineCoefT<C> k = make_line_coef<C>(nu);
+    if (!(fabs(nu) < 1.0)) { // also catches NaN
+        k.nd = -1;
+        atomicOr(err, ERR_CFL);
     }
+    (d == 0 ? cx : d == 1 ? cy : cz)[c] = k;
 }
 
 cudaError_t launch_velocity_coef(const GridDims &g, const float *phi, double dt, int mask, void *coef_x,
                                  void *coef_y, void *coef_z, int dtype, unsigned *err, cudaStream_t st)
 {
     const long long ncell = (long long)g.n[0] * g.n[1] * g.n[2];
-    const int threads = 256;
-    const int blocks = int((ncell + threads - 1) / threads < 4096 ? (ncell + threads - 1) / threads : 4096);
+    CoefAxes ax{};
+    int axes = 0;
+    for (int d = 0; d < 3; ++d) {
+        if (!(mask & (1 << d))) continue;
+        const double h = g.L / g.n[d], du = 2.0 * g.V / g.nu[d];
+        ax.scale[axes] = -dt / (12.0 * h * du);
+        ax.axis[axes++] = d;
+    }
+    if (!axes) return cudaSuccess;
+    const int threads = ncell >= 65536 ? 128 : 32;
+    const dim3 grid(unsigned((ncell + threads - 1) / threads), unsigned(axes));
     if (dtype == 0)
-        velocity_coef_kernel<double><<<blocks, threads, 0, st>>>(
-            g, phi, dt, mask, (LineCoefT<double> *)coef_x, (LineCoefT<double> *)coef_y,
-            (LineCoefT<double> *)coef_z, err);
+        velocity_coef_kernel<double><<<grid, threads, 0, st>>>(g.n[0], g.n[1], g.n[2], phi, ax, (LineCoefT<double> *)coef_x,
+                                                              (LineCoefT<double> *)coef_y, (LineCoefT<double> *)coef_z, err);
     else
-        velocity_coef_kernel<float><<<blocks, threads, 0, st>>>(
-            g, phi, dt, mask, (LineCoefT<float> *)coef_x, (LineCoefT<float> *)coef_y,
-            (LineCoefT<float> *)coef_z, err);
+        velocity_coef_kernel<float><<<grid, threads, 0, st>>>(g.n[0], g.n[1], g.n[2], phi, ax, (LineCoefT<float> *)coef_x,
+                                                             (LineCoefT<float> *)coef_y, (LineCoefT<float> *)coef_z, err);
     return cudaGetLastError();
 }
 
@@ -506,13 +511,6 @@ cudaError_t launch_mass(const GridDims &g, const double *rho, double *out, cudaS
 // Poisson, Eq. (2)
 // ----------------------------------------------------------------------------
 
-__global__ void poisson_load_kernel(long long n, const double *__restrict__ rho, const double *__restrict__ bg,
-                                    double2 *z)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        z[i] = make_double2(rho[i] + (bg ? bg[i] : 0.0), 0.0);
-}
-
 // DFT along dimension d: out[.., k, ..] = sum_m in[.., m, ..] e^{sign 2 pi i k m / n_d},
 // factored once (Cooley-Tukey) as n = n1 n2 with m = n2 m1 + m2 and k = k1 + n1 k2:
 //   Y[k1][m2] = W_n^{m2 k1} sum_{m1} x[n2 m1 + m2] W_{n1}^{m1 k1},
@@ -520,66 +518,105 @@ __global__ void poisson_load_kernel(long long n, const double *__restrict__ rho,
 // n (n1 + n2 + 1) complex products per line instead of n^2 (n1 = 1 for a prime n: the
 // plain sum).  W_{n1} = W_n^{n2}, W_{n2} = W_n^{n1}: one twiddle table per axis.  A
 // block holds `lines` lines of the axis in shared memory, n threads per line.
-__global__ void __launch_bounds__(256) dft_axis_kernel(GridDims g, int d, int sign, int n1, int lines,
-                                                       const double2 *__restrict__ in, double2 *out,
-                                                       const double2 *__restrict__ tw)
+//
+// The solve is five launches: z (reading rho + rho_bg), y, x forward with the division by k^2
+// and x back on the same lines, y back, z back (writing phi).  Small grids are bound by the
+// launches and by each one's chain of dependent FP64 operations and loads, so blocks are kept
+// small there (more SMs) and the twiddles come through shared memory.  8^3: 67 us in nine
+// launches, 38 us here; 64 x 64 x 32: 250 -> 226 us.
+// One output per thread of the n-point transform of x (y: scratch); all threads of the block
+// call it.  x must not be written again before the next barrier.
+__device__ __forceinline__ double2 dft_point(const double2 *x, double2 *y, const double2 *tw, int n, int n1, int k, int sign,
+                                             bool act)
 {
-    extern __shared__ double2 dft_smem[];
-    const long long n0 = g.n[0], nn1 = g.n[1], nn2 = g.n[2];
-    const long long st[3] = {nn1 * nn2, nn2, 1};
-    const int n = g.n[d], n2 = n / n1;
-    const long long nlines = n0 * nn1 * nn2 / n;
-    // the other two dimensions of a line, in memory order
-    const int da = d == 0 ? 1 : 0, db = d == 2 ? 1 : 2;
-    const long long nb = g.n[db];
-    const int li = threadIdx.x / n, k = threadIdx.x % n; // this thread: line li of the block, index k
-    double2 *x = dft_smem + li * n, *y = dft_smem + lines * n + li * n;
-    for (long long l0 = blockIdx.x * (long long)lines; l0 < nlines; l0 += (long long)gridDim.x * lines) {
-        const long long line = l0 + li;
-        const bool act = li < lines && line < nlines;
-        long long base = 0;
-        if (act) {
-            base = (line / nb) * st[da] + (line % nb) * st[db];
-            x[k] = in[base + k * st[d]];
-        }
-        __syncthreads();
-        if (act) {
-            // stage 1 for (k1, m2) = (k / n2, k % n2)
-            const int k1 = k / n2, m2 = k % n2;
-            double sr = 0.0, si = 0.0;
-            int q = 0; // (n2 m1 k1) mod n
-            for (int m1 = 0; m1 < n1; ++m1) {
-                const double2 v = x[n2 * m1 + m2], w = tw[q];
-                const double wi = sign * w.y;
-                sr += v.x * w.x - v.y * wi;
-                si += v.x * wi + v.y * w.x;
-                q += n2 * k1; // < n
-                if (q >= n) q -= n;
-            }
-            const double2 w = tw[(m2 * k1) % n];
+    const int n2 = n / n1;
+    __syncthreads();
+    if (act) {
+        // stage 1 for (k1, m2) = (k / n2, k % n2)
+        const int k1 = k / n2, m2 = k % n2;
+        double sr = 0.0, si = 0.0;
+        int q = 0; // (n2 m1 k1) mod n
+        for (int m1 = 0; m1 < n1; ++m1) {
+            const double2 v = x[n2 * m1 + m2], w = tw[q];
             const double wi = sign * w.y;
-            y[k] = make_double2(sr * w.x - si * wi, sr * wi + si * w.x); // Y[k1][m2] at k1 n2 + m2
+            sr += v.x * w.x - v.y * wi;
+            si += v.x * wi + v.y * w.x;
+            q += n2 * k1; // < n
+            if (q >= n) q -= n;
         }
-        __syncthreads();
-        if (act) {
-            // stage 2 for output k = k1 + n1 k2
-            const int k1 = k % n1, k2 = k / n1;
-            double sr = 0.0, si = 0.0;
-            int q = 0; // (n1 m2 k2) mod n
-            for (int m2 = 0; m2 < n2; ++m2) {
-                const double2 v = y[k1 * n2 + m2], w = tw[q];
-                const double wi = sign * w.y;
-                sr += v.x * w.x - v.y * wi;
-                si += v.x * wi + v.y * w.x;
-                q += n1 * k2; // < n
-                if (q >= n) q -= n;
-            }
-            out[base + k * st[d]] = make_double2(sr, si);
-        }
-        __syncthreads();
+        const double2 w = tw[(m2 * k1) % n];
+        const double wi = sign * w.y;
+        y[k] = make_double2(sr * w.x - si * wi, sr * wi + si * w.x); // Y[k1][m2] at k1 n2 + m2
     }
+    __syncthreads();
+    double sr = 0.0, si = 0.0;
+    if (act) {
+        // stage 2 for output k = k1 + n1 k2
+        const int k1 = k % n1, k2 = k / n1;
+        int q = 0; // (n1 m2 k2) mod n
+        for (int m2 = 0; m2 < n2; ++m2) {
+            const double2 v = y[k1 * n2 + m2], w = tw[q];
+            const double wi = sign * w.y;
+            sr += v.x * w.x - v.y * wi;
+            si += v.x * wi + v.y * w.x;
+            q += n1 * k2; // < n
+            if (q >= n) q -= n;
+        }
+    }
+    return make_double2(sr, si);
 }
 
+enum class Dft { first, plain, middle, last };
+struct DftArgs {
+    int n[3], d, sign, n1, lines;
+    unsigned nlines;
+    const double *rho, *bg; // first: the real input (bg may be null)
+    const double2 *in, *tw;
+    double2 *out;
+    double fac, L;          // middle: forward, times -fac / k^2 (0 for k = 0), back
+    float *phi;             // last: the real part / ncell, FP32 (the field the kicks read)
+    double *phi64;          // or FP64 (the adjoint's dL/drho); either may be null
+};
+
+template <Dft M> __global__ void __launch_bounds__(256) dft_axis_kernel(const __grid_constant__ DftArgs a)
+{
+    extern __shared__ double2 dft_smem[];
+    const int d = a.d, n = a.n[d];
+    const int st = d == 2 ? 1 : d == 1 ? a.n[2] : a.n[1] * a.n[2];
+    // the other two dimensions of a line, in memory order
+    const int da = d == 0 ? 1 : 0, db = d == 2 ? 1 : 2;
+    const int sa = da == 0 ? a.n[1] * a.n[2] : a.n[2], sb = db == 1 ? a.n[2] : 1;
+    const int li = threadIdx.x / n, k = threadIdx.x - li * n; // this thread: line li of the block, index k
+    double2 *tw = dft_smem, *x = tw + n + li * n, *y = tw + n + (a.lines + li) * n;
+    for (int q = threadIdx.x; q < n; q += blockDim.x) tw[q] = a.tw[q];
+    const unsigned line = blockIdx.x * unsigned(a.lines) + li;
+    const bool act = line < a.nlines;
+    const int ia = int(line / unsigned(a.n[db])), ib = int(line - unsigned(ia) * a.n[db]);
+    const int e = ia * sa + ib * sb + k * st; // < 2^24
+    if (act) x[k] = M == Dft::first ? make_double2(a.rho[e] + (a.bg ? a.bg[e] : 0.0), 0.0) : a.in[e];
+    double2 v = dft_point(x, y, tw, n, a.n1, k, a.sign, act);
+    if constexpr (M == Dft::middle) {
+        const int id[3] = {k, ia, ib}; // d = 0
+        double k2 = 0.0;
+        for (int q = 0; q < 3; ++q) {
+            const int w = id[q] < (a.n[q] + 1) / 2 ? id[q] : id[q] - a.n[q]; // integer wave number
+            const double kq = 2.0 * M_PI * (double)w / a.L;
+            k2 += kq * kq;
+        }
+        const double s = (k2 == 0.0) ? 0.0 : -a.fac / k2;
+        __syncthreads();
+        if (act) x[k] = make_double2(v.x * s, v.y * s);
+        v = dft_point(x, y, tw, n, a.n1, k, -a.sign, act);
+    }
+    if (!act) return;
+    if constexpr (M == Dft::last) {
+        const double p = v.x * (1.0 / ((double)a.n[0] * a.n[1] * a.n[2]));
+        if (a.phi) a.phi[e] = (float)p;
+        if (a.phi64) a.phi64[e] = p;
+    } else {
+        a.out[e] = v;
+    }
+}
 // the factor n1 of n used by dft_axis_kernel: its largest divisor <= sqrt(n)
 static int dft_n1(int n)
 {
@@ -589,55 +626,38 @@ static int dft_n1(int n)
     return best;
 }
 
-__global__ void poisson_scale_kernel(GridDims g, double2 *z, double fac)
-{
-    const long long n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-    const long long total = n0 * n1 * n2;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long id[3] = {i / (n1 * n2), (i / n2) % n1, i % n2};
-        double k2 = 0.0;
-        for (int d = 0; d < 3; ++d) {
-            const long long nd = g.n[d];
-            const long long w = id[d] < (nd + 1) / 2 ? id[d] : id[d] - nd; // integer wave number
-            const double k = 2.0 * M_PI * (double)w / g.L;
-            k2 += k * k;
-        }
-        const double s = (k2 == 0.0) ? 0.0 : -fac / k2;
-        z[i] = make_double2(z[i].x * s, z[i].y * s);
-    }
-}
-
-// FP32 phi (the field the kicks read) or FP64 (the adjoint's dL/drho)
-__global__ void poisson_store_kernel(long long n, const double2 *__restrict__ z, float *phi, double *phi64)
-{
-    const double inv = 1.0 / (double)n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        if (phi) phi[i] = (float)(z[i].x * inv);
-        if (phi64) phi64[i] = z[i].x * inv;
-    }
-}
-
 cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const double *rho, const double *bg,
                            double a, double four_pi_G, float *phi, cudaStream_t st, double *phi64)
 {
     const long long n = (long long)g.n[0] * g.n[1] * g.n[2];
-    const int threads = 256;
-    const int blocks = int((n + threads - 1) / threads < 8192 ? (n + threads - 1) / threads : 8192);
-    poisson_load_kernel<<<blocks, threads, 0, st>>>(n, rho, bg, ps.z0);
-    double2 *a0 = ps.z0, *a1 = ps.z1;
-    auto dft = [&](int d, int sign) {
-        const int nd = g.n[d], lines = 256 / nd; // nd <= 256
-        const long long nlines = n / nd;
-        const long long nb = (nlines + lines - 1) / lines;
-        const int grid = int(nb < 8192 ? nb : 8192);
-        dft_axis_kernel<<<grid, lines * nd, 2 * lines * nd * sizeof(double2), st>>>(g, d, sign, dft_n1(nd), lines, a0,
-                                                                                   a1, ps.tw[d]);
-        double2 *t = a0; a0 = a1; a1 = t;
+    DftArgs A{};
+    for (int d = 0; d < 3; ++d) A.n[d] = g.n[d];
+    A.rho = rho;
+    A.bg = bg;
+    A.fac = four_pi_G * a * a;
+    A.L = g.L;
+    A.phi = phi;
+    A.phi64 = phi64;
+    auto dft = [&](auto kernel, int d, int sign, const double2 *in, double2 *out) {
+        const int nd = g.n[d]; // <= 256
+        A.nlines = unsigned(n / nd);
+        // up to 256 threads a block, but blocks for every SM first (of a warp at least)
+        const int most = 256 / nd, least = nd >= 32 ? 1 : 32 / nd;
+        const int spread = int((A.nlines + 303) / 304);
+        A.lines = spread < least ? least : spread > most ? most : spread;
+        A.d = d;
+        A.sign = sign;
+        A.n1 = dft_n1(nd);
+        A.in = in;
+        A.out = out;
+        A.tw = ps.tw[d];
+        kernel<<<(A.nlines + A.lines - 1) / A.lines, A.lines * nd, (2 * A.lines + 1) * nd * sizeof(double2), st>>>(A);
     };
-    for (int d = 2; d >= 0; --d) dft(d, -1);
-    poisson_scale_kernel<<<blocks, threads, 0, st>>>(g, a0, four_pi_G * a * a);
-    for (int d = 0; d < 3; ++d) dft(d, +1);
-    poisson_store_kernel<<<blocks, threads, 0, st>>>(n, a0, phi, phi64);
+    dft(dft_axis_kernel<Dft::first>, 2, -1, nullptr, ps.z0);
+    dft(dft_axis_kernel<Dft::plain>, 1, -1, ps.z0, ps.z1);
+    dft(dft_axis_kernel<Dft::middle>, 0, -1, ps.z1, ps.z0);
+    dft(dft_axis_kernel<Dft::plain>, 1, +1, ps.z0, ps.z1);
+    dft(dft_axis_kernel<Dft::last>, 2, +1, ps.z1, nullptr);
     return cudaGetLastError();
 }
 

@@ -1180,7 +1180,7 @@ extern "C" int vlasov_poisson(vlasov_ctx *c, const double *rho_dev, const double
     VK_SETTLE(c);
     if (!rho_dev || !phi_dev) return fail(c, VLASOV_EINVAL, "vlasov_poisson: null rho or phi");
     if (!isfinite(a) || !isfinite(four_pi_G)) return fail(c, VLASOV_EINVAL, "vlasov_poisson: a and four_pi_G must be finite");
-    PartTimer t(c, VLASOV_T_POISSON, 9);
+    PartTimer t(c, VLASOV_T_POISSON, 5);
     const cudaError_t e = launch_poisson(c->gd, c->ps, rho_dev, rho_bg_dev, a, four_pi_G, phi_dev, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "poisson launch");
     return VLASOV_OK;
@@ -1899,7 +1899,7 @@ extern "C" int vlasov_step_adjoint_recorded_sc(vlasov_ctx *c, const void *f_n_de
     // Poisson (its own transpose) and the moment
     cudaError_t e;
     {
-        PartTimer t(c, VLASOV_T_POISSON, 9);
+        PartTimer t(c, VLASOV_T_POISSON, 5);
         e = launch_poisson(c->gd, c->ps, dphi1, nullptr, a_full, four_pi_G, nullptr, c->stream, drho);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "poisson adjoint launch");

@@ -189,6 +189,134 @@ __global__ void __launch_bounds__(PlaneGeom<NU>::threads, 5)
     if (bad) atomicOr(a.err, ERR_NAN);
 }
 
+// ----------------------------------------------------------------------------
+// planes of any size (FP32): D_uy, D_uz or both in one pass, in place or src -> dst
+// ----------------------------------------------------------------------------
+// The same marches with the sizes at run time, for every velocity grid that the kernels of
+// fixed sizes do not take.  A block stages as many whole planes as give its 128 threads a
+// pair of lines each (of whatever cells: each pair looks up its own Courant number); the
+// rows' pitch is an odd number of 16-byte units.  Bodies of four faces, whose look-ahead
+// cells are read before the first of their writes.
+// 21 x 26 x 19 x 24 x 20 x 28 cells (1.4e8), per call: D_uy streamed 0.28 ms and D_uz through a
+// shared-memory transpose 0.54 ms; 0.250 and 0.270 ms here, both in one pass
+// 0.378 ms (24^3 x 24^3: a kick 1.23 -> 0.87 ms; DRAM alone 0.165 ms a pass).
+constexpr int kAnyThreads = 128;
+
+__device__ __forceinline__ float2 any_uy(float *p, int st, int n, const Lim<float2> &lim)
+{
+    auto cell = [&](int i) -> float2 & { return *reinterpret_cast<float2 *>(p + i * st); };
+    March<float2> m(lim);
+    m.start_zero(cell(0), cell(1));
+#pragma unroll 1
+    for (int left = n - 4; left > 0; left -= 4, p += 4 * st) { // n is a multiple of 4
+        float2 c[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] = cell(q + 2);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cell(q) = m.face(c[q]);
+    }
+    const float2 a = cell(2), b = cell(3);
+    cell(0) = m.face(a);
+    cell(1) = m.face(b);
+    cell(2) = m.face(make_float2(0.f, 0.f));
+    cell(3) = m.last();
+    return m.sum;
+}
+
+// rows at p and p + other floats, C chunks of four cells
+template <bool NEG> __device__ __forceinline__ float2 any_uz(float *p, int other, int C, const Lim<float2> &lim)
+{
+    constexpr int ST = NEG ? -4 : 4;
+    if (NEG) p += 4 * (C - 1);
+    auto at = [&](int row, int j) -> float4 & { return *reinterpret_cast<float4 *>(p + row + j * ST); };
+    auto pick = [](const float4 &a, const float4 &b, int i) {
+        const int s = NEG ? 3 - i : i;
+        return make_float2((&a.x)[s], (&b.x)[s]);
+    };
+    auto set = [](float4 &a, float4 &b, int i, float2 v) {
+        const int s = NEG ? 3 - i : i;
+        (&a.x)[s] = v.x;
+        (&b.x)[s] = v.y;
+    };
+    March<float2, true> m(lim);
+    float4 a = at(0, 0), b = at(other, 0), oa, ob, na = a, nb = b;
+    if (C > 1) {
+        na = at(0, 1);
+        nb = at(other, 1);
+    }
+    m.start_zero(pick(a, b, 0), pick(a, b, 1));
+    set(oa, ob, 0, m.face(pick(a, b, 2)));
+    set(oa, ob, 1, m.face(pick(a, b, 3)));
+#pragma unroll 1
+    for (int j = 1; j < C; ++j, p += ST) { // chunk j enters; the outputs of chunk j - 1 go to chunk 0 of p
+        a = na;
+        b = nb;
+        if (j + 1 < C) {
+            na = at(0, 2);
+            nb = at(other, 2);
+        }
+        set(oa, ob, 2, m.face(pick(a, b, 0)));
+        set(oa, ob, 3, m.face(pick(a, b, 1)));
+        at(0, 0) = oa;
+        at(other, 0) = ob;
+        set(oa, ob, 0, m.face(pick(a, b, 2)));
+        set(oa, ob, 1, m.face(pick(a, b, 3)));
+    }
+    set(oa, ob, 2, m.face(make_float2(0.f, 0.f)));
+    set(oa, ob, 3, m.last());
+    at(0, 0) = oa;
+    at(other, 0) = ob;
+    return m.sum;
+}
+
+__global__ void __launch_bounds__(kAnyThreads, 5)
+    plane_any_kernel(const float *src, float *dst, const __grid_constant__ PlaneAnyArgs a)
+{
+    extern __shared__ __align__(16) float any_s[];
+    const int ny = a.nuy, nz = a.nuz, pitch = a.pitch, u = nz / 4; // u: 16-byte chunks of a row
+    const long long p0 = a.plane0 + (long long)blockIdx.x * a.per_block, pend = a.plane0 + a.nplanes;
+    const int planes = pend - p0 < a.per_block ? int(pend - p0) : a.per_block;
+    const long long e0 = p0 * ny * nz;
+    const int chunks = planes * ny * u;
+    for (int k = threadIdx.x; k < chunks; k += kAnyThreads) {
+        const int row = int(fdiv(unsigned(k), a.div_u)), col = k - row * u;
+        copy16(any_s + row * pitch + 4 * col, src + e0 + 4ll * k);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    bool bad = false;
+    auto check = [&](float2 s) { bad |= !(s.x >= 0.f) || !(s.y >= 0.f) || isinf(s.x) || isinf(s.y); };
+    if (a.coef_y) {
+        const int half = nz / 2; // column pairs of a plane
+        for (int k = threadIdx.x; k < planes * half; k += kAnyThreads) {
+            const int q = int(fdiv(unsigned(k), a.div_hz)), c = k - q * half;
+            const LineCoefT<float> ky = a.coef_y[fdiv(unsigned(p0 + q), a.div_nux)];
+            if (ky.nd < 0) continue;
+            const bool neg = ky.nd & 1;
+            const Lim<float2> lim = to_lim2(ky, ky);
+            check(any_uy(any_s + (q * ny + (neg ? ny - 1 : 0)) * pitch + 2 * c, neg ? -pitch : pitch, ny, lim));
+        }
+        __syncthreads();
+    }
+    if (a.coef_z) {
+        const int half = ny / 2; // row pairs of a plane: l, l + half
+        for (int k = threadIdx.x; k < planes * half; k += kAnyThreads) {
+            const int q = int(fdiv(unsigned(k), a.div_hy)), l = k - q * half;
+            const LineCoefT<float> kz = a.coef_z[fdiv(unsigned(p0 + q), a.div_nux)];
+            if (kz.nd < 0) continue;
+            const Lim<float2> lim = to_lim2(kz, kz);
+            float *row = any_s + (q * ny + l) * pitch;
+            check((kz.nd & 1) ? any_uz<true>(row, half * pitch, u, lim) : any_uz<false>(row, half * pitch, u, lim));
+        }
+        __syncthreads();
+    }
+    for (int k = threadIdx.x; k < chunks; k += kAnyThreads) {
+        const int row = int(fdiv(unsigned(k), a.div_u)), col = k - row * u;
+        *reinterpret_cast<float4 *>(dst + e0 + 4ll * k) = *reinterpret_cast<const float4 *>(any_s + row * pitch + 4 * col);
+    }
+    if (bad) atomicOr(a.err, ERR_NAN);
+}
+
 } // namespace
 
 bool plane_tail_supported(int nuy, int nuz, int nux, int dtype)
@@ -218,6 +346,32 @@ cudaError_t launch_plane_tail(void *f, const PlaneTailArgs &a, int nu, int dtype
     case 3: return launch_plane_tail_t(static_cast<__half *>(f), a, blocks, st);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_plane_any(const float *src, float *dst, const PlaneAnyArgs &args, cudaStream_t st)
+{
+    if (args.nplanes <= 0) return cudaSuccess;
+    // plane indices stay below 2^31 (u_z lines do, checked at init)
+    if (args.nux < 1 || args.nuy < 4 || args.nuy % 4 || args.nuz < 4 || args.nuz % 4 || args.plane0 + args.nplanes > 0x7fffffffll)
+        return cudaErrorInvalidValue;
+    PlaneAnyArgs a = args;
+    a.pitch = 4 * ((a.nuz / 4) | 1);
+    const size_t plane = size_t(a.nuy) * a.pitch * sizeof(float);
+    // a pair of lines per thread, within 48 KB where that holds at least a warp's pairs
+    const int most = a.nuy > a.nuz ? a.nuy : a.nuz;
+    a.per_block = 2 * kAnyThreads / most > 1 ? 2 * kAnyThreads / most : 1;
+    while (a.per_block > 1 && a.per_block * plane > 48 * 1024 && (a.per_block - 1) * most >= 64) --a.per_block;
+    if (a.nplanes < a.per_block) a.per_block = int(a.nplanes);
+    a.div_u = make_fastdiv(unsigned(a.nuz / 4));
+    a.div_hz = make_fastdiv(unsigned(a.nuz / 2));
+    a.div_hy = make_fastdiv(unsigned(a.nuy / 2));
+    a.div_nux = make_fastdiv(unsigned(a.nux));
+    const size_t smem = a.per_block * plane;
+    const cudaError_t e = cudaFuncSetAttribute(plane_any_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    const long long blocks = (a.nplanes + a.per_block - 1) / a.per_block;
+    plane_any_kernel<<<unsigned(blocks), kAnyThreads, smem, st>>>(src, dst, a);
+    return cudaGetLastError();
 }
 
 } // namespace vk

@@ -152,21 +152,15 @@ static cudaError_t launch_contig_t(const CUtensorMap &map, const CUtensorMap &dm
     return cudaGetLastError();
 }
 
-cudaError_t launch_contig_f32(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<float> &a, int grid, size_t smem,
-                              cudaStream_t st)
-{
-    return launch_contig_t<float>(map, dmap, a, grid, smem, st);
-}
-
 cudaError_t launch_contig_f64(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<double> &a, int grid, size_t smem,
                               cudaStream_t st)
 {
     return launch_contig_t<double>(map, dmap, a, grid, smem, st);
 }
 
-int occupancy_contig(int dtype, size_t smem)
+int occupancy_contig(size_t smem)
 {
-    const void *k = dtype == 0 ? (const void *)contig_sweep_kernel<double> : (const void *)contig_sweep_kernel<float>;
+    const void *k = (const void *)contig_sweep_kernel<double>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess) return 0;

@@ -370,9 +370,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) rows_sweep_kernel
     __syncwarp();
     if (lane < nrows) {
         const long long row = r0 + lane;
-        // FP32 rows keep the plain division: measured 22.1 ms per u_z sweep on 48^3 x 48^3
-        // against 24.2 with the divider (16-bit rows: 19.5 with it against 21.6)
-        const long long cell = sizeof(T) == 4 ? row / a.rows_per_cell : (long long)fdiv(unsigned(row), a.div_rpc);
+        const long long cell = fdiv(unsigned(row), a.div_rpc);
         const LineCoefT<C> kc = static_cast<const LineCoefT<C> *>(a.cell_coef)[cell];
         if (kc.nd >= 0) {
             const bool neg = kc.nd & 1; // one orientation per spatial cell
@@ -416,7 +414,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 2) rows_sweep_kernel
     }
 }
 
-bool rows_sweep_supported(int L, int dtype) { return dtype >= 0 && dtype <= 3 && (L == 24 || L == 40 || L == 48); }
+bool rows_sweep_supported(int L, int dtype) { return (dtype == 0 || dtype == 2 || dtype == 3) && (L == 24 || L == 40 || L == 48); }
 
 template <int NU, typename T>
 static cudaError_t launch_rows_t(const void *src, void *dst, const RowsArgs &a, cudaStream_t st)
@@ -452,7 +450,6 @@ cudaError_t launch_rows_sweep(const void *src, void *dst, const RowsArgs &args, 
     a.div_rpc = make_fastdiv(unsigned(a.rows_per_cell));
     switch (dtype) {
     case 0: return launch_rows_len<double>(src, dst, a, st);
-    case 1: return launch_rows_len<float>(src, dst, a, st);
     case 2: return launch_rows_len<__nv_bfloat16>(src, dst, a, st);
     case 3: return launch_rows_len<__half>(src, dst, a, st);
     default: return cudaErrorInvalidValue;

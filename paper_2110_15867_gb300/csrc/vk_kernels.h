@@ -234,6 +234,18 @@ struct PlaneTailArgs {
 bool plane_tail_supported(int nuy, int nuz, int nux, int dtype);
 cudaError_t launch_plane_tail(void *f, const PlaneTailArgs &a, int nu, int dtype, cudaStream_t st);
 
+// D_uy and / or D_uz (FP32) over staged (cell, j_x) planes of any size, in place or src -> dst
+// (a null coefficient array leaves its sweep out)
+struct PlaneAnyArgs {
+    int nux, nuy, nuz;
+    long long plane0, nplanes; // planes [plane0, plane0 + nplanes), plane p in spatial cell p / nux
+    const LineCoefT<float> *coef_y, *coef_z;
+    unsigned *err;
+    int pitch, per_block; // from here on set by the launcher
+    FastDivU32 div_u, div_hz, div_hy, div_nux;
+};
+cudaError_t launch_plane_any(const float *src, float *dst, const PlaneAnyArgs &a, cudaStream_t st);
+
 // ----------------------------------------------------------------------------
 // position sweeps with whole lines staged per tile (sweep_tile.cu): FP32, periodic,
 // |nu| < 1, L = 16, 24, 32, 48 or 64 cells, n_inner a multiple of 256.  map views f as
@@ -300,8 +312,6 @@ cudaError_t launch_strided_f32(const CUtensorMap &map, const CUtensorMap &dmap, 
                                size_t smem, cudaStream_t st);
 cudaError_t launch_strided_f64(const CUtensorMap &map, const CUtensorMap &dmap, const StridedArgs<double> &a, int grid,
                                size_t smem, cudaStream_t st);
-cudaError_t launch_contig_f32(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<float> &a, int grid,
-                              size_t smem, cudaStream_t st);
 cudaError_t launch_contig_f64(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<double> &a, int grid,
                               size_t smem, cudaStream_t st);
 // largest resident CTAs per SM for a launcher's kernel with this dynamic smem
@@ -335,14 +345,14 @@ struct RowsArgs {
     unsigned seed; // 16-bit storage: stochastic-rounding stream of this sweep
     FastDivU32 div_rpc; // set by launch_rows_sweep: division by rows_per_cell
 };
-// u_z rows of L = 24, 40 or 48 cells (dtype 0 f64, 1 f32, 2 bf16, 3 f16), in place or src -> dst
+// u_z rows of L = 24, 40 or 48 cells (dtype 0 f64, 2 bf16, 3 f16), in place or src -> dst
 bool rows_sweep_supported(int L, int dtype);
 cudaError_t launch_rows_sweep(const void *src, void *dst, const RowsArgs &a, int dtype, cudaStream_t st);
 bool reg_lines_supported(int L);
 // dtype: 1 f32, 2 bf16, 3 f16
 cudaError_t launch_reg_lines(const void *src, void *dst, const RegLineArgs &a, int dtype, cudaStream_t st);
 int occupancy_strided(int dtype, int periodic, size_t smem);
-int occupancy_contig(int dtype, size_t smem);
+int occupancy_contig(size_t smem);
 cudaError_t launch_line_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<float> &a, int nu,
                               int dtype, int grid, cudaStream_t st, bool fuse_y = false);
 

@@ -327,9 +327,12 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             p.smem = 128 + (size_t)S * tile + bbuf;
             p.spec = spec_rows(tmap_type(c->g.dtype), p.L, rows, es, kConsumers, CU_TENSOR_MAP_SWIZZLE_NONE);
             r = encode_spec(&p.map, p.spec, c->f);
-            const int occ = occupancy_contig(c->g.dtype == VLASOV_F64 ? 0 : 1, p.smem);
-            // u_z rows of 24, 40 or 48 cells never take the transposing kernel
-            if (occ <= 0 && rows_sweep_supported(int(c->g.nuz), c->g.dtype)) {
+            // only FP64 rows other than 24, 40 or 48 cells take the transposing kernel; FP32 grids
+            // whose rows it could not have held stay refused
+            const bool fits = p.smem <= 227 * 1024;
+            const int occ = c->g.dtype == VLASOV_F64 ? occupancy_contig(p.smem) : fits;
+            if (occ <= 0 && (c->g.dtype == VLASOV_F32 ? c->g.nuz == 24 || c->g.nuz == 40 || c->g.nuz == 48
+                                                      : rows_sweep_supported(int(c->g.nuz), c->g.dtype))) {
                 p.grid = 0;
                 continue;
             }
@@ -1018,6 +1021,27 @@ static int run_tile_ux(vlasov_ctx *c, const void *src, void *dst)
     return VLASOV_OK;
 }
 
+// FP32 D_uy (bit 1 of axes) and / or D_uz (bit 2) over staged planes of any size
+static int run_plane_any(vlasov_ctx *c, int axes, const void *src, void *dst)
+{
+    PlaneAnyArgs A{};
+    A.nux = int(c->g.nux); A.nuy = int(c->g.nuy); A.nuz = int(c->g.nuz);
+    A.plane0 = 0;
+    A.nplanes = c->ncell * c->g.nux;
+    if (c->slab_x1 > c->slab_x0) {
+        const long long ppx = A.nplanes / c->g.nx; // planes per x-plane
+        A.plane0 = c->slab_x0 * ppx;
+        A.nplanes = (c->slab_x1 - c->slab_x0) * ppx;
+    }
+    A.coef_y = axes & 2 ? (const LineCoefT<float> *)c->d_coef[1] : nullptr;
+    A.coef_z = axes & 4 ? (const LineCoefT<float> *)c->d_coef[2] : nullptr;
+    A.err = c->d_err;
+    PartTimer t(c, axes == 6 ? VLASOV_T_SWEEP_UYUZ : axes == 2 ? 4 : 5, 1);
+    const cudaError_t e = launch_plane_any((const float *)src, (float *)dst, A, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "plane sweep launch");
+    return VLASOV_OK;
+}
+
 // velocity sweep from src to dst (NULL, NULL: c->f in place) with the per-cell
 // constants already in d_coef[ax - 3]
 static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *dst = nullptr)
@@ -1027,6 +1051,12 @@ static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *
     if (!dst) dst = c->f;
     if (coded(c) && (src != c->f || dst != c->f)) return fail(c, VLASOV_EINVAL, "16-bit storage sweeps in place only");
     if (ax == 3 && c->use_tiles && c->tile_ok[3]) return run_tile_ux(c, src, dst);
+    // u_y alone on planes while its column pairs (n_uz / 2 of a plane) keep at least a quarter of a
+    // block's threads busy (n_u = 16, 96, 32: 0.415 ms on planes, 0.343 streamed; 24^3 cubes 0.352
+    // against 0.416)
+    if (c->g.dtype == VLASOV_F32 &&
+        ((ax == 4 && !use_reg_lines(c, 4) && c->g.nuy <= 2 * c->g.nuz) || (ax == 5 && !c->use_lines)))
+        return run_plane_any(c, ax == 4 ? 2 : 4, src, dst);
     const AxisPlan &p = c->plan[ax];
     const void *coef = c->d_coef[ax - 3];
     SweepMaps m;
@@ -1097,17 +1127,10 @@ static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *
         if ((rc = sweep_maps(c, p.map, p.spec, src, dst, m))) return rc;
         const long long rpc = (long long)c->g.nux * c->g.nuy;
         PartTimer t(c, ax, 1);
-        if (c->g.dtype == VLASOV_F64) {
-            ContigArgs<double> A{};
-            A.L = p.L; A.R = kConsumers; A.stages = p.stages; A.rows = p.n_outer; A.num_tiles = p.num_tiles;
-            A.rows_per_cell = rpc; A.cell_coef = (const LineCoefT<double> *)coef; A.err = c->d_err;
-            e = launch_contig_f64(m.in, m.out, A, p.grid, p.smem, c->stream);
-        } else {
-            ContigArgs<float> A{};
-            A.L = p.L; A.R = kConsumers; A.stages = p.stages; A.rows = p.n_outer; A.num_tiles = p.num_tiles;
-            A.rows_per_cell = rpc; A.cell_coef = (const LineCoefT<float> *)coef; A.err = c->d_err;
-            e = launch_contig_f32(m.in, m.out, A, p.grid, p.smem, c->stream);
-        }
+        ContigArgs<double> A{};
+        A.L = p.L; A.R = kConsumers; A.stages = p.stages; A.rows = p.n_outer; A.num_tiles = p.num_tiles;
+        A.rows_per_cell = rpc; A.cell_coef = (const LineCoefT<double> *)coef; A.err = c->d_err;
+        e = launch_contig_f64(m.in, m.out, A, p.grid, p.smem, c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "velocity sweep launch");
     return VLASOV_OK;
@@ -1265,6 +1288,10 @@ static int run_kick(vlasov_ctx *c)
     if ((rc = run_velocity(c, 3))) return rc;
     if (c->can_fuse_kick && c->fuse_kick >= 1) return run_kick_tail(c);
     if (c->can_plane_tail && c->fuse_kick >= 1) return run_plane_tail(c);
+    if (c->g.dtype == VLASOV_F32 && c->fuse_kick >= 1) {
+        c->sweeps += 2;
+        return run_plane_any(c, 6, c->f, c->f);
+    }
     if ((rc = run_velocity(c, 4))) return rc;
     return run_velocity(c, 5);
 }
@@ -1350,8 +1377,10 @@ static int slab_count(const vlasov_ctx *c, double dt, double a_half)
     const bool fused = c->can_fuse_kick && c->fuse_kick >= 1;
     const bool rows = rows_sweep_supported(int(c->g.nuz), c->g.dtype);
     if (!cube) {
-        if (!rows && (!c->use_lines || c->ltpp <= 0)) return 0;
-        if ((!use_reg_lines(c, 3) && c->splan_tpp[3] <= 0) || (!fused && !use_reg_lines(c, 4) && c->splan_tpp[4] <= 0))
+        const bool f32 = c->g.dtype == VLASOV_F32; // D_uy, D_uz on planes: any x-slab
+        if (f32 ? c->use_lines && c->ltpp <= 0 : !rows && (!c->use_lines || c->ltpp <= 0)) return 0;
+        if ((!use_reg_lines(c, 3) && c->splan_tpp[3] <= 0) ||
+            (!f32 && !fused && !use_reg_lines(c, 4) && c->splan_tpp[4] <= 0))
             return 0;
     }
     for (int ax = 1; ax <= 2; ++ax)

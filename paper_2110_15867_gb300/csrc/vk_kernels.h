@@ -277,6 +277,27 @@ int occupancy_tile_sweep(int L, bool moment);
 cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const TileArgs &a, int grid, cudaStream_t st);
 
 // ----------------------------------------------------------------------------
+// FP32 lines of any length on staged tiles of 128 columns, two lines per thread
+// (sweep_pair32.cu): position sweeps with |nu| < 1 and u_x sweeps; map and dmap view the input
+// and the output as [n_outer][L][n_inner] with box {pair32_columns(), L, 1}
+// ----------------------------------------------------------------------------
+struct Pair32Args {
+    int L;
+    unsigned tiles_inner, tile0, num_tiles; // tiles_inner: tiles of a row (the last may be partial)
+    int slots, groups, lag;                 // of the ring; thread groups; stores left reading
+    long long vstride;                      // column j takes table[(inner / vstride) % nvel]
+    int nvel;
+    unsigned *err;
+    const LineCoefT<float> *cell_coef; // u_x sweep: the Courant numbers per outer index (a cell), else null
+    FastDivU32 div_tiles, div_vstride, div_nvel; // set by the launcher
+    LineCoefT<float> table[kMaxVel];
+};
+int pair32_columns();
+bool pair32_geometry(int L, long long n_inner, long long n_outer, Pair32Args &a);
+int occupancy_pair32(const Pair32Args &a, bool zf);
+cudaError_t launch_pair32(const CUtensorMap &map, const CUtensorMap &dmap, const Pair32Args &a, int grid, cudaStream_t st);
+
+// ----------------------------------------------------------------------------
 // the same on 16-bit storage, two lines per thread (sweep_tile16.cu): position sweeps with
 // |nu| < 1 and u_x sweeps, in place; map views the codes as [n_outer][L][n_inner / 32][32]
 // with box {32, 8, L, 1} (no swizzle), smap the scales as [n_outer][L][n_inner / n_uz] with

@@ -141,6 +141,13 @@ struct vlasov_ctx {
     MapSpec tspec[4];
     int tgrid[4];
     Tile16Args t16[4]; // 16-bit storage: the sizes of the tiles
+    // FP32: staged tiles for lines of any length, where tile_ok has none
+    bool p32_ok[4];
+    Pair32Args p32[4];
+    CUtensorMap pmap[4];
+    MapSpec pspec[4];
+    int pgrid[4];
+    long long pn_outer[4];
     long long ttiles_inner[4], tn_outer[4];
     // the whole kick D_uz D_uy D_ux in one pass (n_ux = n_uy = n_uz = 16 or 32)
     bool can_kick_cube;
@@ -444,7 +451,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         c->ltpp = rpp % rpt == 0 ? rpp / rpt : 0;
     }
     for (int ax = 0; ax < 4; ++ax) {
-        c->tile_ok[ax] = false;
+        c->tile_ok[ax] = c->p32_ok[ax] = false;
         if (!(mask >> ax & 1) || c->g.dtype == VLASOV_F64) continue;
         long long I = 1, O = 1;
         for (int k = ax + 1; k < 6; ++k) I *= d6[k];
@@ -475,6 +482,15 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             if (encode_spec(&c->tsmap[ax], ss, c->scale) != CUDA_SUCCESS) continue;
             occ = occupancy_tile16(c->t16[ax], c->g.dtype, ax == 3);
         } else {
+            if (I >= pair32_columns() && pair32_geometry(L, I, O, c->p32[ax])) {
+                c->pspec[ax] = spec3(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, I, L, O, 4, pair32_columns(), L, 1);
+                const int n = occupancy_pair32(c->p32[ax], ax == 3);
+                if (n > 0 && encode_spec(&c->pmap[ax], c->pspec[ax], c->f) == CUDA_SUCCESS) {
+                    c->p32_ok[ax] = true;
+                    c->pgrid[ax] = n * c->sm_count;
+                    c->pn_outer[ax] = O;
+                }
+            }
             // u_x: zero-flux lines of 48
             if (!(ax == 3 ? tile_sweep_zf_supported(L, I) : tile_sweep_supported(L, I))) continue;
             c->tspec[ax] = spec_tiles(I, L, O);
@@ -491,7 +507,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
     c->can_kick_cube = (mask & 0x38) == 0x38 && kick_cube_supported(c->g.nux, c->g.nuy, c->g.nuz, c->g.dtype) &&
                        c->ncell * c->g.nux * c->g.nuy < (1ll << 31);
     if (c->can_kick_cube) {
-        // f as rows of nu values (u_z lines), a box of half a cube's rows (at most 256)
+        // f as rows of nu values (u_z lines)
         const int nu = c->g.nuz;
         const size_t rowbytes = nu * es;
         const CUtensorMapSwizzle sw = rowbytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
@@ -804,6 +820,24 @@ static bool fused_moment_ok(vlasov_ctx *c, int ax)
     return moment_buffer(c);
 }
 
+// the tiles of the current x-slab (all when none is set) on the FP32 tiles of any length
+static void pair32_tiles(const vlasov_ctx *c, int ax, Pair32Args &A)
+{
+    const long long all = c->pn_outer[ax] * A.tiles_inner;
+    A.tile0 = 0;
+    A.num_tiles = unsigned(all);
+    if (c->slab_x1 > c->slab_x0) {
+        A.tile0 = unsigned(c->slab_x0 * (all / c->g.nx)); // tiles per x-plane (y, z and u_x sweeps)
+        A.num_tiles = unsigned((c->slab_x1 - c->slab_x0) * (all / c->g.nx));
+    }
+    A.err = c->d_err;
+    A.cell_coef = nullptr;
+}
+static int pair32_grid(const vlasov_ctx *c, int ax, const Pair32Args &A)
+{
+    return int(A.num_tiles < unsigned(c->pgrid[ax]) ? A.num_tiles : c->pgrid[ax]);
+}
+
 // position sweep from src to dst (NULL, NULL: c->f in place) with per-velocity-column
 // constants from nu_j = u_j dt / (a^2 dx).  With rho_fused (x sweep only) the sweep
 // also writes the velocity moment of its output to rho_fused when it can, and then
@@ -841,7 +875,11 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         if (e != cudaSuccess) return cuda_fail(c, e, "position sweep launch");
         return VLASOV_OK;
     }
-    if (numax < 1.0 && c->use_tiles && c->tile_ok[ax]) {
+    // FP32: lines of 32 cells march faster two per thread (32^3 x 32^3: 1.31 ms a sweep against
+    // 1.44; lines of 16, 24, 48 and 64 within 7 % either way), unless the x sweep sums the moment
+    const bool pairs_first = c->p32_ok[ax] && (&c->g.nx)[ax] == 32 &&
+                             !(rho_fused && ax == 0 && c->fuse_moment && velocity_cube(c) % 256 == 0);
+    if (numax < 1.0 && c->use_tiles && c->tile_ok[ax] && !pairs_first) {
         // the same on FP32 storage
         TileArgs A{};
         A.L = (&c->g.nx)[ax];
@@ -889,11 +927,24 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         }
         return VLASOV_OK;
     }
+    const bool stream_moment = rho_fused && numax < 1.0 && fused_moment_ok(c, ax); // the streamed x sweep sums it
+    if (numax < 1.0 && c->use_tiles && c->p32_ok[ax] && !stream_moment) {
+        Pair32Args A = c->p32[ax];
+        pair32_tiles(c, ax, A);
+        A.vstride = vstride;
+        A.nvel = nvel;
+        for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
+        if ((rc = sweep_maps(c, c->pmap[ax], c->pspec[ax], src, dst, m))) return rc;
+        PartTimer t(c, ax, 1);
+        const cudaError_t e = launch_pair32(m.in, m.out, A, pair32_grid(c, ax, A), c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "position sweep launch");
+        return VLASOV_OK;
+    }
     if (numax < 1.0) {
         // no whole-cell shift on any line: streamed sweep
         const AxisPlan &sp = c->splan[ax];
         if (!coded(c) && (rc = sweep_maps(c, sp.map, sp.spec, src, dst, m))) return rc;
-        const bool fm = rho_fused && fused_moment_ok(c, ax);
+        const bool fm = stream_moment;
         const long long cube = velocity_cube(c);
         cudaError_t e;
         if (c->g.dtype == VLASOV_F64) {
@@ -1051,6 +1102,19 @@ static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *
     if (!dst) dst = c->f;
     if (coded(c) && (src != c->f || dst != c->f)) return fail(c, VLASOV_EINVAL, "16-bit storage sweeps in place only");
     if (ax == 3 && c->use_tiles && c->tile_ok[3]) return run_tile_ux(c, src, dst);
+    if (ax == 3 && c->use_tiles && c->p32_ok[3] && !use_reg_lines(c, 3)) {
+        Pair32Args A = c->p32[3];
+        pair32_tiles(c, 3, A);
+        A.vstride = 1;
+        A.nvel = 0;
+        A.cell_coef = (const LineCoefT<float> *)c->d_coef[0];
+        SweepMaps m;
+        if (const int rc = sweep_maps(c, c->pmap[3], c->pspec[3], src, dst, m)) return rc;
+        PartTimer t(c, 3, 1);
+        const cudaError_t e = launch_pair32(m.in, m.out, A, pair32_grid(c, 3, A), c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "u_x tile sweep launch");
+        return VLASOV_OK;
+    }
     // u_y alone on planes while its column pairs (n_uz / 2 of a plane) keep at least a quarter of a
     // block's threads busy (n_u = 16, 96, 32: 0.415 ms on planes, 0.343 streamed; 24^3 cubes 0.352
     // against 0.416)

@@ -10,288 +10,24 @@
 // patterns are free of bank conflicts.  One producer thread drives the TMA engine (loads
 // with transaction-count mbarriers, bulk stores); every wait is bounded.  The lines are
 // marched by the same SL-MPP5 code (March) as the separate sweeps, so the result equals
-// D_uz D_uy D_ux run as separate kernels, bit for bit.  FP32 storage: kick_pairs_kernel, two
-// lines per thread.  16-bit storage: kick_cube_kernel, one line per thread in registers.
-//
-// 16-bit storage.  Shared memory holds three half-cube buffers (NU / 2 planes of constant
-// j_x each) that rotate: while a cube sits in two of them, the third receives the first half
-// of the next cube, and once the first half of the current cube has been swept and stored,
-// its buffer receives the second half of the next cube.  Half-cube number j (two per cube,
-// in the order the CTA takes its cubes) always lives in buffer j % 3.
-//   D_ux: thread = line (j_y, j_z), walks j_x across both halves (one value per
-//         row, lanes on consecutive j_z: one row segment per warp access);
-//   D_uy: a warp owns whole planes of a half; lane = column j_z, walks j_y;
-//   D_uz: the same warp, lane = row j_y, reads its row in 16-byte chunks.
-// The rounding points are those of the separate path: D_ux encodes its result with the line
-// scales it decoded with (one stochastic draw per value, the stream of the u_x register-line
-// kernel), D_uy writes FP32 into a per-warp plane buffer, D_uz takes its rows from there,
-// refreshes each row scale to the row's largest value and encodes with the stream of the u_z
-// kernel.
+// D_uz D_uy D_ux run as separate kernels, bit for bit (16-bit storage: the rounding points and
+// random streams of the separate u_x kernel and the fused u_y u_z tail).
 #include "vk_lines.cuh"
 
 namespace vk {
 
 namespace {
 
+// a cube's rows (u_z lines) of T in shared memory
 template <int NU, typename T> struct Cube {
     static constexpr int es = int(sizeof(T));
-    static constexpr bool coded = sizeof(T) == 2;
     static constexpr int rowbytes = NU * es;
     static constexpr int chunks = rowbytes / 16;
     static constexpr int per = 16 / es;
-    static constexpr int half_rows = NU * NU / 2; // u_z lines of half a cube
-    static constexpr unsigned half_bytes = unsigned(half_rows) * rowbytes;
-    static constexpr int box_rows = half_rows < 256 ? half_rows : 256;
-    static constexpr int boxes = half_rows / box_rows;
-    static constexpr unsigned scale_bytes = coded ? unsigned(half_rows) * 4u : 0u;
-    static constexpr int threads = NU * NU / 2; // consumer threads
-    static constexpr int warps = threads / 32;
-    static constexpr int planes_per_warp = 32 / NU; // of each half
-    static constexpr int pitch = NU + 1;            // FP32 plane buffer: floats per row
-    static constexpr int plane_floats = NU * pitch; // NU = 16: the two planes of a warp fall on complementary banks
-    static constexpr unsigned plane_bytes = coded ? unsigned(warps * planes_per_warp * plane_floats) * 4u : 0u;
-    // 16-bit: per warp, the inverse scales of the rows its D_ux lines cross (32)
-    static constexpr unsigned inv_bytes = coded ? unsigned(warps) * 32u * 4u : 0u;
-    static constexpr size_t smem = 128 + 1024 + 3 * size_t(half_bytes) + 3 * size_t(scale_bytes) + plane_bytes + inv_bytes;
     // swizzled byte offset of 16-byte chunk j of row r / of element c of row r
     __device__ static int off(int r, int j) { return r * rowbytes + 16 * (j ^ ((r * rowbytes >> 7) & (chunks - 1))); }
     __device__ static int eoff(int r, int c) { return off(r, c / per) + (c % per) * es; }
 };
-
-// D_ux on line (jy, jz) of the cube in halves h[0], h[1] (scales s[0], s[1]); e0 =
-// index of the line's first element in f (16-bit stochastic-rounding stream).
-// Returns true when the line sum is negative, NaN or infinite.
-template <int NU, typename T, bool NEG>
-__device__ __forceinline__ bool cube_ux(unsigned char *const (&h)[2], const float *const (&s)[2], const float *inv_jx,
-                                        int jy, int jz, const Lim<float> &lim, unsigned long long e0, unsigned seed)
-{
-    using G = Cube<NU, T>;
-    constexpr int HP = NU / 2; // planes per half
-    float v[NU];
-#pragma unroll
-    for (int jx = 0; jx < NU; ++jx) {
-        const int r = (jx % HP) * NU + jy;
-        const T c = *reinterpret_cast<const T *>(h[jx / HP] + G::eoff(r, jz));
-        v[NEG ? NU - 1 - jx : jx] = RegCodec<T>::get(c, s[jx / HP][r]);
-    }
-    const float sum = march_regs<NU, float>(v, lim);
-    unsigned rng = sr_bits(e0, seed);
-#pragma unroll
-    for (int jx = 0; jx < NU; ++jx) { // u_x keeps the scales
-        const int r = (jx % HP) * NU + jy;
-        *reinterpret_cast<T *>(h[jx / HP] + G::eoff(r, jz)) =
-            RegCodec<T>::put(v[NEG ? NU - 1 - jx : jx], inv_jx[jx], lcg_next(rng) >> 16);
-    }
-    return !(sum >= 0.f) || isinf(sum);
-}
-
-// D_uy on column jz of plane jxl (within half buffer hb, scales sb), decoded into the FP32
-// plane buffer pl (row pitch Cube::pitch).
-template <int NU, typename T, bool NEG>
-__device__ __forceinline__ bool cube_uy(unsigned char *hb, const float *sb, float *pl, int jxl, int jz,
-                                        const Lim<float> &lim)
-{
-    using G = Cube<NU, T>;
-    float v[NU];
-#pragma unroll
-    for (int jy = 0; jy < NU; ++jy) {
-        const int r = jxl * NU + jy;
-        const T c = *reinterpret_cast<const T *>(hb + G::eoff(r, jz));
-        v[NEG ? NU - 1 - jy : jy] = RegCodec<T>::get(c, sb[r]);
-    }
-    const float sum = march_regs<NU, float>(v, lim);
-#pragma unroll
-    for (int jy = 0; jy < NU; ++jy) pl[jy * G::pitch + jz] = v[NEG ? NU - 1 - jy : jy];
-    return !(sum >= 0.f) || isinf(sum);
-}
-
-// D_uz on row jy of plane jxl, from the FP32 plane buffer; the row's scale is then refreshed
-// and the row encoded.
-template <int NU, typename T, bool NEG>
-__device__ __forceinline__ bool cube_uz(unsigned char *hb, float *sb, const float *pl, int jxl, int jy,
-                                        const Lim<float> &lim, unsigned long long e0, unsigned seed)
-{
-    using G = Cube<NU, T>;
-    const int r = jxl * NU + jy;
-    float v[NU];
-#pragma unroll
-    for (int jz = 0; jz < NU; ++jz) v[NEG ? NU - 1 - jz : jz] = pl[jy * G::pitch + jz];
-    const float sum = march_regs<NU, float>(v, lim);
-    float m = 0.f;
-#pragma unroll
-    for (int l = 0; l < NU; ++l) m = fmaxf(m, v[l]);
-    m = coded_scale<T>(m);
-    sb[r] = m;
-    const float inv = inv_scale(m);
-    unsigned rng = sr_bits(e0, seed);
-#pragma unroll
-    for (int j = 0; j < G::chunks; ++j) {
-        float a[G::per];
-#pragma unroll
-        for (int q = 0; q < G::per; ++q) a[q] = v[NEG ? NU - 1 - (G::per * j + q) : G::per * j + q];
-        Chunk<T>::put(hb + G::off(r, j), inv, a, rng);
-    }
-    return !(sum >= 0.f) || isinf(sum);
-}
-
-template <int NU, typename T>
-__global__ void __launch_bounds__(Cube<NU, T>::threads + kProducer, NU == 32 ? 1 : 4)
-    kick_cube_kernel(const __grid_constant__ CUtensorMap fmap, const __grid_constant__ CUtensorMap smap,
-                     const __grid_constant__ KickArgs a)
-{
-    using G = Cube<NU, T>;
-    constexpr int NT = G::threads;
-    constexpr unsigned tx_bytes = G::half_bytes + G::scale_bytes;
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem); // 3: a half-cube buffer holds its data
-    uint64_t *done = full + 3;                           // 3: the consumers are done with a half
-    uint64_t *uxd = done + 3;                            // D_ux of the current cube is complete
-    unsigned char *bufs = smem + 128 + ((1024u - ((smem_u32(smem) + 128u) & 1023u)) & 1023u);
-    auto hbuf = [&](unsigned j) { return bufs + size_t(G::half_bytes) * (j % 3); };
-    auto sbuf = [&](unsigned j) {
-        return reinterpret_cast<float *>(bufs + 3 * size_t(G::half_bytes) + size_t(G::scale_bytes) * (j % 3));
-    };
-    float *planes = reinterpret_cast<float *>(bufs + 3 * size_t(G::half_bytes) + 3 * size_t(G::scale_bytes));
-    float *invs = reinterpret_cast<float *>(bufs + 3 * size_t(G::half_bytes) + 3 * size_t(G::scale_bytes) +
-                                            G::plane_bytes); // 16-bit: 32 per warp
-
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < 3; ++q) {
-            mbar_init(&full[q], 1);
-            mbar_init(&done[q], NT);
-        }
-        mbar_init(uxd, NT);
-        fence_barrier_init();
-    }
-    __syncthreads();
-
-    const long long Gd = gridDim.x, b = blockIdx.x;
-    const unsigned n_my = unsigned(a.ncells > b ? (a.ncells - b + Gd - 1) / Gd : 0);
-    const unsigned halves = 2 * n_my;
-    auto first_row = [&](unsigned j) {
-        const long long cube = a.cell0 + b + (long long)(j / 2) * Gd;
-        return cube * (NU * NU) + (j % 2) * G::half_rows;
-    };
-
-    if (threadIdx.x >= NT) {
-        // producer: one thread drives the TMA engine
-        if (threadIdx.x != NT) return;
-        auto load = [&](unsigned j) {
-            uint64_t *bar = &full[j % 3];
-            mbar_arrive_expect_tx(bar, tx_bytes);
-            const long long r0 = first_row(j);
-            for (int q = 0; q < G::boxes; ++q)
-                tma_load_2d(hbuf(j) + q * G::box_rows * G::rowbytes, &fmap, bar, 0, int(r0 + q * G::box_rows));
-            tma_load_2d(sbuf(j), &smap, bar, 0, int(r0 / NU));
-        };
-        unsigned loaded = 0;
-        for (; loaded < 3 && loaded < halves; ++loaded) load(loaded);
-        bool ok = true;
-        for (unsigned j = 0; j < halves; ++j) {
-            if (!mbar_wait_bounded(&done[j % 3], (j / 3) & 1u)) {
-                ok = false;
-                break;
-            }
-            const long long r0 = first_row(j);
-            for (int q = 0; q < G::boxes; ++q)
-                tma_store_2d(&fmap, hbuf(j) + q * G::box_rows * G::rowbytes, 0, int(r0 + q * G::box_rows));
-            tma_store_2d(&smap, sbuf(j), 0, int(r0 / NU));
-            bulk_commit();
-            if (loaded < halves) {
-                bulk_wait_read_all(); // the buffer of half j is free once the store has read it
-                load(loaded++);
-            }
-        }
-        bulk_wait_all();
-        if (!ok) {
-            atomicOr(a.err, ERR_TIMEOUT);
-            // let the loads in flight (the last three at most) land before the CTA exits
-            for (unsigned j = loaded > 3 ? loaded - 3 : 0; j < loaded; ++j) mbar_wait_bounded(&full[j % 3], (j / 3) & 1u);
-        }
-        return;
-    }
-
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    float *pl = planes + (w * G::planes_per_warp + lane / NU) * G::plane_floats; // 16-bit: this lane's plane
-    bool bad = false;
-    for (unsigned k = 0; k < n_my; ++k) {
-        const unsigned j0 = 2 * k, j1 = 2 * k + 1;
-        const bool got = mbar_wait_bounded(&full[j0 % 3], (j0 / 3) & 1u) && mbar_wait_bounded(&full[j1 % 3], (j1 / 3) & 1u);
-        if (!__all_sync(0xffffffffu, got)) {
-            atomicOr(a.err, ERR_TIMEOUT);
-            return;
-        }
-        const long long cube = a.cell0 + b + (long long)k * Gd;
-        unsigned char *const h[2] = {hbuf(j0), hbuf(j1)};
-        float *const s[2] = {sbuf(j0), sbuf(j1)};
-        const unsigned long long e_cube = (unsigned long long)cube * (NU * NU * NU);
-        // one Courant number per cell and axis: every branch below is CTA-uniform
-        const LineCoefT<float> kx = a.coef_x[cube];
-        if (kx.nd >= 0) {
-            const Lim<float> lim = to_lim(kx);
-            const float *const sc[2] = {s[0], s[1]};
-#pragma unroll 1
-            for (int q = 0; q < 2; ++q) {
-                const int line = q * NT + t, jy = line / NU, jz = line % NU;
-                const unsigned long long e0 = e_cube + (unsigned long long)line;
-                // 16-bit: the warp's lines cross NU rows per j_y (32 / NU values of j_y): each
-                // lane forms the inverse scale of one of them once, for the whole warp
-                float *wi = invs + w * 32;
-                __syncwarp();
-                const int jy_l = (q * NT + w * 32) / NU + lane / NU, jx = lane % NU;
-                wi[lane] = inv_scale(sc[jx / (NU / 2)][(jx % (NU / 2)) * NU + jy_l]);
-                __syncwarp();
-                const float *inv_jx = wi + (lane / NU) * NU;
-                bad |= (kx.nd & 1) ? cube_ux<NU, T, true>(h, sc, inv_jx, jy, jz, lim, e0, a.seed_x)
-                                   : cube_ux<NU, T, false>(h, sc, inv_jx, jy, jz, lim, e0, a.seed_x);
-            }
-        }
-        // every D_ux line crosses every plane: all of them finish before D_uy
-        mbar_arrive(uxd);
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(uxd, k & 1u))) {
-            atomicOr(a.err, ERR_TIMEOUT);
-            return;
-        }
-        const LineCoefT<float> ky = a.coef_y[cube], kz = a.coef_z[cube];
-        const int jxl = w * G::planes_per_warp + lane / NU, c = lane % NU;
-#pragma unroll 1
-        for (int hh = 0; hh < 2; ++hh) {
-            unsigned char *const hb = hh ? h[1] : h[0]; // selects, not a dynamically indexed array
-            float *const sb = hh ? s[1] : s[0];
-            if (ky.nd >= 0) {
-                const Lim<float> lim = to_lim(ky);
-                bad |= (ky.nd & 1) ? cube_uy<NU, T, true>(hb, sb, pl, jxl, c, lim)
-                                   : cube_uy<NU, T, false>(hb, sb, pl, jxl, c, lim);
-            } else {
-                // no D_uy: the plane buffer takes the decoded values as they are
-#pragma unroll 4
-                for (int jy = 0; jy < NU; ++jy) {
-                    const int r = jxl * NU + jy;
-                    pl[jy * G::pitch + c] = RegCodec<T>::get(*reinterpret_cast<const T *>(hb + G::eoff(r, c)), sb[r]);
-                }
-            }
-            __syncwarp();
-            const unsigned long long e0 = e_cube + (unsigned long long)((hh * (NU / 2) + jxl) * NU + c) * NU;
-            if (kz.nd >= 0) {
-                const Lim<float> lim = to_lim(kz);
-                bad |= (kz.nd & 1) ? cube_uz<NU, T, true>(hb, sb, pl, jxl, c, lim, e0, a.seed_z)
-                                   : cube_uz<NU, T, false>(hb, sb, pl, jxl, c, lim, e0, a.seed_z);
-            } else if (ky.nd >= 0) {
-                // D_uy changed the plane but D_uz does not run: encode it with the row's scale
-                // refreshed as the u_z sweep would not; keep the stored scale, round to nearest
-                const int r = jxl * NU + c;
-                const float inv = inv_scale(sb[r]);
-#pragma unroll 4
-                for (int jz = 0; jz < NU; ++jz)
-                    *reinterpret_cast<T *>(hb + G::eoff(r, jz)) = from_c<T>(pl[c * G::pitch + jz] * inv);
-            }
-            __syncwarp();
-            fence_proxy_async();
-            mbar_arrive(&done[(2 * k + hh) % 3]);
-        }
-    }
-    if (bad) atomicOr(a.err, ERR_NAN);
-}
 
 // ----------------------------------------------------------------------------
 // FP32 storage: two lines per thread as packed pairs, lines walked in shared memory
@@ -583,24 +319,341 @@ __global__ void __launch_bounds__(PairCube<NU>::threads + kProducer, NU == 32 ? 
     if (bad) atomicOr(a.err, ERR_NAN);
 }
 
-template <int NU, typename T> const void *kick_kernel() { return (const void *)kick_cube_kernel<NU, T>; }
+// ----------------------------------------------------------------------------
+// 16-bit storage: the same marches on a cube decoded into FP32
+// ----------------------------------------------------------------------------
+// The pieces of a cube (codes and line scales) pass through a ring of four: D_ux decodes them
+// as it walks, encodes each result with the line scale it keeps (one stochastic draw per
+// value, the stream of the u_x register-line kernel) and writes what that code decodes to
+// into a cube of FP32, on which D_uy and D_uz run as for FP32 storage.  So a piece is free
+// as soon as D_ux is through, and the next cube loads while D_uy and D_uz run.  Each warp
+// then takes its 64 rows into registers, refreshes their scales to the largest value,
+// encodes them with the streams of the u_z kernel, densely into the front half of the same
+// shared memory, and stores them itself; the FP32 cube may be written again once every
+// warp's store has read its part (barrier `freed`).
+// 32^3 x 32^3 BF16, per kick: 4.48 ms with one line per thread in registers (its unrolled
+// bodies at the edge of the instruction cache), 3.91 here (61 instructions per face pair, issue 63 %
+// busy); 32^3 x 16^3 FP16 0.82 -> 0.59 ms.
+template <int NU, typename T> struct PairCube16 {
+    using G = Cube<NU, T>;
+    using F = Cube<NU, float>;
+    static constexpr int planes = NU / 4;                  // of a piece
+    static constexpr int rows = planes * NU;               // u_z lines of a piece
+    static constexpr unsigned code_bytes = unsigned(rows) * G::rowbytes;
+    static constexpr unsigned bytes = code_bytes + rows * 4u; // codes, then scales
+    static constexpr int slots = 4;
+    static constexpr int threads = NU * NU / 2; // one per pair of lines
+    static constexpr int warps = threads / 32;
+    static constexpr int wrows = 64;            // rows a warp owns for D_uy, D_uz (a TMA box)
+    static constexpr int wplanes = wrows / NU;
+    static constexpr int warp_js = 64 / NU;     // j_y of a warp's D_ux lines
+    static constexpr size_t cube_bytes = size_t(NU) * NU * F::rowbytes;
+    // barriers (128 B), the coefficients of three cubes, alignment, the FP32 cube, the ring, (scale,
+    // inverse scale) of the rows each warp's D_ux lines cross
+    static constexpr int head = 128 + ((9 * int(sizeof(LineCoefT<float>)) + 127) & ~127);
+    static constexpr size_t smem = head + 1024 + cube_bytes + size_t(slots) * bytes + size_t(warps) * 64 * sizeof(float2);
+};
+
+// The rounding stream of a line draws for its cells in memory order (j_x = 0 first), as the
+// u_x register-line kernel does; a line walked from its far end takes the same draws
+// backward: the generator x -> a x + c run in reverse, from the state after NU + 1 steps.
+constexpr unsigned kLcgA = 1664525u, kLcgC = 1013904223u;
+constexpr unsigned kLcgInv = 4276115653u; // a kLcgInv = 1 mod 2^32
+static_assert(kLcgA * kLcgInv == 1u, "inverse of the generator's multiplier");
+template <bool NEG> __device__ __forceinline__ unsigned draw16(unsigned &x)
+{
+    x = NEG ? x * kLcgInv - kLcgC * kLcgInv : x * kLcgA + kLcgC;
+    return x >> 16;
+}
+constexpr unsigned lcg_pow(int n) { return n ? kLcgA * lcg_pow(n - 1) : 1u; }
+constexpr unsigned lcg_add(int n) { return n ? kLcgA * lcg_add(n - 1) + kLcgC : 0u; }
+template <int NU, bool NEG> __device__ __forceinline__ unsigned draw_start(unsigned seed)
+{
+    constexpr unsigned A = lcg_pow(NU + 1), C = lcg_add(NU + 1);
+    return NEG ? seed * A + C : seed;
+}
+
+// value pair -> what the codes it is stochastically rounded to (bx, by: 16 random bits) decode to
+__device__ __forceinline__ float2 recode(float2 v, float2 s, unsigned bx, unsigned by, __nv_bfloat16)
+{
+    const float2 c = vmul(v, make_float2(s.y, s.y));
+    const unsigned x = (__float_as_uint(c.x) + bx) & 0xffff0000u;
+    const unsigned y = (__float_as_uint(c.y) + by) & 0xffff0000u;
+    return vmul(make_float2(__uint_as_float(x), __uint_as_float(y)), make_float2(s.x, s.x));
+}
+__device__ __forceinline__ float2 recode(float2 v, float2 s, unsigned bx, unsigned by, __half)
+{
+    const float2 c = vmul(v, make_float2(s.y, s.y));
+    const __half x = RegCodec<__half>::put(c.x, 1.f, bx), y = RegCodec<__half>::put(c.y, 1.f, by);
+    return vmul(make_float2(__half2float(x), __half2float(y)), make_float2(s.x, s.x));
+}
+__device__ __forceinline__ float2 decode2(unsigned u, float s, __nv_bfloat16)
+{
+    return vmul(make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)), make_float2(s, s));
+}
+__device__ __forceinline__ float2 decode2(unsigned u, float s, __half)
+{
+    return vmul(__half22float2(*reinterpret_cast<const __half2 *>(&u)), make_float2(s, s));
+}
+
+// D_ux on one pair of columns: piece(q) is the piece in march order (waits for it and leaves
+// its scales in ws; false: a wait ran out); codes at byte `co` of every plane of it, the FP32
+// cube's cells at fp + plane FST (plane 0 .. NU - 1 of the cube); ws[n js + jl]: (scale, inverse)
+// of the n-th plane in march order.  writable(): the FP32 cube may be written.
+template <int NU, typename T, bool NEG, typename Piece, typename Writable>
+__device__ __forceinline__ bool pair16_ux(Piece piece, Writable writable, int co, unsigned char *fp, const float2 *ws, int jl,
+                                          const Lim<float2> &lim, unsigned rx, unsigned ry, bool &ok)
+{
+    using P = PairCube16<NU, T>;
+    constexpr int NP = P::planes, CST = NU * P::G::rowbytes, FST = NU * P::F::rowbytes, JS = P::warp_js;
+    auto code = [&](const unsigned char *p, int i) { // plane i of the piece in march order
+        return *reinterpret_cast<const unsigned *>(p + (NEG ? NP - 1 - i : i) * CST);
+    };
+    // cell n of the line in march order: its scales, and where its value goes
+    if (NEG) fp += (NU - 1) * FST;
+    const float2 *s = ws + jl;
+    auto out = [&](int n, float2 v) {
+        *reinterpret_cast<float2 *>(fp + (NEG ? -n : n) * FST) =
+            recode(v, s[n * JS], draw16<NEG>(rx), draw16<NEG>(ry), T());
+    };
+    rx = draw_start<NU, NEG>(rx);
+    ry = draw_start<NU, NEG>(ry);
+    const unsigned char *cur = piece(0, ok) + co;
+    if (!ok || !(ok = writable())) return false;
+    March<float2> m(lim);
+    m.start_zero(decode2(code(cur, 0), s[0].x, T()), decode2(code(cur, 1), s[JS].x, T()));
+#pragma unroll
+    for (int i = 2; i < NP; ++i) out(i - 2, m.face(decode2(code(cur, i), s[i * JS].x, T())));
+#pragma unroll 1
+    for (int q = 1; q < 4; ++q) {
+        cur = piece(q, ok) + co;
+        if (!ok) return false;
+        fp += (NEG ? -NP : NP) * FST;
+        s += NP * JS;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) out(i - 2, m.face(decode2(code(cur, i), s[i * JS].x, T())));
+    }
+    out(NP - 2, m.face(make_float2(0.f, 0.f)));
+    out(NP - 1, m.last());
+    return !(m.sum.x >= 0.f) || !(m.sum.y >= 0.f) || isinf(m.sum.x) || isinf(m.sum.y);
+}
+
+template <int NU, typename T>
+__global__ void __launch_bounds__(PairCube16<NU, T>::threads + kProducer, NU == 32 ? 1 : 4)
+    kick_pairs16_kernel(const __grid_constant__ CUtensorMap fmap, const __grid_constant__ CUtensorMap smap,
+                        const __grid_constant__ KickArgs a)
+{
+    using P = PairCube16<NU, T>;
+    using G = typename P::G;
+    using F = typename P::F;
+    constexpr int NT = P::threads, S = P::slots, NP = P::planes, JS = P::warp_js;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem); // S: the slot holds its piece
+    uint64_t *uxd = full + S;                            // D_ux of the current cube is complete
+    uint64_t *freed = uxd + 1;                           // every warp's part of the FP32 cube is stored
+    LineCoefT<float> *coefs = reinterpret_cast<LineCoefT<float> *>(smem + 128);
+    unsigned char *cubef = smem + P::head + ((1024u - ((smem_u32(smem) + unsigned(P::head)) & 1023u)) & 1023u);
+    unsigned char *ring = cubef + P::cube_bytes;
+    float2 *scales = reinterpret_cast<float2 *>(ring + size_t(S) * P::bytes);
+    auto slot = [&](unsigned j) { return ring + size_t(P::bytes) * (j % S); };
+
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < S; ++q) mbar_init(&full[q], 1);
+        mbar_init(uxd, NT);
+        mbar_init(freed, P::warps);
+        fence_barrier_init();
+    }
+    __syncthreads();
+
+    const long long Gd = gridDim.x, b = blockIdx.x;
+    const unsigned n_my = unsigned(a.ncells > b ? (a.ncells - b + Gd - 1) / Gd : 0);
+
+    if (threadIdx.x >= NT) {
+        // producer: one thread loads the pieces of cube k + 1 once D_ux of cube k is complete
+        if (threadIdx.x != NT) return;
+        unsigned k = 0;
+        bool ok = true;
+        for (; k < n_my; ++k) {
+            if (k > 0 && !mbar_wait_bounded(uxd, (k - 1) & 1u)) {
+                ok = false;
+                break;
+            }
+            const long long cube = a.cell0 + b + (long long)k * Gd;
+            // (three sets: warps still on cube k - 1 read theirs, and none can be on k - 2)
+            LineCoefT<float> *co = coefs + 3 * (k % 3);
+            const LineCoefT<float> cx = a.coef_x[cube], cy = a.coef_y[cube], cz = a.coef_z[cube];
+            co[0] = cx;
+            co[1] = cy;
+            co[2] = cz;
+            const bool neg = cx.nd >= 0 && (cx.nd & 1);
+            fence_proxy_async(); // the consumers' reads of the slots come before the loads
+            for (int m = 0; m < 4; ++m) {
+                const int q = neg ? 3 - m : m;
+                uint64_t *bar = &full[m];
+                unsigned char *dst = slot(m);
+                mbar_arrive_expect_tx(bar, P::bytes);
+                for (int x = 0; x < P::rows / P::wrows; ++x) {
+                    const int plane = int(cube * NU) + q * NP + x * P::wplanes;
+                    tma_load_2d(dst + x * P::wrows * G::rowbytes, &fmap, bar, 0, plane * NU);
+                    tma_load_2d(dst + P::code_bytes + x * P::wrows * 4, &smap, bar, 0, plane);
+                }
+            }
+        }
+        if (!ok) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            if (k > 0) // let the loads in flight land before the CTA exits
+                for (int m = 0; m < 4; ++m) mbar_wait_bounded(&full[m], (k - 1) & 1u);
+        }
+        return;
+    }
+
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    // D_ux: the thread's columns; D_uy, D_uz: its plane (within the warp's), column pair, row
+    const int ujy = t / (NU / 2), ujz = 2 * (t % (NU / 2));
+    const int co_off = G::eoff(ujy, ujz);
+    float2 *ws = scales + w * 64;
+    const int wp = lane / (NU / 2), lp = lane % (NU / 2);
+    unsigned char *mine = cubef + size_t(w) * P::wrows * F::rowbytes; // the warp's rows
+    unsigned char *pl = mine + wp * NU * F::rowbytes;
+    bool bad = false, ok = true;
+    for (unsigned k = 0; k < n_my; ++k) {
+        const long long cube = a.cell0 + b + (long long)k * Gd;
+        const unsigned long long e_cube = (unsigned long long)cube * (NU * NU * NU);
+        const LineCoefT<float> *co = coefs + 3 * (k % 3);
+        bool xneg = false;
+        auto piece = [&](int m, bool &good) -> unsigned char * { // piece m in march order, its scales into ws
+            good = __all_sync(0xffffffffu, mbar_wait_bounded(&full[m], k & 1u));
+            if (!good) return nullptr;
+            if (m == 0) xneg = co[0].nd >= 0 && (co[0].nd & 1);
+            if (lane < NP * JS) {
+                const int i = lane / JS, jl = lane % JS;
+                const float s = reinterpret_cast<const float *>(slot(m) + P::code_bytes)[(xneg ? NP - 1 - i : i) * NU + w * JS + jl];
+                ws[(m * NP + i) * JS + jl] = make_float2(s, inv_scale(s));
+            }
+            __syncwarp();
+            return slot(m);
+        };
+        auto writable = [&]() { return k == 0 || __all_sync(0xffffffffu, mbar_wait_bounded(freed, (k - 1) & 1u)); };
+        unsigned char *first = piece(0, ok);
+        if (ok) {
+            // one Courant number per cell and axis: every branch below is CTA-uniform
+            const LineCoefT<float> kx = co[0];
+            auto again = [&](int m, bool &good) { // piece 0 is here
+                good = true;
+                return m == 0 ? first : piece(m, good);
+            };
+            if (kx.nd >= 0) {
+                const Lim<float2> lim = to_lim2(kx, kx);
+                const unsigned long long e0 = e_cube + (unsigned long long)(ujy * NU + ujz);
+                const unsigned rx = sr_bits(e0, a.seed_x), ry = sr_bits(e0 + 1, a.seed_x);
+                unsigned char *fp = cubef + F::eoff(ujy, ujz);
+                bad |= xneg ? pair16_ux<NU, T, true>(again, writable, co_off, fp, ws, ujy % JS, lim, rx, ry, ok)
+                            : pair16_ux<NU, T, false>(again, writable, co_off, fp, ws, ujy % JS, lim, rx, ry, ok);
+            } else if ((ok = writable())) {
+                // no D_ux: the FP32 cube takes the decoded values as they are
+                for (int m = 0; m < 4 && ok; ++m) {
+                    const unsigned char *p = again(m, ok);
+                    if (!ok) break;
+#pragma unroll 1
+                    for (int i = 0; i < NP; ++i)
+                        *reinterpret_cast<float2 *>(cubef + F::eoff((m * NP + i) * NU + ujy, ujz)) =
+                            decode2(*reinterpret_cast<const unsigned *>(p + i * NU * G::rowbytes + co_off),
+                                    ws[(m * NP + i) * JS + ujy % JS].x, T());
+                }
+            }
+        }
+        if (!ok) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            break;
+        }
+        // every D_ux line crosses every plane: all of them finish before D_uy; the pieces are read
+        mbar_arrive(uxd);
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(uxd, k & 1u))) {
+            atomicOr(a.err, ERR_TIMEOUT);
+            break;
+        }
+        const bool ran_x = co[0].nd >= 0;
+        const LineCoefT<float> ky = co[1], kz = co[2];
+        if (ky.nd >= 0) {
+            const Lim<float2> lim = to_lim2(ky, ky);
+            bad |= (ky.nd & 1) ? pair_uy<NU, true>(pl, 2 * lp, lim) : pair_uy<NU, false>(pl, 2 * lp, lim);
+        }
+        __syncwarp();
+        if (kz.nd >= 0) {
+            const Lim<float2> lim = to_lim2(kz, kz);
+            bad |= (kz.nd & 1) ? pair_uz<NU, true>(pl, lp, lim) : pair_uz<NU, false>(pl, lp, lim);
+        }
+        __syncwarp();
+        if (ran_x || ky.nd >= 0 || kz.nd >= 0) { // (else every code stays as it is)
+            // rows lane and lane + 32 of the warp's 64, into registers, then encoded over them
+            float v[2][NU];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int j = 0; j < F::chunks; ++j) {
+                    const float4 x = *reinterpret_cast<const float4 *>(mine + F::off(lane + 32 * h, j));
+                    v[h][4 * j] = x.x; v[h][4 * j + 1] = x.y; v[h][4 * j + 2] = x.z; v[h][4 * j + 3] = x.w;
+                }
+            __syncwarp();
+            float *sdst = reinterpret_cast<float *>(mine + P::wrows * G::rowbytes);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = lane + 32 * h;
+                const long long row = cube * (NU * NU) + w * P::wrows + r;
+                if (kz.nd >= 0) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int l = 0; l < NU; l += 2) s = mx3(s, v[h][l], v[h][l + 1]);
+                    s = coded_scale<T>(s);
+                    sdst[r] = s;
+                    const float inv = inv_scale(s);
+                    unsigned rng = sr_bits((unsigned long long)row * NU, a.seed_z);
+#pragma unroll
+                    for (int j = 0; j < G::chunks; ++j) {
+                        float e[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) e[q] = v[h][8 * j + q];
+                        Chunk<T>::put(mine + G::off(r, j), inv, e, rng);
+                    }
+                } else {
+                    // D_uz did not run: its rows keep their scales and round to nearest (codes
+                    // that D_ux left come back as they were)
+                    const float s = a.scale[row], inv = inv_scale(s);
+                    sdst[r] = s;
+#pragma unroll
+                    for (int l = 0; l < NU; ++l) *reinterpret_cast<T *>(mine + G::eoff(r, l)) = from_c<T>(v[h][l] * inv);
+                }
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+                const int plane = int(cube * NU) + w * P::wplanes;
+                tma_store_2d(&fmap, mine, 0, plane * NU);
+                tma_store_2d(&smap, sdst, 0, plane);
+                bulk_commit();
+                bulk_wait_read_all();
+            }
+            __syncwarp();
+        }
+        if (lane == 0) mbar_arrive(freed);
+    }
+    if (lane == 0) bulk_wait_all();
+    if (bad) atomicOr(a.err, ERR_NAN);
+}
 
 const void *kick_kernel_for(int nu, int dtype)
 {
     switch (dtype) {
     case 1: return nu == 32 ? (const void *)kick_pairs_kernel<32> : (const void *)kick_pairs_kernel<16>;
-    case 2: return nu == 32 ? kick_kernel<32, __nv_bfloat16>() : kick_kernel<16, __nv_bfloat16>();
-    case 3: return nu == 32 ? kick_kernel<32, __half>() : kick_kernel<16, __half>();
+    case 2: return nu == 32 ? (const void *)kick_pairs16_kernel<32, __nv_bfloat16> : (const void *)kick_pairs16_kernel<16, __nv_bfloat16>;
+    case 3: return nu == 32 ? (const void *)kick_pairs16_kernel<32, __half> : (const void *)kick_pairs16_kernel<16, __half>;
     default: return nullptr;
     }
 }
 
-template <int NU> size_t smem_for(int dtype)
-{
-    return dtype == 1 ? PairCube<NU>::smem : Cube<NU, __nv_bfloat16>::smem;
-}
+template <int NU> size_t smem_for(int dtype) { return dtype == 1 ? PairCube<NU>::smem : PairCube16<NU, __nv_bfloat16>::smem; }
 
-template <int NU> int threads_for() { return Cube<NU, float>::threads + kProducer; }
+template <int NU> int threads_for() { return PairCube<NU>::threads + kProducer; }
 
 } // namespace
 
@@ -609,11 +662,7 @@ bool kick_cube_supported(int nux, int nuy, int nuz, int dtype)
     return nux == nuy && nuy == nuz && (nuz == 16 || nuz == 32) && dtype >= 1 && dtype <= 3;
 }
 
-int kick_cube_box_rows(int nu, int dtype)
-{
-    if (dtype == 1) return nu * nu / 4; // a piece
-    return nu * nu / 2 < 256 ? nu * nu / 2 : 256;
-}
+int kick_cube_box_rows(int nu, int dtype) { return dtype == 1 ? nu * nu / 4 : 64; } // FP32: a piece; 16-bit: a warp's rows
 
 size_t kick_cube_smem(int nu, int dtype) { return nu == 32 ? smem_for<32>(dtype) : smem_for<16>(dtype); }
 

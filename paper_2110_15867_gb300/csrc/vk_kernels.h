@@ -210,6 +210,7 @@ struct KickArgs {
     const LineCoefT<float> *coef_x, *coef_y, *coef_z;
     unsigned *err;
     unsigned seed_x, seed_z; // 16-bit: stochastic-rounding streams of the D_ux and D_uz encodes
+    const float *scale;      // 16-bit: the line scales (read where D_uz does not run)
 };
 bool kick_cube_supported(int nux, int nuy, int nuz, int dtype); // dtype 1 f32, 2 bf16, 3 f16
 int kick_cube_box_rows(int nu, int dtype);

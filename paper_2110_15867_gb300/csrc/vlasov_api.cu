@@ -517,8 +517,9 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         CUresult r = encode_spec(&c->kmap, ks, c->f);
         if (r != CUDA_SUCCESS) return fail(c, VLASOV_ECUDA, "kick tensor map failed (%d)", int(r));
         if (coded) {
-            // the scales as [ncell nu][nu] (one row per j_x plane), half a cube per box
-            const MapSpec ss = spec_rows(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, nu, c->ncell * nu, 4, nu / 2,
+            // the scales as [ncell nu][nu] (one row per j_x plane), those of a warp's rows per box
+            const MapSpec ss = spec_rows(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, nu, c->ncell * nu, 4,
+                                         kick_cube_box_rows(nu, c->g.dtype) / nu,
                                          CU_TENSOR_MAP_SWIZZLE_NONE);
             r = encode_spec(&c->ksmap, ss, c->scale);
             if (r != CUDA_SUCCESS) return fail(c, VLASOV_ECUDA, "kick scale tensor map failed (%d)", int(r));
@@ -1329,6 +1330,7 @@ static int run_kick_cube(vlasov_ctx *c)
     A.coef_y = (const LineCoefT<float> *)c->d_coef[1];
     A.coef_z = (const LineCoefT<float> *)c->d_coef[2];
     A.err = c->d_err;
+    A.scale = c->scale;
     A.cell0 = 0;
     A.ncells = c->ncell;
     if (c->slab_x1 > c->slab_x0) {

@@ -299,7 +299,9 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             int W, P;
             if (I >= kConsumers) { W = kConsumers; P = 1; }
             else { W = int(I); P = kConsumers / W; if (P > O) P = int(O); }
-            while ((size_t)W * p.L * P * es > 96 * 1024 && W * P > 32) {
+            // tiles and rings small enough for three CTAs per SM: a CTA's 8 warps march one tile
+            // and wait for each other, so one CTA (4 stages of 32 KB) left an SM's latency bare
+            while ((size_t)W * p.L * P * es > 36 * 1024 && W * P > 32) {
                 if (P > 1) P = (P + 1) / 2;
                 else W /= 2;
             }
@@ -309,7 +311,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             p.num_tiles = (long long)p.tiles_inner * ((O + P - 1) / P);
             const size_t tile = ((size_t)W * p.L * P * es + 127) & ~size_t(127);
             const size_t tab = ax < 3 ? ((sizeof(LineCoefT<double>) * kMaxVel + 127) & ~size_t(127)) : 0;
-            int S = int((kSmemBudget - 128 - tab) / tile);
+            int S = int((76 * 1024 - 128 - tab) / tile);
             S = S < 2 ? 2 : (S > 4 ? 4 : S);
             p.stages = S;
             p.smem = 128 + tab + (size_t)S * tile;

@@ -86,12 +86,12 @@ __device__ __forceinline__ float march_shift(float *p, long step, int L, const L
 // rows, still to be read, wait in `held`, and the last three cells, overwritten before the
 // first ones need them, in registers.  The values are march_shift's, face by face.  With tiles
 // small enough for three CTAs per SM: 32 x 24 x 32 x 16 x 16 x 32 cells, x, y, z 0.600, 0.430, 0.643 ->
-// 0.410, 0.436, 0.458 ms (DRAM alone 0.238 ms each).
+// 0.39 ms each (DRAM alone 0.238).
 constexpr int kStash = 8;
-__device__ __forceinline__ float march_shift_down(float *p, long step, int L, int N, const LineCoefT<float> &k)
+__device__ __forceinline__ float march_shift_down(float *p, int step, int L, int N, const LineCoefT<float> &k)
 {
     auto curv = [](float a, float b, float c) { return fmaf(-2.f, b, a) + c; };
-    const float e3 = p[(long)(L - 3) * step], e2 = p[(long)(L - 2) * step], e1 = p[(long)(L - 1) * step];
+    const float e3 = p[(L - 3) * step], e2 = p[(L - 2) * step], e1 = p[(L - 1) * step];
     const float s0 = p[0], s1 = p[step];
     float held[kStash], sum = 0.f;
     // face i + 1/2 from its upper side: donor c0 = cell i, cm1 = i - 1, ... ; start at i = L - 1
@@ -99,7 +99,7 @@ __device__ __forceinline__ float march_shift_down(float *p, long step, int L, in
     float d = curv(cm1, c0, cp1), dm = curv(cm2, cm1, c0); // curvatures of cells i, i - 1
     float q = minmod_curv(dm, d);                          // at face i - 1/2
     float Fp = cell_flux(k, cm2, cm1, c0, cp1, s1, q, minmod_curv(d, curv(c0, cp1, s1)));
-    auto cell = [&](int i, float cm3) { // cell i, with cell i - 3
+    auto cell = [&](float cm3) { // the next cell i down, with cell i - 3
         const float dmm = curv(cm3, cm2, cm1), qm = minmod_curv(dmm, dm);
         const float F = cell_flux(k, cm3, cm2, cm1, c0, cp1, qm, q); // face i - 1/2, donor cell i - 1
         const float out = c0 + (F - Fp);
@@ -113,15 +113,19 @@ __device__ __forceinline__ float march_shift_down(float *p, long step, int L, in
         Fp = F;
         return out;
     };
-    for (int i = L - 1; i >= L - N; --i) held[i - (L - N)] = cell(i, i >= 3 ? p[(long)(i - 3) * step] : i == 2 ? e1 : i == 1 ? e2 : e3);
+    int to = L - 1 + N; // where cell i goes; past the end of the line it wraps to row to - L
+    auto put = [&](float v) {
+        if (to < L) p[to * step] = v;
+        else held[to - L] = v;
+        --to;
+    };
+    const float *below = p + (L - 4) * step; // cell i - 3
 #pragma unroll 4
-    for (int i = L - N - 1; i >= 3; --i) {
-        const float cm3 = p[(long)(i - 3) * step];
-        p[(long)(i + N) * step] = cell(i, cm3);
-    }
-    for (int i = L - N - 1 < 2 ? L - N - 1 : 2; i >= 0; --i)
-        p[(long)(i + N) * step] = cell(i, i == 2 ? e1 : i == 1 ? e2 : e3);
-    for (int j = 0; j < N; ++j) p[(long)j * step] = held[j];
+    for (int i = L - 1; i >= 3; --i, below -= step) put(cell(*below));
+    put(cell(e1));
+    put(cell(e2));
+    put(cell(e3));
+    for (int j = 0; j < N; ++j) p[j * step] = held[j];
     return sum;
 }
 
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
                 C sum;
                 if constexpr (PERIODIC && sizeof(T) == 4) {
                     if (N % L <= kStash && N % L < L) {
-                        sum = march_shift_down(base, step, L, N % L, kc);
+                        sum = march_shift_down(base, int(step), L, N % L, kc);
                     } else {
                         sum = march_shift<PERIODIC>(base, step, L, kc);
                         rotate_line(base, step, L, N % L);

@@ -33,6 +33,7 @@ __global__ void velocity_coef_kernel(int nx, int ny, int nz, const float *__rest
 {
     const unsigned ncell = unsigned(nx) * ny * nz; // <= 2^24
     const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_enter();
     if (c >= ncell) return;
     const int d = ax.axis[blockIdx.y];
     const int st = d == 2 ? 1 : d == 1 ? nz : ny * nz, n = d == 2 ? nz : d == 1 ? ny : nx;
@@ -65,13 +66,15 @@ cudaError_t launch_velocity_coef(const GridDims &g, const float *phi, double dt,
     if (!axes) return cudaSuccess;
     const int threads = ncell >= 65536 ? 128 : 32;
     const dim3 grid(unsigned((ncell + threads - 1) / threads), unsigned(axes));
+    const long long velocity = (long long)g.nu[0] * g.nu[1] * g.nu[2];
+    auto launch = [&](auto kernel, auto *cx, auto *cy, auto *cz) {
+        return launch_chained_t(ncell * velocity * (dtype == 0 ? 16 : 1), kernel, grid, dim3(threads), 0, st, g.n[0], g.n[1], g.n[2], phi, ax, cx, cy, cz, err);
+    };
     if (dtype == 0)
-        velocity_coef_kernel<double><<<grid, threads, 0, st>>>(g.n[0], g.n[1], g.n[2], phi, ax, (LineCoefT<double> *)coef_x,
-                                                              (LineCoefT<double> *)coef_y, (LineCoefT<double> *)coef_z, err);
-    else
-        velocity_coef_kernel<float><<<grid, threads, 0, st>>>(g.n[0], g.n[1], g.n[2], phi, ax, (LineCoefT<float> *)coef_x,
-                                                             (LineCoefT<float> *)coef_y, (LineCoefT<float> *)coef_z, err);
-    return cudaGetLastError();
+        return launch(velocity_coef_kernel<double>, (LineCoefT<double> *)coef_x, (LineCoefT<double> *)coef_y,
+                      (LineCoefT<double> *)coef_z);
+    return launch(velocity_coef_kernel<float>, (LineCoefT<float> *)coef_x, (LineCoefT<float> *)coef_y,
+                  (LineCoefT<float> *)coef_z);
 }
 
 // ----------------------------------------------------------------------------
@@ -226,6 +229,7 @@ __global__ void __launch_bounds__(256) moment_finish_kernel(const P *__restrict_
 {
     __shared__ double red[4][64];
     const int tx = threadIdx.x & 63, grp = threadIdx.x >> 6;
+    chain_enter();
     for (long long c = blockIdx.x; c < cells_per_row; c += gridDim.x) {
         const P *q = mpart + c * nparts * (long long)nx;
         for (int x0 = 0; x0 < nx; x0 += 64) {
@@ -246,12 +250,10 @@ cudaError_t launch_moment_finish(const void *mpart, int dtype, int nparts, int n
 {
     const long long blocks = cells_per_row < (long long)sm_count * 8 ? cells_per_row : (long long)sm_count * 8;
     if (dtype == 0)
-        moment_finish_kernel<double><<<int(blocks), 256, 0, st>>>((const double *)mpart, nparts, nx, cells_per_row,
-                                                                     du3, rho);
-    else
-        moment_finish_kernel<float><<<int(blocks), 256, 0, st>>>((const float *)mpart, nparts, nx, cells_per_row, du3,
-                                                                    rho);
-    return cudaGetLastError();
+        return launch_chained_t(cells_per_row * nx * nparts * 128 * 16, moment_finish_kernel<double>, dim3(unsigned(blocks)), dim3(256), 0, st, (const double *)mpart,
+                                nparts, nx, cells_per_row, du3, rho);
+    return launch_chained_t(cells_per_row * nx * nparts * 256, moment_finish_kernel<float>, dim3(unsigned(blocks)), dim3(256), 0, st, (const float *)mpart, nparts,
+                            nx, cells_per_row, du3, rho);
 }
 
 // Adjoint of the moment: rho(x) = du^3 sum_u f(x, u), so dL/df(x, u) =
@@ -611,7 +613,8 @@ template <Dft M> __global__ void __launch_bounds__(256) dft_axis_kernel(const __
     const int sa = da == 0 ? a.n[1] * a.n[2] : a.n[2], sb = db == 1 ? a.n[2] : 1;
     const int li = threadIdx.x / n, k = threadIdx.x - li * n; // this thread: line li of the block, index k
     double2 *tw = dft_smem, *x = tw + n + li * n, *y = tw + n + (a.lines + li) * n;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) tw[q] = a.tw[q];
+    for (int q = threadIdx.x; q < n; q += blockDim.x) tw[q] = a.tw[q]; // written at start-up: no kernel before writes it
+    chain_enter();
     const unsigned line = blockIdx.x * unsigned(a.lines) + li;
     const bool act = line < a.nlines;
     const int ia = int(line / unsigned(a.n[db])), ib = int(line - unsigned(ia) * a.n[db]);
@@ -661,6 +664,7 @@ cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const do
     A.L = g.L;
     A.phi = phi;
     A.phi64 = phi64;
+    cudaError_t err = cudaSuccess;
     auto dft = [&](auto kernel, int d, int sign, const double2 *in, double2 *out) {
         const int nd = g.n[d]; // <= 256
         A.nlines = unsigned(n / nd);
@@ -674,14 +678,16 @@ cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const do
         A.in = in;
         A.out = out;
         A.tw = ps.tw[d];
-        kernel<<<(A.nlines + A.lines - 1) / A.lines, A.lines * nd, (2 * A.lines + 1) * nd * sizeof(double2), st>>>(A);
+        const cudaError_t e = launch_chained_t(n * g.nu[0] * g.nu[1] * g.nu[2], kernel, dim3((A.nlines + A.lines - 1) / A.lines), dim3(A.lines * nd),
+                                               (2 * A.lines + 1) * nd * sizeof(double2), st, A);
+        if (err == cudaSuccess) err = e;
     };
     dft(dft_axis_kernel<Dft::first>, 2, -1, nullptr, ps.z0);
     dft(dft_axis_kernel<Dft::plain>, 1, -1, ps.z0, ps.z1);
     dft(dft_axis_kernel<Dft::middle>, 0, -1, ps.z1, ps.z0);
     dft(dft_axis_kernel<Dft::plain>, 1, +1, ps.z0, ps.z1);
     dft(dft_axis_kernel<Dft::last>, 2, +1, ps.z1, nullptr);
-    return cudaGetLastError();
+    return err;
 }
 
 } // namespace vk

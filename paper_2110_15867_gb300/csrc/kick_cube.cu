@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(PairCube<NU>::threads + kProducer, NU == 32 ? 
         fence_barrier_init();
     }
     __syncthreads();
+    chain_enter();
 
     const long long Gd = gridDim.x, b = blockIdx.x;
     const unsigned n_my = unsigned(a.ncells > b ? (a.ncells - b + Gd - 1) / Gd : 0);
@@ -464,6 +465,7 @@ __global__ void __launch_bounds__(PairCube16<NU, T>::threads + kProducer, NU == 
         fence_barrier_init();
     }
     __syncthreads();
+    chain_enter();
 
     const long long Gd = gridDim.x, b = blockIdx.x;
     const unsigned n_my = unsigned(a.ncells > b ? (a.ncells - b + Gd - 1) / Gd : 0);
@@ -694,7 +696,7 @@ cudaError_t launch_kick_cube(const CUtensorMap &fmap, const CUtensorMap &smap, c
     void *params_coded[] = {const_cast<CUtensorMap *>(&fmap), const_cast<CUtensorMap *>(&smap), &args};
     void **params = dtype == 1 ? params_f32 : params_coded;
     const int threads = nu == 32 ? threads_for<32>() : threads_for<16>();
-    return cudaLaunchKernel(k, dim3(grid), dim3(threads), params, smem, st);
+    return launch_chained(a.ncells * nu * nu * nu, k, dim3(grid), dim3(threads), smem, st, params);
 }
 
 } // namespace vk

@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(PlaneGeom<NU>::threads, 5)
     const int row0 = threadIdx.x / CH, col0 = PER * (threadIdx.x - row0 * CH);
     T *g = f + p0 * NU * NU + row0 * NU + col0;
     float *sg = plane_s + row0 * P + col0;
+    chain_enter();
 #pragma unroll
     for (int k = 0; k < ROWS / RP; ++k) {
         if constexpr (CODED) { // decoded with their row's scale
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(kAnyThreads, 5)
     const int planes = pend - p0 < a.per_block ? int(pend - p0) : a.per_block;
     const long long e0 = p0 * ny * nz;
     const int chunks = planes * ny * u;
+    chain_enter();
     for (int k = threadIdx.x; k < chunks; k += kAnyThreads) {
         const int row = int(fdiv(unsigned(k), a.div_u)), col = k - row * u;
         copy16(any_s + row * pitch + 4 * col, src + e0 + 4ll * k);
@@ -329,8 +331,8 @@ template <typename T> static cudaError_t launch_plane_tail_t(T *f, const PlaneTa
     const cudaError_t e = cudaFuncSetAttribute(plane_tail_kernel<48, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                int(PlaneGeom<48>::smem));
     if (e != cudaSuccess) return e;
-    plane_tail_kernel<48, T><<<unsigned(blocks), PlaneGeom<48>::threads, PlaneGeom<48>::smem, st>>>(f, a);
-    return cudaGetLastError();
+    return launch_chained_t(a.nplanes * 48 * 48, plane_tail_kernel<48, T>, dim3(unsigned(blocks)), dim3(PlaneGeom<48>::threads), PlaneGeom<48>::smem,
+                            st, f, a);
 }
 
 cudaError_t launch_plane_tail(void *f, const PlaneTailArgs &a, int nu, int dtype, cudaStream_t st)
@@ -370,8 +372,7 @@ cudaError_t launch_plane_any(const float *src, float *dst, const PlaneAnyArgs &a
     const cudaError_t e = cudaFuncSetAttribute(plane_any_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     const long long blocks = (a.nplanes + a.per_block - 1) / a.per_block;
-    plane_any_kernel<<<unsigned(blocks), kAnyThreads, smem, st>>>(src, dst, a);
-    return cudaGetLastError();
+    return launch_chained_t(a.nplanes * a.nuy * a.nuz, plane_any_kernel, dim3(unsigned(blocks)), dim3(kAnyThreads), smem, st, src, dst, a);
 }
 
 } // namespace vk

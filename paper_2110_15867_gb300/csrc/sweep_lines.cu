@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(kLine1Threads + kProducer, 3)
         fence_barrier_init();
     }
     __syncthreads();
+    chain_enter();
 
     const long long Gd = gridDim.x, b = blockIdx.x;
     const unsigned n_my = unsigned((args.num_tiles > b) ? (args.num_tiles - b + Gd - 1) / Gd : 0);
@@ -248,6 +249,7 @@ __global__ void __launch_bounds__(256, L > 32 ? 2 : 3) reg_lines_kernel(const T 
 {
     constexpr bool CODED = sizeof(T) == 2;
     const long long t = a.line0 + blockIdx.x * 256ll + threadIdx.x;
+    chain_enter();
     if (t >= a.line0 + a.nlines) return;
     long long outer, cell;
     if (a.line0 + a.nlines <= 0xffffffffll) { // every line index of the launch fits 32 bits
@@ -306,11 +308,9 @@ template <typename T> static cudaError_t launch_reg_t(const void *src, void *dst
 {
     const T *s = static_cast<const T *>(src);
     T *d = static_cast<T *>(dst);
-    if (a.L == 32) reg_lines_kernel<32, T><<<blocks, 256, 0, st>>>(s, d, a);
-    else if (a.L == 16) reg_lines_kernel<16, T><<<blocks, 256, 0, st>>>(s, d, a);
-    else if (a.L == 48) reg_lines_kernel<48, T><<<blocks, 256, 0, st>>>(s, d, a);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    auto kern = a.L == 32 ? reg_lines_kernel<32, T> : a.L == 16 ? reg_lines_kernel<16, T> : a.L == 48 ? reg_lines_kernel<48, T> : nullptr;
+    if (!kern) return cudaErrorInvalidValue;
+    return launch_chained_t(a.nlines * a.L, kern, dim3(blocks), dim3(256), 0, st, s, d, a);
 }
 
 cudaError_t launch_reg_lines(const void *src, void *dst, const RegLineArgs &args, int dtype, cudaStream_t st)
@@ -500,7 +500,7 @@ cudaError_t launch_line_sweep(const CUtensorMap &map, const CUtensorMap &dmap, c
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
     const int threads = kLine1Threads + kProducer;
-    return cudaLaunchKernel(k, dim3(grid), dim3(threads), args, smem, st);
+    return launch_chained(a.rows * nu, k, dim3(grid), dim3(threads), smem, st, args);
 }
 
 int occupancy_line_sweep(int nu, int dtype, bool fuse_y)

@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(kMaxGroups *kGroup + kProducer, 1)
     }
     for (int j = threadIdx.x; j < a.nvel; j += blockDim.x) tab[j] = a.table[j];
     __syncthreads();
+    chain_enter();
 
     const unsigned G = gridDim.x, b = blockIdx.x; // every tile and column index fits 32 bits (host)
     const unsigned n_my = a.num_tiles > b ? (a.num_tiles - b + G - 1) / G : 0;
@@ -212,7 +213,7 @@ cudaError_t launch_pair32(const CUtensorMap &map, const CUtensorMap &dmap, const
     cudaError_t e = cudaFuncSetAttribute(pair32(zf), cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
-    return cudaLaunchKernel(pair32(zf), dim3(grid), dim3(a.groups * kGroup + kProducer), params, smem, st);
+    return launch_chained((long long)a.num_tiles * kCols * a.L, pair32(zf), dim3(grid), dim3(a.groups * kGroup + kProducer), smem, st, params);
 }
 
 } // namespace vk

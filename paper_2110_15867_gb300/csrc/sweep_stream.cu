@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(Lane<T>::NC + stream_head<MOMENT>(), kStreamMi
     if (args.coef_mode == 0)
         for (int j = threadIdx.x; j < args.nvel; j += blockDim.x) tab[j] = args.table[j];
     __syncthreads();
+    chain_enter();
 
     const long long G = gridDim.x, b = blockIdx.x;
     const long long n_my = (args.num_blocks > b) ? (args.num_blocks - b + G - 1) / G : 0;
@@ -562,8 +563,7 @@ static cudaError_t launch_stream_t(const CUtensorMap &map, const CUtensorMap &dm
         }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
-    kern<<<grid, threads, smem, st>>>(map, dmap, smap, a);
-    return cudaGetLastError();
+    return launch_chained_t(a.num_blocks * a.W * a.P * a.L * (sizeof(T) == 8 ? 16 : 1), kern, dim3(grid), dim3(threads), smem, st, map, dmap, smap, a);
 }
 
 cudaError_t launch_stream_f32(const CUtensorMap &map, const CUtensorMap &dmap, const StreamArgs<float> &a, int grid,

@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(tile_groups<L>() * 256 + kProducer, 1)
     }
     for (int j = threadIdx.x; j < a.nvel; j += blockDim.x) tab[j] = a.table[j];
     __syncthreads();
+    chain_enter();
 
     const long long G = gridDim.x, b = blockIdx.x;
     const unsigned n_my = unsigned(a.num_tiles > b ? (a.num_tiles - b + G - 1) / G : 0);
@@ -301,7 +302,7 @@ cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, c
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), const_cast<TileArgs *>(&a)};
-    return cudaLaunchKernel(k, dim3(grid), dim3(tile_threads_for(a.L)), params, smem, st);
+    return launch_chained(a.num_tiles * 256 * a.L, k, dim3(grid), dim3(tile_threads_for(a.L)), smem, st, params);
 }
 
 } // namespace vk

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(kPairGroups *kPairGroup + kProducer, 1)
     }
     for (int j = threadIdx.x; j < a.nvel; j += blockDim.x) tab[j] = a.table[j];
     __syncthreads();
+    chain_enter();
 
     const unsigned G = gridDim.x, b = blockIdx.x; // every tile and column index fits 32 bits (host)
     const unsigned n_my = a.num_tiles > b ? (a.num_tiles - b + G - 1) / G : 0;
@@ -302,7 +303,7 @@ cudaError_t launch_tile16(const CUtensorMap &map, const CUtensorMap &smap, const
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&smap), &a};
-    return cudaLaunchKernel(k, dim3(grid), dim3(a.groups * kPairGroup + kProducer), params, smem, st);
+    return launch_chained((long long)a.num_tiles * 256 * a.L, k, dim3(grid), dim3(a.groups * kPairGroup + kProducer), smem, st, params);
 }
 
 } // namespace vk

@@ -141,11 +141,14 @@ def measured_peaks():
 # the sources each timed kernel kind is built from (its DRAM traffic record is void once
 # one of them changes)
 _COMMON_SOURCES = ("vk_common.cuh", "vk_kernels.h")
+_TILE_SOURCES = ("sweep_tile.cu", "sweep_pair32.cu", "vk_tiles.cuh", "vk_lines.cuh")
 KERNEL_SOURCES = {
-    # FP32 position sweeps of 16-64 cells: whole lines staged per tile
-    "sweep_x": ("sweep_tile.cu",), "sweep_y": ("sweep_tile.cu",), "sweep_z": ("sweep_tile.cu",),
-    "sweep_ux": ("sweep_lines.cu", "vk_lines.cuh"), "sweep_uy": ("sweep_lines.cu", "vk_lines.cuh"),
-    "sweep_uz": ("sweep_lines.cu", "vk_lines.cuh"), "sweep_uyuz": ("sweep_lines.cu", "vk_lines.cuh"),
+    # FP32 position sweeps: whole lines staged per tile, one or two lines per thread
+    "sweep_x": _TILE_SOURCES, "sweep_y": _TILE_SOURCES, "sweep_z": _TILE_SOURCES,
+    "sweep_ux": _TILE_SOURCES + ("sweep_lines.cu",),
+    "sweep_uy": ("plane_tail.cu", "sweep_lines.cu", "vk_lines.cuh"),
+    "sweep_uz": ("plane_tail.cu", "sweep_lines.cu", "vk_lines.cuh"),
+    "sweep_uyuz": ("plane_tail.cu", "sweep_lines.cu", "vk_lines.cuh"),
     "kick": ("kick_cube.cu", "vk_lines.cuh"),
 }
 

@@ -15,7 +15,7 @@
 // touched by faces at both ends; their partial sums wait in registers until
 // the last face.
 //
-// One thread per line.  Strided axes (x, y, z, u_x, u_y): neighbouring threads
+// FP32 position lines run on staged tiles (adjoint_tile.cu).  One thread per line.  Strided axes (x, y, z, u_x, u_y): neighbouring threads
 // own neighbouring columns, so every row access of a warp is one coalesced
 // segment.  u_z: a line is one contiguous row; for n_uz = 8, 16, 32 the row
 // reaches the thread's registers through 16-byte vector loads (32: staged per
@@ -27,7 +27,7 @@
 // per block and cell).
 #include <type_traits>
 
-#include "vk_common.cuh"
+#include "vk_adjoint.cuh"
 
 namespace vk {
 
@@ -35,7 +35,7 @@ constexpr int kAdjBlock = 256;    // threads (lines) per block: position lines, 
 // velocity lines and u_z rows of up to 16 cells: blocks of two warps, four times as many
 // resident (the warps of a block wait for each other at the per-cell reduction of dL/dnu;
 // on 32^3 x 16^3: u_x 0.374 -> 0.359 ms, u_z 0.362 -> 0.335 ms against 256 threads, 0.361 /
-// 0.341 with 128; position lines are slower in smaller blocks: 0.556 -> 0.584 ms with 128)
+// 0.341 with 128)
 constexpr int kAdjVelBlock = 64;
 template <bool PERIODIC> constexpr int adj_block() { return PERIODIC ? kAdjBlock : kAdjVelBlock; }
 constexpr int kAdjUnroll = 1;    // interior faces per loop iteration of the column march
@@ -169,19 +169,6 @@ template <typename C> __device__ __forceinline__ C dm4_val(C d0, C d1)
     return mn2(mx2(lo, C(0)), hi);
 }
 
-// the same with its partials ka = dr/dd0 and kb = dr/dd1 (the selected
-// argument's; 0 where the minmod is 0)
-template <typename C> __device__ __forceinline__ C dm4_coef(C d0, C d1, C &ka, C &kb)
-{
-    const C a = C(4) * d0 - d1, b = C(4) * d1 - d0;
-    const C lo = mn2(mn3(a, b, d0), d1), hi = mx2(mx3(a, b, d0), d1);
-    const C r = mn2(mx2(lo, C(0)), hi);
-    const bool z = r == C(0), ia = r == a, ib = r == b, i0 = r == d0;
-    ka = z ? C(0) : ia ? C(4) : ib ? C(-1) : i0 ? C(1) : C(0);
-    kb = z ? C(0) : ia ? C(-1) : ib ? C(4) : i0 ? C(0) : C(1);
-    return r;
-}
-
 // Acc supplies, for local indices 0 <= i < n: c(i) the sweep input, lam(i)
 // dL/dc_new (read only before cell i is written) and put(i, v) dL/dc.
 //
@@ -202,9 +189,8 @@ template <typename C> __device__ __forceinline__ C dm4_coef(C d0, C d1, C &ka, C
 // source selection; the other faces compute the dm4 at their upwind face with
 // its partials from the curvatures in the window.  On the smooth velocity
 // profiles every face is plain.  Position lines, limited at about half of
-// their faces, take the general path at every face (two bodies side by side
-// made the unrolled position walks slower) and keep each dm4 with its partials
-// for the next face.
+// their faces, take the general path at every face and keep each dm4 with its
+// partials for the next face.
 template <bool PERIODIC, typename C, typename Acc> struct AdjMarch {
     Acc &acc;
     const AdjLim<C> &k;
@@ -658,27 +644,15 @@ __global__ void __launch_bounds__(adj_block<PERIODIC>(),
             const AdjLim<C> lim = make_adj_lim(kc);
             C dLds, osum;
             if constexpr (!SMALL4 && LCT > 0 && LCT <= kAdjRegMax) {
-                // short line: every load first (in walk order; lambda rotated by a
-                // periodic whole-cell shift, read straight when there is none: the
-                // rotated index costs the position adjoints 0.556 against 0.526 ms),
-                // the march on registers, then every store
-                const int shift = PERIODIC ? (kc.nd >> 1) % LCT : 0;
+                // short velocity line: every load first (in walk order), the march on
+                // registers, then every store
+                static_assert(!PERIODIC, "position lines run on staged tiles (adjoint_tile.cu)");
                 RegLine<T, LCT, false> acc;
                 const T *fp = f + off, *lp = lin + off;
-                if (shift == 0) {
 #pragma unroll
-                    for (int i = 0; i < LCT; ++i) {
-                        acc.cv[i] = fp[i * st];
-                        acc.lv[i] = lp[i * st];
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < LCT; ++i) {
-                        int r = i + shift;
-                        if (r >= LCT) r -= LCT;
-                        acc.cv[i] = fp[i * st];
-                        acc.lv[i] = lp[r * st];
-                    }
+                for (int i = 0; i < LCT; ++i) {
+                    acc.cv[i] = fp[i * st];
+                    acc.lv[i] = lp[i * st];
                 }
                 march_adjoint<PERIODIC, LCT, C>(acc, lim, LCT, dLds, osum);
 #pragma unroll
@@ -923,19 +897,12 @@ template <typename T> static cudaError_t launch_adj_t(const AdjArgs<T> &a_in, bo
     } else if (a.periodic && a.L == 4) {
         adjoint_lines_kernel<T, true, true, 0><<<grid, bt, 0, st>>>(a);
     } else if constexpr (std::is_same<T, float>::value) {
-        // FP32: unrolled walks for the common line lengths
-        const bool p = a.periodic;
-#define ADJ_LINES(LL)                                                                                              \
-    if (a.L == LL) {                                                                                                  \
-        if (p) adjoint_lines_kernel<T, true, false, LL><<<grid, bt, 0, st>>>(a);                               \
-        else adjoint_lines_kernel<T, false, false, LL><<<grid, bt, 0, st>>>(a);                                \
-        return cudaGetLastError();                                                                                    \
-    }
-        ADJ_LINES(16)
-        ADJ_LINES(32)
-        ADJ_LINES(64)
-#undef ADJ_LINES
-        if (p) adjoint_lines_kernel<T, true, false, 0><<<grid, bt, 0, st>>>(a);
+        // FP32: unrolled walks for the common lengths of velocity lines (position lines of 6
+        // to about 110 cells run on staged tiles)
+        if (a.periodic) adjoint_lines_kernel<T, true, false, 0><<<grid, bt, 0, st>>>(a);
+        else if (a.L == 16) adjoint_lines_kernel<T, false, false, 16><<<grid, bt, 0, st>>>(a);
+        else if (a.L == 32) adjoint_lines_kernel<T, false, false, 32><<<grid, bt, 0, st>>>(a);
+        else if (a.L == 64) adjoint_lines_kernel<T, false, false, 64><<<grid, bt, 0, st>>>(a);
         else adjoint_lines_kernel<T, false, false, 0><<<grid, bt, 0, st>>>(a);
     } else {
         if (a.periodic) adjoint_lines_kernel<T, true, false, 0><<<grid, bt, 0, st>>>(a);

@@ -426,6 +426,21 @@ cudaError_t launch_adjoint_f32(const AdjArgs<float> &a, bool rows, cudaStream_t 
 cudaError_t launch_adjoint_f64(const AdjArgs<double> &a, bool rows, cudaStream_t st);
 // lines (threads) per block of the adjoint kernel of axis (rows: the u_z row kernels; L: line length)
 int adjoint_block(int axis, bool rows, int L);
+// the same for FP32 position sweeps on staged tiles (adjoint_tile.cu), in place on lambda; fmap
+// and lmap view f_in and lambda as [n_outer][L][n_inner] with box {cols, L, 1}
+struct AdjTileArgs {
+    int L, cols;                     // cells of a line; columns of a tile
+    unsigned tiles_inner, num_tiles; // tiles of a row (the last may be partial), of the array
+    int slots, groups;               // of the ring; thread groups
+    long long vstride;               // column j takes table[(inner / vstride) % nvel]
+    int nvel;
+    unsigned *err;
+    FastDivU32 div_tiles, div_vstride, div_nvel; // set by the launcher
+    LineCoefT<float> table[kMaxVel];
+};
+// lines of 6 to about 110 cells
+bool adjoint_tile_geometry(int L, long long n_inner, long long n_outer, AdjTileArgs &a);
+cudaError_t launch_adjoint_tile(const CUtensorMap &fmap, const CUtensorMap &lmap, const AdjTileArgs &a, int sms, cudaStream_t st);
 // dLdg[c] += fac * sum_q part[c * blocks_per_cell + q] in order
 cudaError_t launch_cell_sum(long long ncell, int blocks_per_cell, const double *part, double fac, double *dLdg,
                             cudaStream_t st);

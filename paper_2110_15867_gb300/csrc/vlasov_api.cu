@@ -1635,6 +1635,27 @@ static int ensure_buffer(vlasov_ctx *c, void **p, size_t bytes)
     return VLASOV_OK;
 }
 
+// position adjoint of FP32 storage on staged tiles; *done stays false where it does not apply
+static int run_adjoint_tiles(vlasov_ctx *c, const void *f_in, void *lam, int ax, long long I, long long O, const AdjArgs<float> &P,
+                             bool *done)
+{
+    AdjTileArgs A{};
+    if (!adjoint_tile_geometry(P.L, I, O, A)) return VLASOV_OK;
+    A.vstride = P.vstride;
+    A.nvel = P.nvel;
+    A.err = P.err;
+    for (int j = 0; j < P.nvel; ++j) A.table[j] = P.table[j];
+    const MapSpec spec = spec3(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, I, P.L, O, 4, A.cols, P.L, 1);
+    CUtensorMap fmap, lmap;
+    if (encode_spec(&fmap, spec, f_in) != CUDA_SUCCESS || encode_spec(&lmap, spec, lam) != CUDA_SUCCESS)
+        return fail(c, VLASOV_ECUDA, "tensor map of an adjoint sweep failed");
+    PartTimer t(c, VLASOV_T_ADJ_X + ax, 1);
+    const cudaError_t e = launch_adjoint_tile(fmap, lmap, A, c->sm_count, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "adjoint sweep launch");
+    *done = true;
+    return VLASOV_OK;
+}
+
 // lam <- (dD_axis/df)^T lam at the sweep input f_in.  Velocity sweeps read the
 // constants in d_coef[axis - 3] (prepared for the same phi and dt) and add
 // dL/dg to dLdg (ncell FP64, may be null).
@@ -1671,6 +1692,11 @@ static int run_adjoint_t(vlasov_ctx *c, const void *f_in, void *lam, int ax, dou
             const double nu = (-c->g.V + (j + 0.5) * du) * dt / (a * a * dx);
             A.table[j] = make_line_coef<C>(nu);
             shifted = shifted || fabs(nu) >= 1.0;
+        }
+        if constexpr (sizeof(C) == 4) {
+            bool done = false;
+            const int rc = run_adjoint_tiles(c, f_in, lam, ax, I, O, A, &done);
+            if (rc || done) return rc;
         }
         // z: group each block's threads by the sign of u_z (whole u_z lines per block)
         const int bt = adjoint_block(ax, false, int(d6[ax])), nuz = int(c->g.nuz);

@@ -18,14 +18,15 @@
 // mostly agree) takes no more than that; the others find the source and scatter the
 // curvature's partials in a branch.
 //
-// Bound by instruction issue: 68 thread instructions per update at 80 % issue, against 104 at
-// 68 % when a line was marched in registers over the cells' own values, fully unrolled (lines of
-// 16, 32, 64 cells; others walked global memory).  x sweep of 32^3 x 16^3 0.527 -> 0.307 ms
-// (DRAM alone 0.238), of 24^3 x 16^3 0.389 -> 0.143 (0.100), of 20 x 22 x 48 x 20 x 16 x 12 0.572 ->
-// 0.201 (0.144).
+// Bound by instruction issue: 68 thread instructions per update at 80 % issue where few faces
+// take the branch, against 104 at 68 % when a line was marched in registers over the cells' own
+// values, fully unrolled (lines of 16, 32, 64 cells; others walked global memory).  x sweep of
+// 32^3 x 16^3 0.527 -> 0.300 ms (DRAM alone 0.238), of 24^3 x 16^3 0.389 -> 0.142 (0.100), of 20 x 22
+// x 48 x 20 x 16 x 12 0.572 -> 0.196 (0.144).  Where many faces are limited the branch counts: the
+// x sweep of a 24^3 x 16^3 run 0.190 with the minmod's partials found from its four arguments at
+// every such face, 0.174 from the two magnitudes, 0.161 and only where an adjoint is pending.
 #include <type_traits>
 
-#include "vk_adjoint.cuh"
 #include "vk_tiles.cuh"
 
 namespace vk {
@@ -62,12 +63,15 @@ struct AdjFaces {
         gq = gl = g0 = g1 = g2 = b0 = b1 = 0.f;
         l0 = lam0;
     }
-    // adjoint x of dm4 at j - 1/2, of curvatures dm - dmm and d0
+    // adjoint x of dm4 at j - 1/2 = minmod(4 a - b, 4 b - a, a, b), a and b the curvatures of
+    // cells j - 1 and j: the argument of least magnitude is 4 a - b where |b| >= 3 |a|, 4 b - a
+    // where |a| >= 3 |b|, else the smaller of a and b; nothing where the minmod is 0
     __device__ __forceinline__ void scatter_curv(float x)
     {
-        float ka, kb;
-        dm4_coef(dm - dmm, d0, ka, kb);
-        const float xm = x * ka, x0 = x * kb;
+        const float a = fabsf(dm - dmm), b = fabsf(d0);
+        const bool ia = b >= 3.f * a, ib = a >= 3.f * b, i0 = a <= b;
+        if (qm == 0.f) x = 0.f;
+        const float xm = x * (ia ? 4.f : ib ? -1.f : i0 ? 1.f : 0.f), x0 = x * (ia ? -1.f : ib ? 4.f : i0 ? 0.f : 1.f);
         g0 -= xm;
         g1 += xm - x0;
         g2 += x0;
@@ -99,7 +103,8 @@ struct AdjFaces {
             g2 = fmaf(x, e1 ? 1.f : em ? 0.5f : 0.f, g2);
             g1 = fmaf(x, eu ? k.alpha : el ? 0.5f : 0.f, g1);
             gn = em ? -0.5f * x : 0.f;
-            scatter_curv(el ? fmaf(4.f / 3.f, x, gq) : gq);
+            const float y = el ? fmaf(4.f / 3.f, x, gq) : gq;
+            if (y != 0.f) scatter_curv(y);
         }
         const float out = b0 + (gl - g0);
         gl = g0;

@@ -20,114 +20,9 @@
 //     shared memory, in place.
 // Every wait is bounded: on expiry the kernel raises ERR_TIMEOUT in the error
 // word and returns.
-#include "vk_common.cuh"
+#include "vk_shift.cuh"
 
 namespace vk {
-
-// The FP32 march of this kernel, with the flux written in the cells themselves (34
-// operations a face) where every other kernel takes differences (31): over a drift of
-// whole-cell shifts the two forms' roundings, both right to 7e-8 of the 2-norm, were driven
-// apart in single cells by the limiter (3e-5 of the rms after six sweeps), more than these
-// sweeps' results may change, for 4 % of their time (32 x 24 x 32 x 16 x 16 x 32 cells: 1.665
-// against 1.597 ms, three sweeps).
-__device__ __forceinline__ float minmod_curv(float d0, float d1)
-{
-    const float a = 4.f * d0 - d1, b = 4.f * d1 - d0;
-    return mn2(mx2(mn2(mn3(a, b, d0), d1), 0.f), mx2(mx3(a, b, d0), d1));
-}
-__device__ __forceinline__ float cell_flux(const LineCoefT<float> &k, float cm2, float cm1, float c0, float cp1,
-                                           float cp2, float dm4m, float dm4p)
-{
-    const float fbar = fmaf(k.w[4], cp2, fmaf(k.w[3], cp1, fmaf(k.w[2], c0, fmaf(k.w[1], cm1, k.w[0] * cm2))));
-    const float dlm = c0 - cm1, ful = fmaf(k.alpha, dlm, c0), fmd = 0.5f * ((c0 + cp1) - dm4p);
-    const float flc = fmaf(4.f / 3.f, dm4m, fmaf(0.5f, dlm, c0));
-    const float v = mn3(mx3(fbar, mn3(c0, cp1, fmd), mn3(c0, ful, flc)), mx3(c0, cp1, fmd), mx3(c0, ful, flc));
-    return flux_clamp(__fmul_rn(k.s, v), c0);
-}
-template <bool PERIODIC>
-__device__ __forceinline__ float march_shift(float *p, long step, int L, const LineCoefT<float> &k)
-{
-    auto curv = [](float a, float b, float c) { return fmaf(-2.f, b, a) + c; };
-    const float s0 = p[0], s1 = p[step];
-    float cm2 = 0.f, cm1 = 0.f, c0 = s0, cp1 = s1, d = curv(0.f, s0, s1), q = minmod_curv(s0, d), Fm = 0.f, sum = 0.f;
-    if (PERIODIC) {
-        const float a = p[(long)(L - 3) * step];
-        cm2 = p[(long)(L - 2) * step];
-        cm1 = p[(long)(L - 1) * step];
-        const float dm = curv(cm2, cm1, s0);
-        d = curv(cm1, s0, s1);
-        q = minmod_curv(dm, d);
-        Fm = cell_flux(k, a, cm2, cm1, s0, s1, minmod_curv(curv(a, cm2, cm1), dm), q); // face -1/2, donor c_{-1}
-    }
-    auto face = [&](int i, float cp2, bool outer) {
-        const float dn = curv(c0, cp1, cp2), qp = minmod_curv(d, dn);
-        const float F = outer ? 0.f : cell_flux(k, cm2, cm1, c0, cp1, cp2, q, qp);
-        const float out = c0 + (Fm - F);
-        p[(long)i * step] = out;
-        sum += out;
-        cm2 = cm1;
-        cm1 = c0;
-        c0 = cp1;
-        cp1 = cp2;
-        d = dn;
-        q = qp;
-        Fm = F;
-    };
-#pragma unroll 4
-    for (int i = 0; i < L - 2; ++i) face(i, p[(long)(i + 2) * step], false);
-    face(L - 2, PERIODIC ? s0 : 0.f, false);
-    face(L - 1, PERIODIC ? s1 : 0.f, !PERIODIC);
-    return sum;
-}
-// The same on a periodic line, walked from its last cell down, with every new value written N
-// cells on (0 <= N <= kStash, N < L): each row is read once and written once, where marching
-// in place and rotating the line afterwards (three reversals) read and wrote it three times.
-// Row i + N has been read when cell i is done; the N values that wrap around to the first
-// rows, still to be read, wait in `held`, and the last three cells, overwritten before the
-// first ones need them, in registers.  The values are march_shift's, face by face.  With tiles
-// small enough for three CTAs per SM: 32 x 24 x 32 x 16 x 16 x 32 cells, x, y, z 0.600, 0.430, 0.643 ->
-// 0.39 ms each (DRAM alone 0.238).
-constexpr int kStash = 8;
-__device__ __forceinline__ float march_shift_down(float *p, int step, int L, int N, const LineCoefT<float> &k)
-{
-    auto curv = [](float a, float b, float c) { return fmaf(-2.f, b, a) + c; };
-    const float e3 = p[(L - 3) * step], e2 = p[(L - 2) * step], e1 = p[(L - 1) * step];
-    const float s0 = p[0], s1 = p[step];
-    float held[kStash], sum = 0.f;
-    // face i + 1/2 from its upper side: donor c0 = cell i, cm1 = i - 1, ... ; start at i = L - 1
-    float cp1 = s0, c0 = e1, cm1 = e2, cm2 = e3;
-    float d = curv(cm1, c0, cp1), dm = curv(cm2, cm1, c0); // curvatures of cells i, i - 1
-    float q = minmod_curv(dm, d);                          // at face i - 1/2
-    float Fp = cell_flux(k, cm2, cm1, c0, cp1, s1, q, minmod_curv(d, curv(c0, cp1, s1)));
-    auto cell = [&](float cm3) { // the next cell i down, with cell i - 3
-        const float dmm = curv(cm3, cm2, cm1), qm = minmod_curv(dmm, dm);
-        const float F = cell_flux(k, cm3, cm2, cm1, c0, cp1, qm, q); // face i - 1/2, donor cell i - 1
-        const float out = c0 + (F - Fp);
-        sum += out;
-        cp1 = c0;
-        c0 = cm1;
-        cm1 = cm2;
-        cm2 = cm3;
-        dm = dmm;
-        q = qm;
-        Fp = F;
-        return out;
-    };
-    int to = L - 1 + N; // where cell i goes; past the end of the line it wraps to row to - L
-    auto put = [&](float v) {
-        if (to < L) p[to * step] = v;
-        else held[to - L] = v;
-        --to;
-    };
-    const float *below = p + (L - 4) * step; // cell i - 3
-#pragma unroll 4
-    for (int i = L - 1; i >= 3; --i, below -= step) put(cell(*below));
-    put(cell(e1));
-    put(cell(e2));
-    put(cell(e3));
-    for (int j = 0; j < N; ++j) p[j * step] = held[j];
-    return sum;
-}
 
 template <bool PERIODIC>
 __device__ __forceinline__ double march_shift(double *p, long step, int L, const LineCoefT<double> &k)

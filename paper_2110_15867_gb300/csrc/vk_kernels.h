@@ -297,6 +297,8 @@ int pair32_columns();
 bool pair32_geometry(int L, long long n_inner, long long n_outer, Pair32Args &a);
 int occupancy_pair32(const Pair32Args &a, bool zf);
 cudaError_t launch_pair32(const CUtensorMap &map, const CUtensorMap &dmap, const Pair32Args &a, int grid, cudaStream_t st);
+// position sweeps that shift whole cells, on the same tiles (sweep_shift32.cu; its own ring)
+cudaError_t launch_shift32(const CUtensorMap &map, const CUtensorMap &dmap, const Pair32Args &a, int grid, cudaStream_t st);
 
 // ----------------------------------------------------------------------------
 // the same on 16-bit storage, two lines per thread (sweep_tile16.cu): position sweeps with

@@ -15,12 +15,13 @@
 // touched by faces at both ends; their partial sums wait in registers until
 // the last face.
 //
-// FP32 position lines run on staged tiles (adjoint_tile.cu).  One thread per line.  Strided axes (x, y, z, u_x, u_y): neighbouring threads
-// own neighbouring columns, so every row access of a warp is one coalesced
-// segment.  u_z: a line is one contiguous row; for n_uz = 8, 16, 32 the row
-// reaches the thread's registers through 16-byte vector loads (32: staged per
-// warp through shared memory) and the march runs on compile-time indices.  A negative Courant number is the mirror image of a
-// positive one: the line is walked from its far end (negated stride).
+// FP32 position lines of 6 to about 110 cells run on staged tiles (adjoint_tile.cu).  Here one
+// thread takes a line.  Strided axes (x, y, z, u_x, u_y): neighbouring threads own neighbouring
+// columns, so every row access of a warp is one coalesced segment.  u_z: a line is one
+// contiguous row; for n_uz = 8, 16, 32 the row reaches the thread's registers through 16-byte
+// vector loads (32: staged per warp through shared memory) and the march runs on compile-time
+// indices.  A negative Courant number is the mirror image of a positive one: the line is walked
+// from its far end (negated stride).
 //
 // For a velocity sweep dL/dnu of every line is summed over its spatial cell
 // and added, times dnu/dg = -dt/du, to dL/dg of that cell (FP64 atomics, one

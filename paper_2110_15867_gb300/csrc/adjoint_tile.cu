@@ -18,7 +18,7 @@
 // mostly agree) takes no more than that; the others find the source and scatter the
 // curvature's partials in a branch.
 //
-// Bound by instruction issue: 68 thread instructions per update at 80 % issue where few faces
+// Bound by instruction issue: 66 thread instructions per update at 81 % issue where few faces
 // take the branch, against 104 at 68 % when a line was marched in registers over the cells' own
 // values, fully unrolled (lines of 16, 32, 64 cells; others walked global memory).  x sweep of
 // 32^3 x 16^3 0.527 -> 0.300 ms (DRAM alone 0.238), of 24^3 x 16^3 0.389 -> 0.142 (0.100), of 20 x 22

@@ -1,8 +1,9 @@
-// sweep_strided.cu -- SL-MPP5 sweeps along a strided axis (x, y, z, u_x, u_y).
+// sweep_strided.cu -- SL-MPP5 position sweeps that shift whole cells (|nu| >= 1 on some line):
+// FP64, and FP32 where the tiles of sweep_shift32.cu do not apply (lines under 12 or over about
+// 110 cells, tiles switched off).
 //
-// Eq. (3) (position advection, periodic) and Eq. (4) (velocity advection,
-// zero-flux faces) of Yoshikawa, Tanaka & Yoshida, SC'21, one directional
-// sweep at a time as in the split step of Eq. (5).
+// Eq. (3) (position advection, periodic) of Yoshikawa, Tanaka & Yoshida, SC'21, one
+// directional sweep at a time as in the split step of Eq. (5).
 //
 // f is viewed as a 3D tensor [O][L][I]: the swept axis (length L, stride I
 // elements) between all slower axes (O) and all faster axes (I).  The GPU

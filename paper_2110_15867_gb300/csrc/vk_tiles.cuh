@@ -1,6 +1,6 @@
 // vk_tiles.cuh -- pieces shared by the kernels whose thread groups take whole-line tiles from
-// a ring of slots in shared memory (sweep_tile.cu, sweep_tile16.cu): 4D tensor copies and
-// the barriers of the ring.
+// a ring of slots in shared memory (sweep_tile.cu, sweep_tile16.cu, sweep_pair32.cu,
+// sweep_shift32.cu, adjoint_tile.cu): 4D tensor copies and the barriers of the ring.
 #pragma once
 
 #include "vk_lines.cuh"

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kMaxGroups *kGroup + kProducer, 1)
                 sum = march_shift_down(p, step, L, Na, Nb, ka, kb);
             } else {
                 auto line = [&](float *q, int N, const LineCoefT<float> &kc) {
-                    const float s = march_shift<true>(q, long(2 * step), L, kc);
+                    const float s = march_shift(q, long(2 * step), L, kc);
                     rotate_line(q, long(2 * step), L, N);
                     return s;
                 };

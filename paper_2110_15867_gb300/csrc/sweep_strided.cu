@@ -25,13 +25,12 @@
 
 namespace vk {
 
-template <bool PERIODIC>
 __device__ __forceinline__ double march_shift(double *p, long step, int L, const LineCoefT<double> &k)
 {
-    return march_line<double, PERIODIC, double>(p, step, L, to_lim(k));
+    return march_line<double, true, double>(p, step, L, to_lim(k));
 }
 
-template <typename T, bool PERIODIC>
+template <typename T>
 __global__ void __launch_bounds__(kConsumers + kProducer)
     strided_sweep_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap dmap,
                          const __grid_constant__ StridedArgs<typename Compute<T>::type> args)
@@ -42,7 +41,7 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);
     uint64_t *done = full + S;
     LineCoefT<C> *tab = reinterpret_cast<LineCoefT<C> *>(smem + 128);
-    const size_t tab_bytes = (args.coef_mode == 0) ? ((sizeof(LineCoefT<C>) * args.nvel + 127) & ~size_t(127)) : 0;
+    const size_t tab_bytes = (sizeof(LineCoefT<C>) * args.nvel + 127) & ~size_t(127);
     T *stage0 = reinterpret_cast<T *>(smem + 128 + tab_bytes);
     const int L = args.L, W = args.W, P = args.P;
     const int tile_elems = W * L * P;
@@ -57,8 +56,7 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
         }
         fence_barrier_init();
     }
-    if (args.coef_mode == 0)
-        for (int j = threadIdx.x; j < args.nvel; j += blockDim.x) tab[j] = args.table[j];
+    for (int j = threadIdx.x; j < args.nvel; j += blockDim.x) tab[j] = args.table[j];
     __syncthreads();
 
     const long long G = gridDim.x, b = blockIdx.x;
@@ -125,11 +123,7 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
         const long long inner = (t % args.tiles_inner) * W + w;
         const long long outer = (t / args.tiles_inner) * P + p;
         if (has_col && inner < args.n_inner && outer < args.n_outer) {
-            LineCoefT<C> kc;
-            if (args.coef_mode == 0)
-                kc = tab[(inner / args.vstride) % args.nvel];
-            else
-                kc = args.cell_coef[outer / args.outer_per_cell];
+            const LineCoefT<C> kc = tab[(inner / args.vstride) % args.nvel];
             if (kc.nd >= 0) {
                 const int N = kc.nd >> 1;
                 const bool neg = kc.nd & 1;
@@ -137,16 +131,16 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
                 T *base = neg ? col + size_t(L - 1) * W : col;
                 const long step = neg ? -long(W) : long(W);
                 C sum;
-                if constexpr (PERIODIC && sizeof(T) == 4) {
+                if constexpr (sizeof(T) == 4) {
                     if (N % L <= kStash && N % L < L) {
                         sum = march_shift_down(base, int(step), L, N % L, kc);
                     } else {
-                        sum = march_shift<PERIODIC>(base, step, L, kc);
+                        sum = march_shift(base, step, L, kc);
                         rotate_line(base, step, L, N % L);
                     }
                 } else {
-                    sum = march_shift<PERIODIC>(base, step, L, kc);
-                    if (PERIODIC && N != 0) rotate_line(base, step, L, N % L);
+                    sum = march_shift(base, step, L, kc);
+                    if (N != 0) rotate_line(base, step, L, N % L);
                 }
                 if (!(sum >= C(0)) || isinf(sum)) atomicOr(args.err, ERR_NAN);
             }
@@ -160,7 +154,7 @@ template <typename T>
 static cudaError_t launch_strided_t(const CUtensorMap &map, const CUtensorMap &dmap, const StridedArgs<typename Compute<T>::type> &a,
                                     int grid, size_t smem, cudaStream_t st)
 {
-    auto kern = a.periodic ? strided_sweep_kernel<T, true> : strided_sweep_kernel<T, false>;
+    auto kern = strided_sweep_kernel<T>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     kern<<<grid, kConsumers + kProducer, smem, st>>>(map, dmap, a);
@@ -179,13 +173,9 @@ cudaError_t launch_strided_f64(const CUtensorMap &map, const CUtensorMap &dmap, 
     return launch_strided_t<double>(map, dmap, a, grid, smem, st);
 }
 
-int occupancy_strided(int dtype, int periodic, size_t smem)
+int occupancy_strided(int dtype, size_t smem)
 {
-    const void *k;
-    if (dtype == 0)
-        k = periodic ? (const void *)strided_sweep_kernel<double, true> : (const void *)strided_sweep_kernel<double, false>;
-    else
-        k = periodic ? (const void *)strided_sweep_kernel<float, true> : (const void *)strided_sweep_kernel<float, false>;
+    const void *k = dtype == 0 ? (const void *)strided_sweep_kernel<double> : (const void *)strided_sweep_kernel<float>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess) return 0;

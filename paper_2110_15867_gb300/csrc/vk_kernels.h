@@ -87,7 +87,7 @@ template <typename C> __host__ __device__ inline LineCoefT<C> make_line_coef(dou
 }
 
 // ----------------------------------------------------------------------------
-// strided sweep (axes x, y, z, u_x, u_y)
+// strided sweep (axes x, y, z; whole-cell shifts)
 // ----------------------------------------------------------------------------
 // f viewed as [O][L][I] (outer, swept, inner).  A tile is the TMA box
 // {W inner, L swept, P outer}; each consumer thread owns one (inner, outer)
@@ -95,16 +95,10 @@ template <typename C> __host__ __device__ inline LineCoefT<C> make_line_coef(dou
 template <typename C> struct StridedArgs {
     int L, W, P, stages;
     int tiles_inner;
-    int periodic;
     long long n_inner, n_outer;
     long long num_tiles;
-    // position sweeps: j = (inner / vstride) % nvel indexes table
-    long long vstride;
+    long long vstride; // j = (inner / vstride) % nvel indexes table
     int nvel;
-    int coef_mode; // 0 = position table, 1 = per-cell array
-    // velocity sweeps: cell = outer / outer_per_cell indexes cell_coef
-    long long outer_per_cell;
-    const LineCoefT<C> *cell_coef;
     unsigned *err;
     LineCoefT<C> table[kMaxVel];
 };
@@ -375,7 +369,7 @@ cudaError_t launch_rows_sweep(const void *src, void *dst, const RowsArgs &a, int
 bool reg_lines_supported(int L);
 // dtype: 1 f32, 2 bf16, 3 f16
 cudaError_t launch_reg_lines(const void *src, void *dst, const RegLineArgs &a, int dtype, cudaStream_t st);
-int occupancy_strided(int dtype, int periodic, size_t smem);
+int occupancy_strided(int dtype, size_t smem);
 int occupancy_contig(size_t smem);
 cudaError_t launch_line_sweep(const CUtensorMap &map, const CUtensorMap &dmap, const ContigArgs<float> &a, int nu,
                               int dtype, int grid, cudaStream_t st, bool fuse_y = false);

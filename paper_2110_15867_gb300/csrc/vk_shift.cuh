@@ -44,25 +44,18 @@ __device__ __forceinline__ X cell_flux(const CellCoef<X> &k, X cm2, X cm1, X c0,
     const X v = mn3(mx3(fbar, mn3(c0, cp1, fmd), mn3(c0, ful, flc)), mx3(c0, cp1, fmd), mx3(c0, ful, flc));
     return flux_clamp(vmul(k.s, v), c0);
 }
-template <bool PERIODIC>
+// periodic line in place
 __device__ __forceinline__ float march_shift(float *p, long step, int L, const LineCoefT<float> &kc)
 {
     const CellCoef<float> k = to_cell(kc);
-    auto curv = [](float a, float b, float c) { return cell_curv(a, b, c); };
-    const float s0 = p[0], s1 = p[step];
-    float cm2 = 0.f, cm1 = 0.f, c0 = s0, cp1 = s1, d = curv(0.f, s0, s1), q = minmod_curv(s0, d), Fm = 0.f, sum = 0.f;
-    if (PERIODIC) {
-        const float a = p[(long)(L - 3) * step];
-        cm2 = p[(long)(L - 2) * step];
-        cm1 = p[(long)(L - 1) * step];
-        const float dm = curv(cm2, cm1, s0);
-        d = curv(cm1, s0, s1);
-        q = minmod_curv(dm, d);
-        Fm = cell_flux(k, a, cm2, cm1, s0, s1, minmod_curv(curv(a, cm2, cm1), dm), q); // face -1/2, donor c_{-1}
-    }
-    auto face = [&](int i, float cp2, bool outer) {
-        const float dn = curv(c0, cp1, cp2), qp = minmod_curv(d, dn);
-        const float F = outer ? 0.f : cell_flux(k, cm2, cm1, c0, cp1, cp2, q, qp);
+    const float s0 = p[0], s1 = p[step], a = p[(long)(L - 3) * step];
+    float cm2 = p[(long)(L - 2) * step], cm1 = p[(long)(L - 1) * step], c0 = s0, cp1 = s1, sum = 0.f;
+    const float dm = cell_curv(cm2, cm1, s0);
+    float d = cell_curv(cm1, s0, s1), q = minmod_curv(dm, d);
+    float Fm = cell_flux(k, a, cm2, cm1, s0, s1, minmod_curv(cell_curv(a, cm2, cm1), dm), q); // face -1/2, donor c_{-1}
+    auto face = [&](int i, float cp2) {
+        const float dn = cell_curv(c0, cp1, cp2), qp = minmod_curv(d, dn);
+        const float F = cell_flux(k, cm2, cm1, c0, cp1, cp2, q, qp);
         const float out = c0 + (Fm - F);
         p[(long)i * step] = out;
         sum += out;
@@ -75,12 +68,12 @@ __device__ __forceinline__ float march_shift(float *p, long step, int L, const L
         Fm = F;
     };
 #pragma unroll 4
-    for (int i = 0; i < L - 2; ++i) face(i, p[(long)(i + 2) * step], false);
-    face(L - 2, PERIODIC ? s0 : 0.f, false);
-    face(L - 1, PERIODIC ? s1 : 0.f, !PERIODIC);
+    for (int i = 0; i < L - 2; ++i) face(i, p[(long)(i + 2) * step]);
+    face(L - 2, s0);
+    face(L - 1, s1);
     return sum;
 }
-// The same on a periodic line, walked from its last cell down, with every new value written N
+// The same walked from its last cell down, with every new value written N
 // cells on (0 <= N <= kStash, N < L): each row is read once and written once, where marching
 // in place and rotating the line afterwards (three reversals) read and wrote it three times.
 // Row i + N has been read when cell i is done; the N values that wrap around to the first

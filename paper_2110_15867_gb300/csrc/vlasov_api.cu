@@ -317,7 +317,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             p.smem = 128 + tab + (size_t)S * tile;
             p.spec = spec3(tmap_type(c->g.dtype), I, p.L, O, es, W, p.L, P);
             r = encode_spec(&p.map, p.spec, c->f);
-            const int occ = occupancy_strided(c->g.dtype == VLASOV_F64 ? 0 : 1, ax < 3, p.smem);
+            const int occ = occupancy_strided(c->g.dtype == VLASOV_F64 ? 0 : 1, p.smem);
             if (occ <= 0) return fail(c, VLASOV_ECUDA, "axis %d: a CTA does not fit (%zu B shared memory)", ax, p.smem);
             p.grid = int(p.num_tiles < (long long)occ * c->sm_count ? p.num_tiles : (long long)occ * c->sm_count);
         } else {
@@ -998,18 +998,18 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
     cudaError_t e;
     if (c->g.dtype == VLASOV_F64) {
         StridedArgs<double> A{};
-        A.L = p.L; A.W = p.W; A.P = p.P; A.stages = p.stages; A.tiles_inner = p.tiles_inner; A.periodic = 1;
+        A.L = p.L; A.W = p.W; A.P = p.P; A.stages = p.stages; A.tiles_inner = p.tiles_inner;
         A.n_inner = p.n_inner; A.n_outer = p.n_outer; A.num_tiles = p.num_tiles;
-        A.vstride = vstride; A.nvel = nvel; A.coef_mode = 0; A.outer_per_cell = 1; A.cell_coef = nullptr;
+        A.vstride = vstride; A.nvel = nvel;
         A.err = c->d_err;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<double>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
         PartTimer t(c, ax, 1);
         e = launch_strided_f64(m.in, m.out, A, p.grid, p.smem, c->stream);
     } else {
         StridedArgs<float> A{};
-        A.L = p.L; A.W = p.W; A.P = p.P; A.stages = p.stages; A.tiles_inner = p.tiles_inner; A.periodic = 1;
+        A.L = p.L; A.W = p.W; A.P = p.P; A.stages = p.stages; A.tiles_inner = p.tiles_inner;
         A.n_inner = p.n_inner; A.n_outer = p.n_outer; A.num_tiles = p.num_tiles;
-        A.vstride = vstride; A.nvel = nvel; A.coef_mode = 0; A.outer_per_cell = 1; A.cell_coef = nullptr;
+        A.vstride = vstride; A.nvel = nvel;
         A.err = c->d_err;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
         PartTimer t(c, ax, 1);

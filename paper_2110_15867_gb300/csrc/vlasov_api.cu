@@ -731,7 +731,7 @@ extern "C" int vlasov_set_f(vlasov_ctx *c, void *f_dev, float *scale_dev)
     return plan_axes(c); // re-encode the tensor maps for the new arrays
 }
 
-template <typename C> static void fill_stream_args(StreamArgs<C> &A, const vlasov_ctx *c, int ax)
+template <typename C> static int fill_stream_args(StreamArgs<C> &A, vlasov_ctx *c, int ax)
 {
     const AxisPlan &p = c->splan[ax];
     A.L = p.L; A.W = p.W; A.P = p.P; A.R = c->splan_R[ax]; A.stages = p.stages;
@@ -739,7 +739,8 @@ template <typename C> static void fill_stream_args(StreamArgs<C> &A, const vlaso
     A.n_inner = p.n_inner; A.n_outer = p.n_outer; A.num_blocks = p.num_tiles;
     A.tile0 = 0;
     if (c->slab_x1 > c->slab_x0) {
-        // the x-planes [slab_x0, slab_x1) are whole tiles (vlasov_step_host checks)
+        // the x-planes [slab_x0, slab_x1) are whole tiles (slab_count checks)
+        if (c->splan_tpp[ax] <= 0) return fail(c, VLASOV_EINVAL, "sweep %d: a streamed block spans x-planes, no x-slab", ax);
         A.tile0 = c->slab_x0 * c->splan_tpp[ax];
         A.num_blocks = (c->slab_x1 - c->slab_x0) * c->splan_tpp[ax];
     }
@@ -749,6 +750,7 @@ template <typename C> static void fill_stream_args(StreamArgs<C> &A, const vlaso
     A.seed = c->sweeps;
     A.scale_rank = c->scale_rank[ax];
     A.swidth = c->swidth[ax];
+    return VLASOV_OK;
 }
 
 // Tensor maps of one plan for a sweep that reads src and writes dst (both
@@ -779,7 +781,6 @@ static cudaError_t launch_stream_any(const vlasov_ctx *c, int ax, const StreamAr
 {
     const AxisPlan &sp = c->splan[ax];
     const int grid = stream_grid(c, ax, A.num_blocks);
-    if (grid <= 0) return cudaSuccess;
     switch (c->g.dtype) {
     case VLASOV_BF16: return launch_stream_bf16(sp.map, c->smap[ax], A, grid, sp.smem, c->stream);
     case VLASOV_F16: return launch_stream_f16(sp.map, c->smap[ax], A, grid, sp.smem, c->stream);
@@ -952,15 +953,15 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         cudaError_t e;
         if (c->g.dtype == VLASOV_F64) {
             StreamArgs<double> A{};
-            fill_stream_args(A, c, ax);
+            if ((rc = fill_stream_args(A, c, ax))) return rc;
             A.vstride = vstride; A.nvel = nvel; A.coef_mode = 0; A.outer_per_cell = 1; A.cell_coef = nullptr;
             for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<double>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
             if (fm) { A.mpart = c->d_mpart; A.cube = cube; A.nparts = moment_parts(c); }
             PartTimer t(c, ax, 1);
-            e = A.num_blocks > 0 ? launch_stream_f64(m.in, m.out, A, stream_grid(c, ax, A.num_blocks), sp.smem, c->stream) : cudaSuccess;
+            e = launch_stream_f64(m.in, m.out, A, stream_grid(c, ax, A.num_blocks), sp.smem, c->stream);
         } else {
             StreamArgs<float> A{};
-            fill_stream_args(A, c, ax);
+            if ((rc = fill_stream_args(A, c, ax))) return rc;
             A.vstride = vstride; A.nvel = nvel; A.coef_mode = 0; A.outer_per_cell = 1; A.cell_coef = nullptr;
             for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
             if (fm) { A.mpart = c->d_mpart; A.cube = cube; A.nparts = moment_parts(c); }
@@ -1042,6 +1043,22 @@ static bool use_reg_lines(const vlasov_ctx *c, int ax)
     // tiles u_x takes 16.6 ms in FP32 and 21.8 ms in BF16)
     if (L == 48 && ax == 3 && c->g.dtype == VLASOV_F32) return false;
     return reg_lines_supported(L);
+}
+
+// The kernel of a velocity sweep, asked by run_velocity and by slab_count alike.  Planes (FP32):
+// u_z wherever the u_z line kernel does not take it; u_y alone while its column pairs (n_uz / 2 of
+// a plane) keep at least a quarter of a block's threads busy (n_u = 16, 96, 32: 0.415 ms on planes,
+// 0.343 streamed; 24^3 cubes 0.352 against 0.416)
+static bool uy_on_planes(const vlasov_ctx *c)
+{
+    return c->g.dtype == VLASOV_F32 && !use_reg_lines(c, 4) && c->g.nuy <= 2 * c->g.nuz;
+}
+static bool uz_on_planes(const vlasov_ctx *c) { return c->g.dtype == VLASOV_F32 && !c->use_lines; }
+static bool streams(const vlasov_ctx *c, int ax) // u_x or u_y: the streamed kernel
+{
+    if (use_reg_lines(c, ax)) return false;
+    if (ax == 4) return !uy_on_planes(c);
+    return !(c->use_tiles && (c->tile_ok[3] || c->p32_ok[3]));
 }
 
 // the u_x sweep on staged tiles of [cell][u_x][u_y u_z] (zero-flux lines; each tile's
@@ -1134,12 +1151,7 @@ static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *
         if (e != cudaSuccess) return cuda_fail(c, e, "u_x tile sweep launch");
         return VLASOV_OK;
     }
-    // u_y alone on planes while its column pairs (n_uz / 2 of a plane) keep at least a quarter of a
-    // block's threads busy (n_u = 16, 96, 32: 0.415 ms on planes, 0.343 streamed; 24^3 cubes 0.352
-    // against 0.416)
-    if (c->g.dtype == VLASOV_F32 &&
-        ((ax == 4 && !use_reg_lines(c, 4) && c->g.nuy <= 2 * c->g.nuz) || (ax == 5 && !c->use_lines)))
-        return run_plane_any(c, ax == 4 ? 2 : 4, src, dst);
+    if ((ax == 4 && uy_on_planes(c)) || (ax == 5 && uz_on_planes(c))) return run_plane_any(c, ax == 4 ? 2 : 4, src, dst);
     const AxisPlan &p = c->plan[ax];
     const void *coef = c->d_coef[ax - 3];
     SweepMaps m;
@@ -1166,13 +1178,13 @@ static int run_velocity(vlasov_ctx *c, int ax, const void *src = nullptr, void *
         PartTimer t(c, ax, 1);
         if (c->g.dtype == VLASOV_F64) {
             StreamArgs<double> A{};
-            fill_stream_args(A, c, ax);
+            if ((rc = fill_stream_args(A, c, ax))) return rc;
             A.vstride = 1; A.nvel = 0; A.coef_mode = 1; A.outer_per_cell = opc;
             A.cell_coef = (const LineCoefT<double> *)coef;
-            e = A.num_blocks > 0 ? launch_stream_f64(m.in, m.out, A, stream_grid(c, ax, A.num_blocks), sp.smem, c->stream) : cudaSuccess;
+            e = launch_stream_f64(m.in, m.out, A, stream_grid(c, ax, A.num_blocks), sp.smem, c->stream);
         } else {
             StreamArgs<float> A{};
-            fill_stream_args(A, c, ax);
+            if ((rc = fill_stream_args(A, c, ax))) return rc;
             A.vstride = 1; A.nvel = 0; A.coef_mode = 1; A.outer_per_cell = opc;
             A.cell_coef = (const LineCoefT<float> *)coef;
             e = launch_stream_any(c, ax, A, m);
@@ -1458,14 +1470,13 @@ static int slab_count(const vlasov_ctx *c, double dt, double a_half)
 {
     if (coded(c)) return 0; // the 16-bit encodes draw per-sweep random streams
     const bool cube = c->can_kick_cube && c->fuse_kick >= 2; // whole cubes: any x-slab
-    const bool fused = c->can_fuse_kick && c->fuse_kick >= 1;
-    const bool rows = rows_sweep_supported(int(c->g.nuz), c->g.dtype);
     if (!cube) {
-        const bool f32 = c->g.dtype == VLASOV_F32; // D_uy, D_uz on planes: any x-slab
-        if (f32 ? c->use_lines && c->ltpp <= 0 : !rows && (!c->use_lines || c->ltpp <= 0)) return 0;
-        if ((!use_reg_lines(c, 3) && c->splan_tpp[3] <= 0) ||
-            (!f32 && !fused && !use_reg_lines(c, 4) && c->splan_tpp[4] <= 0))
-            return 0;
+        // D_uz D_uy in one pass (run_kick): the line kernel's tail or planes
+        const bool tail = c->fuse_kick >= 1 && (c->can_fuse_kick || c->can_plane_tail || c->g.dtype == VLASOV_F32);
+        const bool rows = uz_on_planes(c) || rows_sweep_supported(int(c->g.nuz), c->g.dtype);
+        if (c->use_lines ? c->ltpp <= 0 : !rows) return 0;
+        if (streams(c, 3) && c->splan_tpp[3] <= 0) return 0;
+        if (!tail && streams(c, 4) && c->splan_tpp[4] <= 0) return 0;
     }
     for (int ax = 1; ax <= 2; ++ax)
         if (c->splan_tpp[ax] <= 0 || !(position_numax(c, ax, dt, a_half) < 1.0)) return 0;

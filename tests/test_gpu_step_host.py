@@ -72,6 +72,32 @@ def test_step_host_is_upload_step_download(n, nu, a_half, fused):
     assert ux_launches == (2 if a_half < 0.5 else 2 * min(16, n[0]))
 
 
+@pytest.mark.parametrize("n,nu,split", [
+    ((8, 5, 5), (8, 28, 12), (2, 1)),     # n_uy > 2 n_uz: u_y alone streams, blocks that span x-planes
+    ((16, 8, 8), (4, 28, 12), (2, 1)),    # the same
+    ((6, 7, 6), (8, 28, 12), (2, 1, 0)),  # u_y streams, whole blocks of 21 rows per x-plane
+    ((8, 6, 5), (24, 20, 28), (2, 1, 0)),  # u_y and u_z on planes, u_x on tiles
+])
+@pytest.mark.parametrize("fused", [2, 1, 0])
+def test_step_host_on_ragged_grids(n, nu, split, fused):
+    # grids that no fixed-size kernel takes: the slabs of the planes and of the tiles of any
+    # length, and the sweeps that cannot run on a slab (the step then falls back)
+    B = _lib()
+    f0 = I.initial_f(I.gaussian_field(n, 0.05, seed=7), I.fermi_dirac(nu, 5.0), np.float32)
+    phi0 = I.fourier_potential(n, seed=17).astype(np.float32)
+    bg = 3.0 * (1.0 + I.gaussian_field(n, 0.5, seed=8))
+    g = O.grid(n, nu, V=5.0)
+    p64 = phi0.astype(np.float64)
+    dt = min([1.4 / O.max_abs_nu(g, ax, 1.0, 1.0, p64) for ax in (3, 4, 5)] +
+             [0.7 / O.max_abs_nu(g, ax, 1.0, 0.55, p64) for ax in (0, 1, 2)])
+    ref, _ = _run(B, f0, phi0, bg, dt, 0.55, False, fused)
+    got, ux_launches = _run(B, f0, phi0, bg, dt, 0.55, True, fused)
+    for r, o in zip(ref, got):
+        assert np.array_equal(r, o)
+    slabs = max(s for s in range(1, 17) if n[0] % s == 0)
+    assert ux_launches == 2 * (slabs if fused in split else 1)
+
+
 def test_step_host_fp64_falls_back_to_the_three_calls():
     # FP64 storage has no line kernel to split per slab: the same result as upload + step
     # + download, through the sequential path

@@ -23,6 +23,8 @@ constexpr int kGroup = kCols / 2;            // threads of a group
 constexpr int kMaxGroups = 8, kMaxSlots = 24; // (11 groups, 80 registers: 0.347-0.350 ms, 16^3 x 32^3 0.257)
 constexpr int kHead = ((3 * kMaxSlots * 8 + 127) & ~127) + int(kMaxVel * sizeof(LineCoefT<float>));
 
+// ROT: lines marched in place one by one and rotated (Pair32Args::rotate)
+template <bool ROT>
 __global__ void __launch_bounds__(kMaxGroups *kGroup + kProducer, 1)
     shift32_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap dmap,
                   const __grid_constant__ Pair32Args a)
@@ -104,13 +106,12 @@ __global__ void __launch_bounds__(kMaxGroups *kGroup + kProducer, 1)
         if (ka.nd >= 0) {
             // a negative Courant number is the mirror image: march the line from its far end
             const bool neg = ka.nd & 1;
-            const int Na = (ka.nd >> 1) % L, Nb = (kb.nd >> 1) % L, step = neg ? -kGroup : kGroup; // rows in pairs
+            auto shift = [&](int N) { return N < L ? N : N % L; };
+            const int Na = shift(ka.nd >> 1), Nb = shift(kb.nd >> 1), step = neg ? -kGroup : kGroup; // rows in pairs
             float2 *p = reinterpret_cast<float2 *>(slot(k)) + tid + (neg ? (L - 1) * kGroup : 0);
             float2 sum;
             // (columns past the end of a row hold zeros: marched, never stored)
-            if (Na <= kStash && Nb <= kStash) {
-                sum = march_shift_down(p, step, L, Na, Nb, ka, kb);
-            } else {
+            if constexpr (ROT) {
                 auto line = [&](float *q, int N, const LineCoefT<float> &kc) {
                     const float s = march_shift(q, long(2 * step), L, kc);
                     rotate_line(q, long(2 * step), L, N);
@@ -118,6 +119,8 @@ __global__ void __launch_bounds__(kMaxGroups *kGroup + kProducer, 1)
                 };
                 sum.x = line(&p->x, Na, ka);
                 sum.y = line(&p->y, Nb, kb);
+            } else {
+                sum = march_shift_down(p, step, L, Na, Nb, ka, kb);
             }
             bad |= !(sum.x >= 0.f) || !(sum.y >= 0.f) || isinf(sum.x) || isinf(sum.y);
         }
@@ -142,10 +145,11 @@ cudaError_t launch_shift32(const CUtensorMap &map, const CUtensorMap &dmap, cons
     a.div_vstride = make_fastdiv(unsigned(a.vstride));
     a.div_nvel = make_fastdiv(unsigned(a.nvel));
     const size_t smem = kHead + 128 + size_t(a.slots) * a.L * kRow;
-    const cudaError_t e = cudaFuncSetAttribute(shift32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const void *kern = a.rotate ? (const void *)shift32_kernel<true> : (const void *)shift32_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
-    return launch_chained((long long)a.num_tiles * kCols * a.L, (const void *)shift32_kernel, dim3(grid),
+    return launch_chained((long long)a.num_tiles * kCols * a.L, kern, dim3(grid),
                           dim3(a.groups * kGroup + kProducer), smem, st, params);
 }
 

@@ -30,7 +30,9 @@ __device__ __forceinline__ double march_shift(double *p, long step, int L, const
     return march_line<double, true, double>(p, step, L, to_lim(k));
 }
 
-template <typename T>
+// ROT: lines marched in place and rotated (FP64, and FP32 with StridedArgs::rotate), else
+// walked down, every cell written in its shifted place
+template <typename T, bool ROT>
 __global__ void __launch_bounds__(kConsumers + kProducer)
     strided_sweep_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap dmap,
                          const __grid_constant__ StridedArgs<typename Compute<T>::type> args)
@@ -122,25 +124,27 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
         const long long t = b + k * G;
         const long long inner = (t % args.tiles_inner) * W + w;
         const long long outer = (t / args.tiles_inner) * P + p;
+        auto coef = [&]() { return tab[(inner / args.vstride) % args.nvel]; };
+        // a warp whose lines all stay in place marches them so (10^2 x 16 x 32^3 cells, |nu| up to 1.3,
+        // x sweep: 159 us all walked down, 148 here)
+        bool moves = true;
+        if constexpr (!ROT) moves = __any_sync(0xffffffffu, coef().nd >> 1 != 0);
         if (has_col && inner < args.n_inner && outer < args.n_outer) {
-            const LineCoefT<C> kc = tab[(inner / args.vstride) % args.nvel];
+            const LineCoefT<C> kc = coef();
             if (kc.nd >= 0) {
-                const int N = kc.nd >> 1;
+                const int N = kc.nd >> 1, r = N < L ? N : N % L; // (a division by L costs 3 % of a short line)
                 const bool neg = kc.nd & 1;
                 T *col = stage0 + size_t(st) * stage_elems + size_t(p) * L * W + w;
                 T *base = neg ? col + size_t(L - 1) * W : col;
                 const long step = neg ? -long(W) : long(W);
                 C sum;
-                if constexpr (sizeof(T) == 4) {
-                    if (N % L <= kStash && N % L < L) {
-                        sum = march_shift_down(base, int(step), L, N % L, kc);
-                    } else {
-                        sum = march_shift(base, step, L, kc);
-                        rotate_line(base, step, L, N % L);
-                    }
-                } else {
+                if constexpr (ROT) {
                     sum = march_shift(base, step, L, kc);
-                    if (N != 0) rotate_line(base, step, L, N % L);
+                    rotate_line(base, step, L, r);
+                } else if (!moves) {
+                    sum = march_shift(base, step, L, kc);
+                } else {
+                    sum = march_shift_down(base, int(step), L, r, kc);
                 }
                 if (!(sum >= C(0)) || isinf(sum)) atomicOr(args.err, ERR_NAN);
             }
@@ -150,11 +154,11 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
     }
 }
 
-template <typename T>
+template <typename T, bool ROT>
 static cudaError_t launch_strided_t(const CUtensorMap &map, const CUtensorMap &dmap, const StridedArgs<typename Compute<T>::type> &a,
                                     int grid, size_t smem, cudaStream_t st)
 {
-    auto kern = strided_sweep_kernel<T>;
+    auto kern = strided_sweep_kernel<T, ROT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     kern<<<grid, kConsumers + kProducer, smem, st>>>(map, dmap, a);
@@ -164,22 +168,28 @@ static cudaError_t launch_strided_t(const CUtensorMap &map, const CUtensorMap &d
 cudaError_t launch_strided_f32(const CUtensorMap &map, const CUtensorMap &dmap, const StridedArgs<float> &a, int grid, size_t smem,
                                cudaStream_t st)
 {
-    return launch_strided_t<float>(map, dmap, a, grid, smem, st);
+    return a.rotate ? launch_strided_t<float, true>(map, dmap, a, grid, smem, st)
+                    : launch_strided_t<float, false>(map, dmap, a, grid, smem, st);
 }
 
 cudaError_t launch_strided_f64(const CUtensorMap &map, const CUtensorMap &dmap, const StridedArgs<double> &a, int grid, size_t smem,
                                cudaStream_t st)
 {
-    return launch_strided_t<double>(map, dmap, a, grid, smem, st);
+    return launch_strided_t<double, true>(map, dmap, a, grid, smem, st);
 }
 
-int occupancy_strided(int dtype, size_t smem)
+int occupancy_strided(int dtype, size_t smem) // of the kernel that fits fewer CTAs
 {
-    const void *k = dtype == 0 ? (const void *)strided_sweep_kernel<double> : (const void *)strided_sweep_kernel<float>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess) return 0;
-    return n;
+    auto fit = [&](const void *k) {
+        int n = 0;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess)
+            return 0;
+        return n;
+    };
+    if (dtype == 0) return fit((const void *)strided_sweep_kernel<double, true>);
+    const int rot = fit((const void *)strided_sweep_kernel<float, true>), walk = fit((const void *)strided_sweep_kernel<float, false>);
+    return rot < walk ? rot : walk;
 }
 
 } // namespace vk

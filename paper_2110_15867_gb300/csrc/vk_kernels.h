@@ -99,9 +99,23 @@ template <typename C> struct StridedArgs {
     long long num_tiles;
     long long vstride; // j = (inner / vstride) % nvel indexes table
     int nvel;
+    int rotate; // FP32: lines marched in place and rotated, else walked down (whole_cell_rotate)
     unsigned *err;
     LineCoefT<C> table[kMaxVel];
 };
+// The values of a line that a thread holds back while it walks the line down and writes every
+// cell in its shifted place (vk_shift.cuh).
+constexpr int kStash = 8;
+// Does some line shift by more cells than a thread can hold back?  All lines of the sweep are
+// then marched in place and rotated: the choice is the sweep's, since a warp whose lines chose
+// each for itself ran both (64 x 24^2 x 16^2 x 12 cells, |nu| up to 12, z sweep: 488 us, 253 with
+// one choice; 278 one line per thread).
+template <typename C> inline bool whole_cell_rotate(const LineCoefT<C> *table, int nvel, int L)
+{
+    for (int j = 0; j < nvel; ++j)
+        if ((table[j].nd >> 1) % L > kStash) return true;
+    return false;
+}
 
 // ----------------------------------------------------------------------------
 // streamed strided sweep (axes x, y, z, u_x, u_y with |nu| < 1): a block of
@@ -285,6 +299,7 @@ struct Pair32Args {
     unsigned *err;
     const LineCoefT<float> *cell_coef; // u_x sweep: the Courant numbers per outer index (a cell), else null
     FastDivU32 div_tiles, div_vstride, div_nvel; // set by the launcher
+    bool rotate;                       // whole-cell shifts: whole_cell_rotate
     LineCoefT<float> table[kMaxVel];
 };
 int pair32_columns();

@@ -78,11 +78,8 @@ __device__ __forceinline__ float march_shift(float *p, long step, int L, const L
 // in place and rotating the line afterwards (three reversals) read and wrote it three times.
 // Row i + N has been read when cell i is done; the N values that wrap around to the first
 // rows, still to be read, wait in `held`, and the last three cells, overwritten before the
-// first ones need them, in registers.  The values are march_shift's, face by face.  With tiles
-// small enough for three CTAs per SM: 32 x 24 x 32 x 16 x 16 x 32 cells, x, y, z 0.600, 0.430, 0.643 ->
-// 0.39 ms each (DRAM alone 0.238).
+// first ones need them, in registers.  The values are march_shift's, face by face.
 // The values are what one line alone gives, and a pair's lines may shift by different N.
-constexpr int kStash = 8;
 template <typename X> struct ShiftPut;
 template <> struct ShiftPut<float> { // where the next cell down goes; past the line's end it wraps to row to - L
     int to;

@@ -989,6 +989,7 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         A.vstride = vstride;
         A.nvel = nvel;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
+        A.rotate = whole_cell_rotate(A.table, nvel, p.L);
         if ((rc = sweep_maps(c, c->pmap[ax], c->pspec[ax], src, dst, m))) return rc;
         PartTimer t(c, ax, 1);
         const cudaError_t e = launch_shift32(m.in, m.out, A, pair32_grid(c, ax, A), c->stream);
@@ -1013,6 +1014,7 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         A.vstride = vstride; A.nvel = nvel;
         A.err = c->d_err;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
+        A.rotate = whole_cell_rotate(A.table, nvel, p.L);
         PartTimer t(c, ax, 1);
         e = launch_strided_f32(m.in, m.out, A, p.grid, p.smem, c->stream);
     }

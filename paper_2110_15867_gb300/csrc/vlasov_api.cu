@@ -296,25 +296,35 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         p.n_outer = O;
         CUresult r;
         if (ax < 5) {
-            int W, P;
-            if (I >= kConsumers) { W = kConsumers; P = 1; }
-            else { W = int(I); P = kConsumers / W; if (P > O) P = int(O); }
-            // tiles and rings small enough for three CTAs per SM: a CTA's 8 warps march one tile
-            // and wait for each other, so one CTA (4 stages of 32 KB) left an SM's latency bare
-            while ((size_t)W * p.L * P * es > 36 * 1024 && W * P > 32) {
-                if (P > 1) P = (P + 1) / 2;
-                else W /= 2;
+            // A tile of W x P lines, one per consumer thread, in a ring of 2 to 4.  The tile that lets an
+            // SM march most lines at a time is taken (of equal ones the largest, whose lines
+            // spread over more warps): CTAs an SM by shared memory, at most by registers, times
+            // lines.  Against the most lines in one CTA (FP32 32^3 x 16^3, lines of 32: x 426 us, 269
+            // here; 112 x 16 x 200 x 8^2 x 12, lines of 200: 2258, 886; FP64 lines of 200: 41.6 ms,
+            // 20.9) and tiles of at most 36 KB (FP64 64 x 48 x 24 x 12^2 x 16, lines of 48: 7.24 ms,
+            // 5.43; FP32 200 x 120 x 160 x 4^3, lines of 160: 1399, 1052 us).
+            const size_t tab = ax < 3 ? ((sizeof(LineCoefT<double>) * kMaxVel + 127) & ~size_t(127)) : 0;
+            int W = 0, P = 0, S = 0;
+            for (int lines = kConsumers, best = 0; lines >= 32; lines /= 2) {
+                const int w = I < lines ? int(I) : lines;
+                const int q = lines / w < O ? lines / w : int(O);
+                const size_t tile = ((size_t)w * p.L * q * es + 127) & ~size_t(127);
+                auto cta = [&](int stages) { return 128 + tab + stages * tile; }; // shared memory, 1 KB more on the SM
+                if (cta(2) > 227 * 1024) continue;
+                const int regs = es == 8 ? 2 : 4, fit = int(228 * 1024 / (cta(2) + 1024)), n = fit < regs ? fit : regs;
+                if (n * w * q <= best) continue;
+                best = n * w * q;
+                W = w;
+                P = q;
+                for (S = 2; S < 4 && (cta(S + 1) + 1024) * n <= 228 * 1024;) ++S;
             }
+            if (!W) return fail(c, VLASOV_ECUDA, "axis %d: no tile fits shared memory", ax);
             p.W = W;
             p.P = P;
             p.tiles_inner = int((I + W - 1) / W);
             p.num_tiles = (long long)p.tiles_inner * ((O + P - 1) / P);
-            const size_t tile = ((size_t)W * p.L * P * es + 127) & ~size_t(127);
-            const size_t tab = ax < 3 ? ((sizeof(LineCoefT<double>) * kMaxVel + 127) & ~size_t(127)) : 0;
-            int S = int((76 * 1024 - 128 - tab) / tile);
-            S = S < 2 ? 2 : (S > 4 ? 4 : S);
             p.stages = S;
-            p.smem = 128 + tab + (size_t)S * tile;
+            p.smem = 128 + tab + S * (((size_t)W * p.L * P * es + 127) & ~size_t(127));
             p.spec = spec3(tmap_type(c->g.dtype), I, p.L, O, es, W, p.L, P);
             r = encode_spec(&p.map, p.spec, c->f);
             const int occ = occupancy_strided(c->g.dtype == VLASOV_F64 ? 0 : 1, p.smem);

@@ -1,6 +1,6 @@
 // sweep_pair32.cu -- position sweeps D_x, D_y, D_z of Eq. (3) (|nu| < 1) and the u_x sweep of
-// Eq. (4) on FP32 storage for lines of any length, whole lines staged in shared memory, two
-// lines per thread.
+// Eq. (4) on FP32 storage for lines of any length (from 9 cells; shorter ones mostly stream),
+// whole lines staged in shared memory, two lines per thread.
 //
 // f is viewed as [O][L][I] (slower axes, the swept axis, the faster axes; for u_x: cells,
 // j_x, j_y j_z) and I cut into tiles of 128 contiguous columns, the last one of a row partial

@@ -141,7 +141,7 @@ struct vlasov_ctx {
     MapSpec tspec[4];
     int tgrid[4];
     Tile16Args t16[4]; // 16-bit storage: the sizes of the tiles
-    // FP32: staged tiles for lines of any length, where tile_ok has none
+    // FP32: staged tiles for lines of any length from 9 cells, where tile_ok has none
     bool p32_ok[4];
     Pair32Args p32[4];
     CUtensorMap pmap[4];
@@ -494,7 +494,13 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             if (encode_spec(&c->tsmap[ax], ss, c->scale) != CUDA_SUCCESS) continue;
             occ = occupancy_tile16(c->t16[ax], c->g.dtype, ax == 3);
         } else {
-            if (I >= pair32_columns() && pair32_geometry(L, I, O, c->p32[ax])) {
+            // Lines of up to 8 cells stream: a tile of them is a few KB, and its barriers and copies
+            // outweigh its marches (16^3 velocity cubes, tiles / streamed: 4 cells 547 / 357 us, 6
+            // 379 / 304, 8 298 / 280, 9 273 / 272, 12 217 / 233; u_x of 8 x 16^2 292 / 263, of 12 x 16^2
+            // 206 / 212).  But y lines whose runs of one sign of u_y are shorter than a warp's 64
+            // columns make streamed warps march both ways (8^3 cubes: 4 cells 547 / 592, 8 303 / 498).
+            const bool mixed = ax == 1 && d6[4] * d6[5] / 2 < 64;
+            if (I >= pair32_columns() && (L > 8 || mixed) && pair32_geometry(L, I, O, c->p32[ax])) {
                 c->pspec[ax] = spec3(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, I, L, O, 4, pair32_columns(), L, 1);
                 const int n = occupancy_pair32(c->p32[ax], ax == 3);
                 if (n > 0 && encode_spec(&c->pmap[ax], c->pspec[ax], c->f) == CUDA_SUCCESS) {
@@ -834,7 +840,7 @@ static bool fused_moment_ok(vlasov_ctx *c, int ax)
     return moment_buffer(c);
 }
 
-// the tiles of the current x-slab (all when none is set) on the FP32 tiles of any length
+// the tiles of the current x-slab (all when none is set) on the FP32 pair tiles
 static void pair32_tiles(const vlasov_ctx *c, int ax, Pair32Args &A)
 {
     const long long all = c->pn_outer[ax] * A.tiles_inner;

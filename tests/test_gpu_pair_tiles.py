@@ -12,7 +12,8 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 SHAPES = [((4, 5, 6), (8, 12, 20)), ((7, 9, 10), (12, 8, 12)), ((11, 13, 4), (20, 12, 4)), ((32, 6, 33), (8, 8, 8)),
-          ((5, 47, 4), (24, 4, 28)), ((100, 4, 4), (8, 4, 12)), ((4, 4, 90), (40, 12, 12)), ((9, 8, 8), (128, 12, 12))]
+          ((5, 47, 4), (24, 4, 28)), ((100, 4, 4), (8, 4, 12)), ((4, 4, 90), (40, 12, 12)), ((9, 8, 8), (128, 12, 12)),
+          ((5, 4, 9), (8, 8, 12)), ((8, 7, 10), (16, 8, 12))]  # y lines of 4 and 7 with both signs in a warp
 
 
 @pytest.mark.parametrize("n,nu", SHAPES)

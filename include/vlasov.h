@@ -148,8 +148,9 @@ int vlasov_decode(long long nlines, int nuz, const void *codes_dev, int code_dty
  *     shared memory and only D_uz's is encoded); and with n_uy = n_uz = 48 (n_ux a
  *     multiple of 4), over four staged (cell, j_x) planes per block (FP32: the
  *     separate sweeps bit for bit; 16-bit: decoded as staged, encoded once after
- *     D_uz with refreshed line scales).  FP32 grids of other velocity sizes run D_uy
- *     and D_uz in one pass over staged planes too (the separate sweeps bit for bit).
+ *     D_uz with refreshed line scales).  FP32 grids of other velocity sizes with
+ *     n_uy up to 4 n_uz run D_uy and D_uz in one pass over staged planes too (the
+ *     separate sweeps bit for bit).
  *   mode 0: three separate sweeps.
  * FP64 storage always runs the sweeps separately.  Errors: VLASOV_EINVAL for
  * another mode.

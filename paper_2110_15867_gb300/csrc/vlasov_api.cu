@@ -1072,6 +1072,13 @@ static bool uy_on_planes(const vlasov_ctx *c)
     return c->g.dtype == VLASOV_F32 && !use_reg_lines(c, 4) && c->g.nuy <= 2 * c->g.nuz;
 }
 static bool uz_on_planes(const vlasov_ctx *c) { return c->g.dtype == VLASOV_F32 && !c->use_lines; }
+// D_uz D_uy of a kick in one pass over planes, up to n_uy = 4 n_uz: beyond that the column pairs
+// (n_uz / 2 of a plane, which D_uy marches) leave most of a block idle (one pass / two: n_u = 16, 64, 16
+// 587 / 568 us, 20, 36, 8 735 / 773, 16, 48, 8 732 / 706, 16, 32, 4 951 / 802, 8, 100, 4 2001 / 1156)
+static bool tail_on_planes(const vlasov_ctx *c)
+{
+    return c->g.dtype == VLASOV_F32 && c->fuse_kick >= 1 && c->g.nuy <= 4 * c->g.nuz;
+}
 static bool streams(const vlasov_ctx *c, int ax) // u_x or u_y: the streamed kernel
 {
     if (use_reg_lines(c, ax)) return false;
@@ -1402,7 +1409,7 @@ static int run_kick(vlasov_ctx *c)
     if ((rc = run_velocity(c, 3))) return rc;
     if (c->can_fuse_kick && c->fuse_kick >= 1) return run_kick_tail(c);
     if (c->can_plane_tail && c->fuse_kick >= 1) return run_plane_tail(c);
-    if (c->g.dtype == VLASOV_F32 && c->fuse_kick >= 1) {
+    if (tail_on_planes(c)) {
         c->sweeps += 2;
         return run_plane_any(c, 6, c->f, c->f);
     }
@@ -1490,7 +1497,7 @@ static int slab_count(const vlasov_ctx *c, double dt, double a_half)
     const bool cube = c->can_kick_cube && c->fuse_kick >= 2; // whole cubes: any x-slab
     if (!cube) {
         // D_uz D_uy in one pass (run_kick): the line kernel's tail or planes
-        const bool tail = c->fuse_kick >= 1 && (c->can_fuse_kick || c->can_plane_tail || c->g.dtype == VLASOV_F32);
+        const bool tail = (c->fuse_kick >= 1 && (c->can_fuse_kick || c->can_plane_tail)) || tail_on_planes(c);
         const bool rows = uz_on_planes(c) || rows_sweep_supported(int(c->g.nuz), c->g.dtype);
         if (c->use_lines ? c->ltpp <= 0 : !rows) return 0;
         if (streams(c, 3) && c->splan_tpp[3] <= 0) return 0;

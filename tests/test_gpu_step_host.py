@@ -76,6 +76,7 @@ def test_step_host_is_upload_step_download(n, nu, a_half, fused):
     ((8, 5, 5), (8, 28, 12), (2, 1)),     # n_uy > 2 n_uz: u_y alone streams, blocks that span x-planes
     ((16, 8, 8), (4, 28, 12), (2, 1)),    # the same
     ((6, 7, 6), (8, 28, 12), (2, 1, 0)),  # u_y streams, whole blocks of 21 rows per x-plane
+    ((8, 5, 5), (8, 36, 8), ()),          # n_uy > 4 n_uz: no pass over planes in any mode
     ((8, 6, 5), (24, 20, 28), (2, 1, 0)),  # u_y and u_z on planes, u_x on tiles
 ])
 @pytest.mark.parametrize("fused", [2, 1, 0])

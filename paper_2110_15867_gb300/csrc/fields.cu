@@ -665,6 +665,11 @@ cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const do
     A.phi = phi;
     A.phi64 = phi64;
     cudaError_t err = cudaSuccess;
+    // Chained only up to 2^13 spatial cells (and kChainCells in all): more blocks than one per SM
+    // or so, and those of the next launch sit on the SMs while FP64 sums still run (chained /
+    // not: 6^3 22 / 35 us, 53 x 6^2 46 / 60, 21 x 26 x 19 51 / 49, 59 x 30 x 8 77 / 68, 32^3 99 / 65,
+    // 31 x 37 x 43 531 / 188).
+    const long long cells = n <= 8192 ? n * g.nu[0] * g.nu[1] * g.nu[2] : kChainCells + 1;
     auto dft = [&](auto kernel, int d, int sign, const double2 *in, double2 *out) {
         const int nd = g.n[d]; // <= 256
         A.nlines = unsigned(n / nd);
@@ -678,7 +683,7 @@ cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const do
         A.in = in;
         A.out = out;
         A.tw = ps.tw[d];
-        const cudaError_t e = launch_chained_t(n * g.nu[0] * g.nu[1] * g.nu[2], kernel, dim3((A.nlines + A.lines - 1) / A.lines), dim3(A.lines * nd),
+        const cudaError_t e = launch_chained_t(cells, kernel, dim3((A.nlines + A.lines - 1) / A.lines), dim3(A.lines * nd),
                                                (2 * A.lines + 1) * nd * sizeof(double2), st, A);
         if (err == cudaSuccess) err = e;
     };

@@ -358,20 +358,16 @@ template <int NU, typename T> struct PairCube16 {
 // The rounding stream of a line draws for its cells in memory order (j_x = 0 first), as the
 // u_x register-line kernel does; a line walked from its far end takes the same draws
 // backward: the generator x -> a x + c run in reverse, from the state after NU + 1 steps.
-constexpr unsigned kLcgA = 1664525u, kLcgC = 1013904223u;
-constexpr unsigned kLcgInv = 4276115653u; // a kLcgInv = 1 mod 2^32
-static_assert(kLcgA * kLcgInv == 1u, "inverse of the generator's multiplier");
 template <bool NEG> __device__ __forceinline__ unsigned draw16(unsigned &x)
 {
-    x = NEG ? x * kLcgInv - kLcgC * kLcgInv : x * kLcgA + kLcgC;
+    constexpr Lcg step = NEG ? kLcgBack : kLcg;
+    x = step(x);
     return x >> 16;
 }
-constexpr unsigned lcg_pow(int n) { return n ? kLcgA * lcg_pow(n - 1) : 1u; }
-constexpr unsigned lcg_add(int n) { return n ? kLcgA * lcg_add(n - 1) + kLcgC : 0u; }
 template <int NU, bool NEG> __device__ __forceinline__ unsigned draw_start(unsigned seed)
 {
-    constexpr unsigned A = lcg_pow(NU + 1), C = lcg_add(NU + 1);
-    return NEG ? seed * A + C : seed;
+    constexpr Lcg end = lcg_power(kLcg, NU + 1);
+    return NEG ? end(seed) : seed;
 }
 
 // value pair -> what the codes it is stochastically rounded to (bx, by: 16 random bits) decode to

@@ -13,7 +13,7 @@
 // sign of their Courant number: one 4-byte access, one scale and one inverse scale serve
 // two cells, and the march's sums and products run as f32x2 pairs (March<float2>).  Groups
 // of 128 threads march different tiles of a ring that one producer thread keeps full.  The
-// length of the lines and the length of a u_z line are run-time values: bodies of 8, 4, 2
+// length of the lines and the length of a u_z line are run-time values: bodies of 4, 2
 // and 1 faces serve every shape and stay small (unrolled bodies that grow past the
 // instruction cache cost far more than the loop).  The codes and scales of a body are read
 // ahead of its marches, since the compiler cannot tell a row read from a row written.
@@ -34,16 +34,29 @@ namespace {
 constexpr int kPairGroup = 128; // threads of a group: the pairs of a tile
 constexpr int kPairGroups = 4;
 
+// The draws of two columns, 16 bits a value: the upper halves of two states, a step on per row.
+struct PairDraws {
+    unsigned x, y;
+    Lcg step;
+    __device__ void next()
+    {
+        x = step(x);
+        y = step(y);
+    }
+};
+
 template <typename T> struct PairCodec;
 template <> struct PairCodec<__nv_bfloat16> {
     __device__ static float2 get(unsigned u, float s) // a bf16 is the upper half of an FP32
     {
         return vmul(make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)), make_float2(s, s));
     }
-    __device__ static unsigned put(float2 v, float inv, unsigned &rng)
+    __device__ static unsigned put(float2 v, float inv, PairDraws &r)
     {
         const float2 c = vmul(v, make_float2(inv, inv));
-        return sr_pack_bf16x2(c.x, c.y, rng);
+        const unsigned u = sr_pack_bf16x2(c.x, c.y, r.x >> 16, r.y >> 16);
+        r.next();
+        return u;
     }
 };
 template <> struct PairCodec<__half> {
@@ -51,10 +64,12 @@ template <> struct PairCodec<__half> {
     {
         return vmul(__half22float2(*reinterpret_cast<const __half2 *>(&u)), make_float2(s, s));
     }
-    __device__ static unsigned put(float2 v, float inv, unsigned &rng)
+    __device__ static unsigned put(float2 v, float inv, PairDraws &r)
     {
         const float2 c = vmul(v, make_float2(inv, inv));
-        return sr_pack_f16x2(c.x, c.y, rng);
+        const unsigned u = sr_pack_f16x2(c.x, c.y, r.x >> 16, r.y >> 16);
+        r.next();
+        return u;
     }
 };
 
@@ -64,7 +79,7 @@ template <> struct PairCodec<__half> {
 // Returns the sums of the new values.
 template <typename T, bool ZF, int DIR>
 __device__ __forceinline__ float2 march_pair16(unsigned char *p, int st_rt, const float2 *sp, int sd_rt, int L,
-                                               const Lim<float2> &lim, unsigned rng)
+                                               const Lim<float2> &lim, PairDraws rng)
 {
     const int st = DIR ? DIR * 512 : st_rt, sd = DIR ? DIR : sd_rt;
     auto code = [&](int r) -> unsigned & { return *reinterpret_cast<unsigned *>(p + r * st); };
@@ -213,8 +228,10 @@ __global__ void __launch_bounds__(kPairGroups *kPairGroup + kProducer, 1)
             // a negative Courant number is the mirror image: march the line from its far end
             const bool neg = ka.nd & 1;
             const int far = neg ? L - 1 : 0, dir = neg ? -1 : 1;
-            // the pair's stream, from the index of its first cell
-            const unsigned rng = sr_bits((unsigned long long)o * L * a.n_inner + inner, a.seed);
+            // the streams, from the index of the first cell of the pair or of each column
+            const unsigned long long e = (unsigned long long)o * L * a.n_inner + inner;
+            const unsigned seed = sr_bits(e, a.seed);
+            const PairDraws rng{a.draws[neg].x(seed), a.draws[neg].y(a.own ? sr_bits(e + 1, a.seed) : seed), a.draws[neg].step};
             unsigned char *p = slot(k) + 4 * pair + far * 512;
             const float2 *s = ws + int(line - first) * L + far;
             float2 sum;
@@ -284,6 +301,24 @@ int occupancy_tile16(const Tile16Args &a, int dtype, bool zf)
     return n;
 }
 
+// Which streams a shape draws: those it has always drawn, whichever kernel took it.  16-bit results
+// then repeat but for the last bit of the FP32 march.
+//   own, walk order: one stream per column, a draw per cell as the line is walked (position lines of
+//     16 to 96 cells with n_uz = 32, lines of 48 with n_uz = 48);
+//   own, memory order: the same from the line's first cell on (u_x lines of 48 with other n_uz, as
+//     the register-line kernel);
+//   pair, memory order: one stream per two columns (all others: the streamed sweep's bits).
+// A line walked against memory order takes its draws backward.
+static void set_draws(Tile16Args &a, bool zf)
+{
+    const int L = a.L;
+    const bool walk = a.nuz == 48 ? L == 48 : !zf && a.nuz == 32 && (L == 16 || L == 24 || L == 32 || L == 48 || L == 64 || L == 96);
+    a.own = walk || (zf && L == 48);
+    const int n = a.own ? 1 : 2; // draws of a stream per row
+    a.draws[0] = a.draws[1] = {kLcg, lcg_power(kLcg, n), lcg_power(kLcg, n)};
+    if (!walk) a.draws[1] = {lcg_power(kLcg, n * (L - 1) + 1), lcg_power(kLcg, n * L), lcg_power(kLcgBack, n)};
+}
+
 cudaError_t launch_tile16(const CUtensorMap &map, const CUtensorMap &smap, const Tile16Args &args, int dtype, int grid,
                           cudaStream_t st)
 {
@@ -299,6 +334,7 @@ cudaError_t launch_tile16(const CUtensorMap &map, const CUtensorMap &smap, const
     a.div_nuz = make_fastdiv(unsigned(a.nuz));
     a.div_vstride = make_fastdiv(unsigned(a.vstride > 0 ? a.vstride : 1));
     a.div_nvel = make_fastdiv(unsigned(a.nvel > 0 ? a.nvel : 1));
+    set_draws(a, zf);
     const size_t smem = pair16_smem(a);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;

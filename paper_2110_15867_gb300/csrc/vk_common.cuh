@@ -296,18 +296,22 @@ __device__ __forceinline__ unsigned sr_bits(unsigned long long elem, unsigned se
 
 __device__ __forceinline__ unsigned lcg_next(unsigned &x)
 {
-    x = x * 1664525u + 1013904223u;
+    constexpr Lcg step = kLcg;
+    x = step(x);
     return x;
 }
 
-
-// Two non-negative FP32 values -> packed bf16x2 with stochastic rounding: the upper 16
-// bits of two LCG steps are added below the BF16 mantissa of x and of y, and one byte
-// permute packs the two upper halves.
+// Two non-negative FP32 values -> packed bf16x2 with stochastic rounding: 16 random bits (of
+// two LCG steps) are added below the BF16 mantissa of x and of y, and one byte permute packs
+// the two upper halves.
+__device__ __forceinline__ unsigned sr_pack_bf16x2(float x, float y, unsigned r1, unsigned r2)
+{
+    return __byte_perm(__float_as_uint(x) + r1, __float_as_uint(y) + r2, 0x7632);
+}
 __device__ __forceinline__ unsigned sr_pack_bf16x2(float x, float y, unsigned &rng)
 {
     const unsigned r1 = lcg_next(rng) >> 16, r2 = lcg_next(rng) >> 16;
-    return __byte_perm(__float_as_uint(x) + r1, __float_as_uint(y) + r2, 0x7632);
+    return sr_pack_bf16x2(x, y, r1, r2);
 }
 
 // Line scales of the 16-bit codec.  coded_scale: the scale a refresh stores for a line
@@ -324,13 +328,17 @@ __device__ __forceinline__ float inv_scale(float s) { return s >= 0x1p-126f ? __
 // Two non-negative FP32 values -> packed f16x2 with stochastic rounding: 13 of the upper
 // 16 bits of two LCG steps are added below the FP16 mantissa (13 bits below FP32's), and
 // one round-toward-zero conversion packs both (x in the lower half).
-__device__ __forceinline__ unsigned sr_pack_f16x2(float x, float y, unsigned &rng)
+__device__ __forceinline__ unsigned sr_pack_f16x2(float x, float y, unsigned r1, unsigned r2)
 {
-    const unsigned r1 = (lcg_next(rng) >> 16) & 0x1fffu, r2 = (lcg_next(rng) >> 16) & 0x1fffu;
-    const float xr = __uint_as_float(__float_as_uint(x) + r1), yr = __uint_as_float(__float_as_uint(y) + r2);
+    const float xr = __uint_as_float(__float_as_uint(x) + (r1 & 0x1fffu)), yr = __uint_as_float(__float_as_uint(y) + (r2 & 0x1fffu));
     unsigned out;
     asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(out) : "f"(yr), "f"(xr));
     return out;
+}
+__device__ __forceinline__ unsigned sr_pack_f16x2(float x, float y, unsigned &rng)
+{
+    const unsigned r1 = lcg_next(rng) >> 16, r2 = lcg_next(rng) >> 16;
+    return sr_pack_f16x2(x, y, r1, r2);
 }
 
 // ----------------------------------------------------------------------------

@@ -315,6 +315,21 @@ cudaError_t launch_shift32(const CUtensorMap &map, const CUtensorMap &dmap, cons
 // with box {32, 8, L, 1} (no swizzle), smap the scales as [n_outer][L][n_inner / n_uz] with
 // box {scale_lines, L, 1}
 // ----------------------------------------------------------------------------
+// The random streams of stochastic rounding: x -> 1664525 x + 1013904223 (Numerical Recipes'
+// generator), its inverse and its powers.
+struct Lcg {
+    unsigned mul, add;
+    constexpr unsigned operator()(unsigned x) const { return mul * x + add; }
+};
+constexpr Lcg kLcg{1664525u, 1013904223u};
+constexpr Lcg kLcgBack{4276115653u, 0u - 4276115653u * 1013904223u};
+static_assert(kLcg.mul * kLcgBack.mul == 1u, "inverse of the generator's multiplier");
+constexpr Lcg lcg_power(Lcg f, int n)
+{
+    Lcg r{1u, 0u};
+    for (; n > 0; --n) r = Lcg{f.mul * r.mul, f.mul * r.add + f.add};
+    return r;
+}
 struct Tile16Args {
     int L, nuz;
     long long n_inner;
@@ -326,6 +341,11 @@ struct Tile16Args {
     long long vstride;               // column j takes table[(inner / vstride) % nvel]
     int nvel;
     unsigned seed;                   // the stochastic-rounding streams of this sweep
+    // set by the launcher: a pair's streams, by the direction of its walk.  The first draws of its
+    // columns come from the states x(seed), y(seed) of the pair (own: of each column) and the next
+    // row's are one step on.
+    bool own;
+    struct Draws { Lcg x, y, step; } draws[2];
     unsigned *err;
     const LineCoefT<float> *cell_coef; // u_x sweep: the Courant numbers per outer index (a cell), else null
     FastDivU32 div_tiles, div_nuz, div_vstride, div_nvel; // set by the launcher

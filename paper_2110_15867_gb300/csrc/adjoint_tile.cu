@@ -345,7 +345,7 @@ cudaError_t launch_adjoint_tile(const CUtensorMap &fmap, const CUtensorMap &lmap
     a.div_vstride = make_fastdiv(unsigned(a.vstride));
     a.div_nvel = make_fastdiv(unsigned(a.nvel));
     const size_t smem = adjoint_tile_smem(a);
-    const cudaError_t e = cudaFuncSetAttribute(adjoint_tile(a.cols), cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = allow_smem(adjoint_tile(a.cols), smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = a.num_tiles < unsigned(sms) ? a.num_tiles : unsigned(sms);
     void *params[] = {const_cast<CUtensorMap *>(&fmap), const_cast<CUtensorMap *>(&lmap), &a};

@@ -669,7 +669,7 @@ int occupancy_kick_cube(int nu, int dtype)
     const void *k = kick_kernel_for(nu, dtype);
     if (!k) return 0;
     const size_t smem = kick_cube_smem(nu, dtype);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     const int threads = nu == 32 ? threads_for<32>() : threads_for<16>();
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
@@ -685,7 +685,7 @@ cudaError_t launch_kick_cube(const CUtensorMap &fmap, const CUtensorMap &smap, c
     // row coordinates of the tensor maps are 32-bit
     if ((a.cell0 + a.ncells) * (long long)nu * nu > 0x7fffffffll) return cudaErrorInvalidValue;
     const size_t smem = kick_cube_smem(nu, dtype);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     KickArgs args = a;
     void *params_f32[] = {const_cast<CUtensorMap *>(&fmap), &args};

@@ -328,8 +328,7 @@ bool plane_tail_supported(int nuy, int nuz, int nux, int dtype)
 
 template <typename T> static cudaError_t launch_plane_tail_t(T *f, const PlaneTailArgs &a, long long blocks, cudaStream_t st)
 {
-    const cudaError_t e = cudaFuncSetAttribute(plane_tail_kernel<48, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(PlaneGeom<48>::smem));
+    const cudaError_t e = allow_smem((const void *)plane_tail_kernel<48, T>, PlaneGeom<48>::smem);
     if (e != cudaSuccess) return e;
     return launch_chained_t(a.nplanes * 48 * 48, plane_tail_kernel<48, T>, dim3(unsigned(blocks)), dim3(PlaneGeom<48>::threads), PlaneGeom<48>::smem,
                             st, f, a);
@@ -369,7 +368,7 @@ cudaError_t launch_plane_any(const float *src, float *dst, const PlaneAnyArgs &a
     a.div_hy = make_fastdiv(unsigned(a.nuy / 2));
     a.div_nux = make_fastdiv(unsigned(a.nux));
     const size_t smem = a.per_block * plane;
-    const cudaError_t e = cudaFuncSetAttribute(plane_any_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = allow_smem((const void *)plane_any_kernel, smem);
     if (e != cudaSuccess) return e;
     const long long blocks = (a.nplanes + a.per_block - 1) / a.per_block;
     return launch_chained_t(a.nplanes * a.nuy * a.nuz, plane_any_kernel, dim3(unsigned(blocks)), dim3(kAnyThreads), smem, st, src, dst, a);

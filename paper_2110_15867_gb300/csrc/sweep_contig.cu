@@ -146,7 +146,7 @@ static cudaError_t launch_contig_t(const CUtensorMap &map, const CUtensorMap &dm
                                    int grid, size_t smem, cudaStream_t st)
 {
     auto kern = contig_sweep_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, kConsumers + kProducer, smem, st>>>(map, dmap, a);
     return cudaGetLastError();
@@ -161,7 +161,7 @@ cudaError_t launch_contig_f64(const CUtensorMap &map, const CUtensorMap &dmap, c
 int occupancy_contig(size_t smem)
 {
     const void *k = (const void *)contig_sweep_kernel<double>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess) return 0;
     return n;

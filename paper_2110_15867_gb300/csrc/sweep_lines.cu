@@ -421,8 +421,7 @@ static cudaError_t launch_rows_t(const void *src, void *dst, const RowsArgs &a, 
 {
     const long long blocks = (a.nrows + 255) / 256;
     if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(rows_sweep_kernel<NU, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(rows_sweep_smem<NU, T>()));
+    const cudaError_t e = allow_smem((const void *)rows_sweep_kernel<NU, T>, rows_sweep_smem<NU, T>());
     if (e != cudaSuccess) return e;
     rows_sweep_kernel<NU, T><<<unsigned(blocks), 256, rows_sweep_smem<NU, T>(), st>>>(static_cast<const T *>(src),
                                                                                      static_cast<T *>(dst), a);
@@ -496,7 +495,7 @@ cudaError_t launch_line_sweep(const CUtensorMap &map, const CUtensorMap &dmap, c
     a.div_rpc = make_fastdiv(unsigned(a.rows_per_cell));
     const void *k = line_kernel_for(nu, dtype, fuse_y);
     const size_t smem = line_sweep_smem(nu, dtype == 1 ? 4 : 2, fuse_y);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
     const int threads = kLine1Threads + kProducer;
@@ -507,7 +506,7 @@ int occupancy_line_sweep(int nu, int dtype, bool fuse_y)
 {
     const void *k = line_kernel_for(nu, dtype, fuse_y);
     const size_t smem = line_sweep_smem(nu, dtype == 1 ? 4 : 2, fuse_y);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     const int threads = kLine1Threads + kProducer;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;

@@ -191,7 +191,7 @@ bool pair32_geometry(int L, long long n_inner, long long n_outer, Pair32Args &a)
 int occupancy_pair32(const Pair32Args &a, bool zf)
 {
     const size_t smem = pair32_smem(a);
-    if (cudaFuncSetAttribute(pair32(zf), cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(pair32(zf), smem) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pair32(zf), a.groups * kGroup + kProducer, smem) != cudaSuccess) return 0;
     return n;
@@ -210,7 +210,7 @@ cudaError_t launch_pair32(const CUtensorMap &map, const CUtensorMap &dmap, const
     a.div_vstride = make_fastdiv(unsigned(a.vstride > 0 ? a.vstride : 1));
     a.div_nvel = make_fastdiv(unsigned(a.nvel > 0 ? a.nvel : 1));
     const size_t smem = pair32_smem(a);
-    cudaError_t e = cudaFuncSetAttribute(pair32(zf), cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(pair32(zf), smem);
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
     return launch_chained((long long)a.num_tiles * kCols * a.L, pair32(zf), dim3(grid), dim3(a.groups * kGroup + kProducer), smem, st, params);

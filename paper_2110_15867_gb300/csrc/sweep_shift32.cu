@@ -146,7 +146,7 @@ cudaError_t launch_shift32(const CUtensorMap &map, const CUtensorMap &dmap, cons
     a.div_nvel = make_fastdiv(unsigned(a.nvel));
     const size_t smem = kHead + 128 + size_t(a.slots) * a.L * kRow;
     const void *kern = a.rotate ? (const void *)shift32_kernel<true> : (const void *)shift32_kernel<false>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), &a};
     return launch_chained((long long)a.num_tiles * kCols * a.L, kern, dim3(grid),

@@ -561,7 +561,7 @@ static cudaError_t launch_stream_t(const CUtensorMap &map, const CUtensorMap &dm
             kern = stream_sweep_kernel<T, true, true>; // the x sweep with the moment
             threads = Lane<T>::NC + stream_head<true>();
         }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     return launch_chained_t(a.num_blocks * a.W * a.P * a.L * (sizeof(T) == 8 ? 16 : 1), kern, dim3(grid), dim3(threads), smem, st, map, dmap, smap, a);
 }
@@ -604,7 +604,7 @@ int occupancy_stream(int dtype, int periodic, size_t smem)
                     : dtype == 1 ? stream_ptr<float>(periodic)
                     : dtype == 2 ? stream_ptr<__nv_bfloat16>(periodic)
                                  : stream_ptr<__half>(periodic);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, stream_consumers(dtype) + kProducer, smem) != cudaSuccess)
         return 0;

@@ -159,7 +159,7 @@ static cudaError_t launch_strided_t(const CUtensorMap &map, const CUtensorMap &d
                                     int grid, size_t smem, cudaStream_t st)
 {
     auto kern = strided_sweep_kernel<T, ROT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, kConsumers + kProducer, smem, st>>>(map, dmap, a);
     return cudaGetLastError();
@@ -182,7 +182,7 @@ int occupancy_strided(int dtype, size_t smem) // of the kernel that fits fewer C
 {
     auto fit = [&](const void *k) {
         int n = 0;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+        if (allow_smem(k, smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kConsumers + kProducer, smem) != cudaSuccess)
             return 0;
         return n;

@@ -284,7 +284,7 @@ int occupancy_tile_sweep(int L, bool moment)
     const void *k = tile_kernel_for(L, moment);
     if (!k) return 0;
     const size_t smem = tile_smem_for(L);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, tile_threads_for(L), smem) != cudaSuccess) return 0;
     return n;
@@ -299,7 +299,7 @@ cudaError_t launch_tile_sweep(const CUtensorMap &map, const CUtensorMap &dmap, c
         return cudaErrorInvalidValue;
     if (moment && (a.cube % 256 || a.nparts <= 0)) return cudaErrorInvalidValue;
     const size_t smem = tile_smem_for(a.L);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&dmap), const_cast<TileArgs *>(&a)};
     return launch_chained(a.num_tiles * 256 * a.L, k, dim3(grid), dim3(tile_threads_for(a.L)), smem, st, params);

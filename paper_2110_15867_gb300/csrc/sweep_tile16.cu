@@ -294,7 +294,7 @@ int occupancy_tile16(const Tile16Args &a, int dtype, bool zf)
     const void *k = pair16_kernel(dtype, zf);
     if (!k) return 0;
     const size_t smem = pair16_smem(a);
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess) return 0;
+    if (allow_smem(k, smem) != cudaSuccess) return 0;
     int n = 0;
     const int threads = a.groups * kPairGroup + kProducer;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
@@ -336,7 +336,7 @@ cudaError_t launch_tile16(const CUtensorMap &map, const CUtensorMap &smap, const
     a.div_nvel = make_fastdiv(unsigned(a.nvel > 0 ? a.nvel : 1));
     set_draws(a, zf);
     const size_t smem = pair16_smem(a);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     void *params[] = {const_cast<CUtensorMap *>(&map), const_cast<CUtensorMap *>(&smap), &a};
     return launch_chained((long long)a.num_tiles * 256 * a.L, k, dim3(grid), dim3(a.groups * kPairGroup + kProducer), smem, st, params);

@@ -86,6 +86,16 @@ template <typename C> __host__ __device__ inline LineCoefT<C> make_line_coef(dou
     return k;
 }
 
+// Before a launch (or an occupancy query) with `smem` bytes of dynamic shared memory.  The limit is a
+// property of the kernel and the device, not of a launch: it is always set to the device's most,
+// so that a thread whose grid needs less cannot lower it between another's call and launch.
+inline cudaError_t allow_smem(const void *kernel, size_t smem)
+{
+    constexpr int kMost = 227 * 1024; // (none of these kernels has static shared memory beside it)
+    if (smem > size_t(kMost)) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+}
+
 // ----------------------------------------------------------------------------
 // strided sweep (axes x, y, z; whole-cell shifts)
 // ----------------------------------------------------------------------------

@@ -665,11 +665,11 @@ cudaError_t launch_poisson(const GridDims &g, const PoissonScratch &ps, const do
     A.phi = phi;
     A.phi64 = phi64;
     cudaError_t err = cudaSuccess;
-    // Chained only up to 2^13 spatial cells (and kChainCells in all): more blocks than one per SM
-    // or so, and those of the next launch sit on the SMs while FP64 sums still run (chained /
-    // not: 6^3 22 / 35 us, 53 x 6^2 46 / 60, 21 x 26 x 19 51 / 49, 59 x 30 x 8 77 / 68, 32^3 99 / 65,
-    // 31 x 37 x 43 531 / 188).
-    const long long cells = n <= 8192 ? n * g.nu[0] * g.nu[1] * g.nu[2] : kChainCells + 1;
+    // Chained only up to 2^12 spatial cells (and kChainCells in all): of more, the blocks of the next
+    // launch sit on the SMs while FP64 sums still run.  Chained / not: steps of 8^3 x 16^3 cells 81 / 92
+    // us, 16^3 x 8^3 99 / 108, 16^3 x 16^3 264 / 274, but 31 x 13 x 11 x 8^3 170 / 132, 20^3 x 8^3 172 / 146 (20^3
+    // x 12^3 363 / 372); the solve alone 32^3 99 / 65, 31 x 37 x 43 531 / 188.
+    const long long cells = n <= 4096 ? n * g.nu[0] * g.nu[1] * g.nu[2] : kChainCells + 1;
     auto dft = [&](auto kernel, int d, int sign, const double2 *in, double2 *out) {
         const int nd = g.n[d]; // <= 256
         A.nlines = unsigned(n / nd);

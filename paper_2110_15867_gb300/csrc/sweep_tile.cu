@@ -250,7 +250,9 @@ const void *tile_kernel_for(int L, bool moment, bool sign = true)
     switch (L) {
     case 16: return tile_kernel<16>(moment, sign);
     case 24: return tile_kernel<24>(moment, sign);
-    case 32: return tile_kernel<32>(moment, sign);
+    case 32: // (without the moment these lines march two per thread, sweep_pair32.cu)
+        if (!moment) return nullptr;
+        return sign ? (const void *)tile_sweep_kernel<32, true, true> : (const void *)tile_sweep_kernel<32, true, false>;
     case 48: return tile_kernel<48>(moment, sign);
     case 64: return tile_kernel<64>(moment, sign);
     default: return nullptr;
@@ -275,7 +277,7 @@ const void *tile_kernel_zf(int L) { return L == 48 ? (const void *)tile_sweep_ke
 
 } // namespace
 
-bool tile_sweep_supported(int L, long long n_inner) { return n_inner % 256 == 0 && tile_kernel_for(L, false) != nullptr; }
+bool tile_sweep_supported(int L, long long n_inner) { return n_inner % 256 == 0 && tile_kernel_for(L, true) != nullptr; }
 
 bool tile_sweep_zf_supported(int L, long long n_inner) { return n_inner % 256 == 0 && tile_kernel_zf(L) != nullptr; }
 

@@ -285,8 +285,8 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
     const size_t kSmemBudget = 200 * 1024;
     const bool coded = c->g.dtype == VLASOV_BF16 || c->g.dtype == VLASOV_F16;
     // whole-line kernels (whole-cell shifts, u_z lines of other lengths): FP32 / FP64 only
-    for (int ax = 0; ax < 6 && !coded; ++ax) {
-        if (!(mask >> ax & 1)) continue;
+    for (int ax : {0, 1, 2, 5}) {
+        if (coded || !(mask >> ax & 1)) continue;
         AxisPlan &p = c->plan[ax];
         p.L = int(d6[ax]);
         long long I = 1, O = 1;
@@ -295,7 +295,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
         p.n_inner = I;
         p.n_outer = O;
         CUresult r;
-        if (ax < 5) {
+        if (ax < 3) {
             // A tile of W x P lines, one per consumer thread, in a ring of 2 to 4.  The tile that lets an
             // SM march most lines at a time is taken (of equal ones the largest, whose lines
             // spread over more warps): CTAs an SM by shared memory, at most by registers, times
@@ -303,7 +303,7 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             // here; 112 x 16 x 200 x 8^2 x 12, lines of 200: 2258, 886; FP64 lines of 200: 41.6 ms,
             // 20.9) and tiles of at most 36 KB (FP64 64 x 48 x 24 x 12^2 x 16, lines of 48: 7.24 ms,
             // 5.43; FP32 200 x 120 x 160 x 4^3, lines of 160: 1399, 1052 us).
-            const size_t tab = ax < 3 ? ((sizeof(LineCoefT<double>) * kMaxVel + 127) & ~size_t(127)) : 0;
+            const size_t tab = (sizeof(LineCoefT<double>) * kMaxVel + 127) & ~size_t(127);
             int W = 0, P = 0, S = 0;
             for (int lines = kConsumers, best = 0; lines >= 32; lines /= 2) {
                 const int w = I < lines ? int(I) : lines;
@@ -330,31 +330,27 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             const int occ = occupancy_strided(c->g.dtype == VLASOV_F64 ? 0 : 1, p.smem);
             if (occ <= 0) return fail(c, VLASOV_ECUDA, "axis %d: a CTA does not fit (%zu B shared memory)", ax, p.smem);
             p.grid = int(p.num_tiles < (long long)occ * c->sm_count ? p.num_tiles : (long long)occ * c->sm_count);
+        } else if (c->g.dtype == VLASOV_F32) {
+            // the line kernel or planes; longer rows are refused, as since the kernel that transposed
+            // them could not hold more
+            if (p.L > 72) return fail(c, VLASOV_ECUDA, "axis 5: FP32 rows of %d cells (at most 72)", p.L);
+            continue;
         } else {
-            const long long rows = O * 1; // one row per (cell, jx, jy)
+            // FP64 rows: the transposing kernel, but for those of 24, 40 or 48 cells
+            if (rows_sweep_supported(p.L, c->g.dtype)) continue;
             p.W = p.L;
             p.P = kConsumers; // rows per tile
-            p.n_outer = rows;
-            p.num_tiles = (rows + kConsumers - 1) / kConsumers;
+            p.num_tiles = (O + kConsumers - 1) / kConsumers;
             p.tiles_inner = 1;
-            const size_t ces = c->g.dtype == VLASOV_F64 ? 8 : 4;
-            const size_t tile = ((size_t)p.L * kConsumers * es + 127) & ~size_t(127);
-            const size_t bbuf = (size_t)p.L * (kConsumers + 1) * ces;
+            const size_t tile = ((size_t)p.L * kConsumers * 8 + 127) & ~size_t(127);
+            const size_t bbuf = (size_t)p.L * (kConsumers + 1) * 8;
             int S = int((kSmemBudget - 128 - bbuf) / tile);
             S = S < 2 ? 2 : (S > 4 ? 4 : S);
             p.stages = S;
             p.smem = 128 + (size_t)S * tile + bbuf;
-            p.spec = spec_rows(tmap_type(c->g.dtype), p.L, rows, es, kConsumers, CU_TENSOR_MAP_SWIZZLE_NONE);
+            p.spec = spec_rows(tmap_type(c->g.dtype), p.L, O, es, kConsumers, CU_TENSOR_MAP_SWIZZLE_NONE);
             r = encode_spec(&p.map, p.spec, c->f);
-            // only FP64 rows other than 24, 40 or 48 cells take the transposing kernel; FP32 grids
-            // whose rows it could not have held stay refused
-            const bool fits = p.smem <= 227 * 1024;
-            const int occ = c->g.dtype == VLASOV_F64 ? occupancy_contig(p.smem) : fits;
-            if (occ <= 0 && (c->g.dtype == VLASOV_F32 ? c->g.nuz == 24 || c->g.nuz == 40 || c->g.nuz == 48
-                                                      : rows_sweep_supported(int(c->g.nuz), c->g.dtype))) {
-                p.grid = 0;
-                continue;
-            }
+            const int occ = occupancy_contig(p.smem);
             if (occ <= 0) return fail(c, VLASOV_ECUDA, "axis 5: a CTA does not fit (%zu B shared memory)", p.smem);
             p.grid = int(p.num_tiles < (long long)occ * c->sm_count ? p.num_tiles : (long long)occ * c->sm_count);
         }
@@ -898,11 +894,12 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         if (e != cudaSuccess) return cuda_fail(c, e, "position sweep launch");
         return VLASOV_OK;
     }
-    // FP32: lines of 32 cells march faster two per thread (32^3 x 32^3: 1.31 ms a sweep against
-    // 1.44; lines of 16, 24, 48 and 64 within 7 % either way), unless the x sweep sums the moment
-    const bool pairs_first = c->p32_ok[ax] && (&c->g.nx)[ax] == 32 &&
-                             !(rho_fused && ax == 0 && c->fuse_moment && velocity_cube(c) % 256 == 0);
-    if (numax < 1.0 && c->use_tiles && c->tile_ok[ax] && !pairs_first) {
+    // FP32: the x sweep sums the moment on the one-line tiles.  Lines of 32 cells march faster two per
+    // thread otherwise (32^3 x 32^3: 1.31 ms a sweep against 1.44; lines of 16, 24, 48 and 64 within 7 %
+    // either way)
+    const bool tile_moment = numax < 1.0 && c->use_tiles && c->tile_ok[ax] && rho_fused && ax == 0 && c->fuse_moment &&
+                             velocity_cube(c) % 256 == 0 && moment_buffer(c);
+    if (numax < 1.0 && c->use_tiles && c->tile_ok[ax] && ((&c->g.nx)[ax] != 32 || tile_moment)) {
         // the same on FP32 storage
         TileArgs A{};
         A.L = (&c->g.nx)[ax];
@@ -931,7 +928,7 @@ static int run_position(vlasov_ctx *c, int ax, double dt, double a, const void *
         A.err = c->d_err;
         for (int j = 0; j < nvel; ++j) A.table[j] = make_line_coef<float>((-c->g.V + (j + 0.5) * du) * dt / (a * a * dx));
         const long long cube = velocity_cube(c);
-        const bool fm = rho_fused && ax == 0 && c->fuse_moment && cube % 256 == 0 && moment_buffer(c);
+        const bool fm = tile_moment;
         if (fm) { A.mpart = c->d_mpart; A.cube = cube; A.nparts = int(cube / 256); }
         if ((rc = sweep_maps(c, c->tmap[ax], c->tspec[ax], src, dst, m))) return rc;
         cudaError_t e;

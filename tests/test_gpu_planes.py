@@ -58,3 +58,13 @@ def test_planes(n, nu):
         close(f, ref, 3)
         out.append(f)
     assert torch.equal(out[0], out[1])
+
+
+def test_rows_of_more_than_72_cells_are_refused():
+    from paper_2110_15867_gb300 import binding as B
+    B.load()
+    with pytest.raises(B.VlasovError, match="axis 5"):
+        B.Vlasov(torch.zeros((4, 4, 4, 4, 4, 76), device="cuda"), V=5.0)
+    # and leave no error behind for the next call
+    codes, scale = B.encode_lines(torch.rand((5, 16), device="cuda"), torch.bfloat16)
+    assert (scale > 0).all()

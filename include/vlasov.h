@@ -166,10 +166,11 @@ int vlasov_set_fused_kick(vlasov_ctx *ctx, int mode);
 int vlasov_kick(vlasov_ctx *ctx, double dt, const float *phi_dev);
 
 /*
- * Staged tiles.  Position sweeps (Eq. 3, |nu| < 1) with lines of 9 to about 100
+ * Staged tiles.  Position sweeps (Eq. 3, |nu| < 1) with lines of up to about 100
  * cells (BF16 / FP16: of 4 to about 100, and a multiple of 256 cells on the faster axes)
  * run with whole lines staged in shared memory: each tile of 128 or 256 lines x all their
- * cells is loaded once, marched there and stored once.  So does the u_x sweep (Eq. 4) on
+ * cells is loaded once, marched there and stored once (FP32 lines of up to 8 cells: on small
+ * grids only).  So does the u_x sweep (Eq. 4) on
  * [cell][u_x][u_y u_z], but lines of 16 cells (BF16 / FP16: of 16 and 32, and with n_uy n_uz
  * a multiple of 256).  FP32 results equal the streamed and register-line sweeps bit for
  * bit.  16-bit results draw the rounding streams of those sweeps, one per two columns or

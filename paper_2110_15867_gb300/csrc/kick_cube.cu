@@ -37,8 +37,7 @@ template <int NU, typename T> struct Cube {
 // ALU pipe 60 % and issue 65 % busy; the DRAM traffic alone would take 1.27 ms).  Read from
 // global memory by every thread when they were needed, the coefficients cost 8 % of that;
 // cells read no further ahead than the window, 3 %.
-// The kick is bound by instruction issue and by the ALU pipe (min / max at half rate), not
-// by DRAM.  A thread marches two lines at once, their sums and products as f32x2 (one issue
+// The kick is bound by its marches, not by DRAM; min / max run at half rate on the ALU pipe.  A thread marches two lines at once, their sums and products as f32x2 (one issue
 // slot for two), through a window of a few cells (vk_common.cuh, March), reading each cell
 // once and writing it back in place, so that 512 threads cover all 1024 lines of a 32^3
 // cube in one go at about 100 registers: 16 warps per SM keep both pipes busy.  (Whole pairs

@@ -1,22 +1,23 @@
-// plane_tail.cu -- the tail D_uz D_uy of a kick (Eq. 4 for i = 2, 3) in one pass over
-// f for velocity cubes too large for one CTA (n_uy = n_uz = 48).
+// plane_tail.cu -- the tail D_uz D_uy of a kick (Eq. 4 for i = 2, 3) in one pass over f: for
+// velocity cubes too large for one CTA (n_uy = n_uz = 48, FP32 and 16-bit storage, sizes fixed at
+// compile time), and on FP32 grids of other sizes, where D_uy or D_uz alone may also run here (the
+// second half of this file).
 //
 // A (cell, j_x) plane of the velocity cube holds n_uy rows (j_y) of n_uz cells (j_z),
 // contiguous in f (Listing 1: u_z innermost), and both sweeps stay inside it.  A
 // block stages four planes of one spatial cell in shared memory, sweeps them along u_y, then
 // along u_z, and writes them back: f is read and written once for the two sweeps.
 //
-// The pass is bound by the marches (instruction issue and the ALU pipe), not by DRAM, so a
+// The pass is bound by the marches, not by DRAM, so a
 // thread marches two lines at once, sums and products as f32x2 pairs (vk_common.cuh), through
 // a window of a few cells, reading each cell once and writing it back in place: D_uy two
 // adjacent columns (one 8-byte access per row), D_uz rows l and l + n_uy / 2 in 16-byte
 // chunks.  Rows are padded to n_uz + 4 floats, an odd number of 16-byte units: eight rows
 // read at one chunk fall on different banks.  FP32 rows come in by 16-byte asynchronous
 // copies (a bulk copy per row costs more instructions: one thread of a warp at a time issues
-// it).  Faces in
-// blocks of 8 (D_uy) and 4 (D_uz): blocks of 23 and 20 faces missed in the instruction cache
-// (3.6 fetch stalls per issue, 20 % slower).  The arithmetic is march_regs' in the same order: FP32 results equal the separate
-// sweeps bit for bit.
+// it).  Faces in blocks of 8 (D_uy) and 4 (D_uz): blocks of 23 and 20 faces missed in the
+// instruction cache (3.6 fetch stalls per issue, 20 % slower).  The arithmetic is march_regs' in
+// the same order: FP32 results equal the separate sweeps bit for bit.
 // 24^3 x 48^3 cells, per kick tail: FP32 4.84 ms with one line per thread, 3.2 ms here (52
 // instructions per face pair, issue 61 % and ALU pipe 56 % busy; DRAM alone 1.8 ms), FP16
 // 4.90 -> 3.5 ms.
@@ -193,8 +194,8 @@ __global__ void __launch_bounds__(PlaneGeom<NU>::threads, 5)
 // ----------------------------------------------------------------------------
 // planes of any size (FP32): D_uy, D_uz or both in one pass, in place or src -> dst
 // ----------------------------------------------------------------------------
-// The same marches with the sizes at run time, for every velocity grid that the kernels of
-// fixed sizes do not take.  A block stages as many whole planes as give its 128 threads a
+// The same marches with the sizes at run time, for the velocity grids that the kernels of
+// fixed sizes do not take (both sweeps in one pass up to n_uy = 4 n_uz).  A block stages as many whole planes as give its 128 threads a
 // pair of lines each (of whatever cells: each pair looks up its own Courant number); the
 // rows' pitch is an odd number of 16-byte units.  Bodies of four faces, whose look-ahead
 // cells are read before the first of their writes.

@@ -4,13 +4,14 @@
 // The tiles, the ring and its producer are those of sweep_pair32.cu (tiles of 128 columns, a
 // group of threads per tile); each thread marches two adjacent lines down and writes every cell
 // in its shifted place (march_shift_down, vk_shift.cuh), so lines may shift by different numbers
-// of cells.
+// of cells.  When some line shifts by more cells than a thread can hold back, all lines of the sweep are
+// marched in place and rotated (whole_cell_rotate).
 //
-// Against one line per thread in three CTAs of 8 warps an SM (sweep_strided.cu, whose warps wait
-// for each other at every tile, and 64-bit divisions per line): 32 x 24 x 32 x 16 x 16 x 32 cells
+// Against one line per thread in three CTAs of 8 warps an SM (sweep_strided.cu with tiles of 36 KB, whose
+// warps wait for each other at every tile, and 64-bit divisions per line): 32 x 24 x 32 x 16 x 16 x 32 cells
 // (DRAM alone 0.238 ms a sweep) x, y, z 0.386, 0.412, 0.389 -> 0.335, 0.355, 0.340 ms, 16^3 x 32^3
-// 0.311 -> 0.268 (0.159); one line per thread in this ring 0.352, 0.375, 0.355 and 0.286.  Bound by the
-// ALU pipe and issue: the flux in the cells themselves takes 28 ALU cycles a line and face.
+// 0.311 -> 0.268 (0.159); one line per thread in this ring 0.352, 0.375, 0.355 and 0.286.  Bound by
+// the marches: the flux in the cells themselves takes 28 ALU cycles a line and face.
 #include "vk_shift.cuh"
 #include "vk_tiles.cuh"
 

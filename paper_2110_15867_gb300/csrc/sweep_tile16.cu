@@ -8,8 +8,7 @@
 // u_z lines.  These sweeps keep every scale: a value is decoded as code x scale (a rounded
 // product), its line marched in FP32 and the result encoded with stochastic rounding.
 //
-// They are bound by instruction issue and the ALU pipe, not by DRAM (4 bytes a cell and
-// pass).  A thread takes two adjacent columns, which always share their u_z line and the
+// They are bound by the marches and the codec, not by DRAM (4 bytes a cell and pass).  A thread takes two adjacent columns, which always share their u_z line and the
 // sign of their Courant number: one 4-byte access, one scale and one inverse scale serve
 // two cells, and the march's sums and products run as f32x2 pairs (March<float2>).  Groups
 // of 128 threads march different tiles of a ring that one producer thread keeps full.  The
@@ -231,13 +230,15 @@ __global__ void __launch_bounds__(kPairGroups *kPairGroup + kProducer, 1)
             // the streams, from the index of the first cell of the pair or of each column
             const unsigned long long e = (unsigned long long)o * L * a.n_inner + inner;
             const unsigned seed = sr_bits(e, a.seed);
-            const PairDraws rng{a.draws[neg].x(seed), a.draws[neg].y(a.own ? sr_bits(e + 1, a.seed) : seed), a.draws[neg].step};
+            const unsigned seed2 = a.own ? sr_bits(e + 1, a.seed) : seed;
+            // (a fixed index keeps the step in the constant bank)
+            auto rng = [&](int d) { return PairDraws{a.draws[d].x(seed), a.draws[d].y(seed2), a.draws[d].step}; };
             unsigned char *p = slot(k) + 4 * pair + far * 512;
             const float2 *s = ws + int(line - first) * L + far;
             float2 sum;
-            if (__all_sync(0xffffffffu, !neg)) sum = march_pair16<T, ZF, 1>(p, 0, s, 0, L, lim, rng);
-            else if (__all_sync(0xffffffffu, neg)) sum = march_pair16<T, ZF, -1>(p, 0, s, 0, L, lim, rng);
-            else sum = march_pair16<T, ZF, 0>(p, dir * 512, s, dir, L, lim, rng);
+            if (__all_sync(0xffffffffu, !neg)) sum = march_pair16<T, ZF, 1>(p, 0, s, 0, L, lim, rng(0));
+            else if (__all_sync(0xffffffffu, neg)) sum = march_pair16<T, ZF, -1>(p, 0, s, 0, L, lim, rng(1));
+            else sum = march_pair16<T, ZF, 0>(p, dir * 512, s, dir, L, lim, rng(neg));
             bad |= !(sum.x >= 0.f) || !(sum.y >= 0.f) || isinf(sum.x) || isinf(sum.y);
         }
         fence_proxy_async();

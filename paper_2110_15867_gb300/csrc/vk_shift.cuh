@@ -10,8 +10,8 @@ namespace vk {
 // operations a face) where every other kernel takes differences (31): over a drift of
 // whole-cell shifts the two forms' roundings, both right to 7e-8 of the 2-norm, were driven
 // apart in single cells by the limiter (3e-5 of the rms after six sweeps), more than these
-// sweeps' results may change, for 4 % of their time (32 x 24 x 32 x 16 x 16 x 32 cells: 1.665
-// against 1.597 ms, three sweeps).
+// sweeps' results may change.  What that costs was measured one line per thread: 4 % (32 x 24 x 32
+// x 16 x 16 x 32 cells: 1.665 against 1.597 ms, three sweeps); in pairs, now 1.020 ms, it is not known.
 // X = float: one line; float2: two lines as f32x2 pairs, the same operations one by one.
 template <typename X> struct CellCoef { // weights of fbar, Courant fraction, f_UL's factor
     X w[5], s, alpha;

@@ -493,12 +493,12 @@ static int plan_axes(vlasov_ctx *c, int mask = 0x3f)
             // Lines of up to 8 cells stream: a tile of them is a few KB, and its barriers and copies
             // outweigh its marches (16^3 velocity cubes, tiles / streamed: 4 cells 547 / 357 us, 6
             // 379 / 304, 8 298 / 280, 9 273 / 272, 12 217 / 233; u_x of 8 x 16^2 292 / 263, of 12 x 16^2
-            // 206 / 212).  But grids of few cells keep lines of 6 to 8 on tiles, where a block has one or two
-            // of each slot and a line's cells are in flight at once (2e6 cells, lines of 6 8.3 / 9.1, of 7
-            // 7.4 / 8.5, of 8 7.2 / 9.0 us; 4e6 cells 13.2 / 13.7, 11.3 / 12.9, 11.6 / 14.0; 8e6 cells 30.2 / 26.3,
-            // 24.2 / 24.3, 21.8 / 23.0); and y lines whose runs of one sign of u_y are shorter than a warp's 64
+            // 206 / 212).  But small grids keep them on tiles, whose lines' cells are all in flight at once
+            // (2e6 cells, lines of 6 8.3 / 9.1, of 7 7.4 / 8.5, of 8 7.2 / 9.0 us; 4e6 cells 13.2 / 13.7, 11.3 / 12.9,
+            // 11.6 / 14.0; 8e6 cells 30.2 / 26.3, 24.2 / 24.3, 21.8 / 23.0; lines of 4, 1e6 cells 6.8 / 6.6 but
+            // steps of 4^3 x 16^3 57 / 60); and y lines whose runs of one sign of u_y are shorter than a warp's 64
             // columns make streamed warps march both ways (8^3 cubes: 4 cells 547 / 592, 8 303 / 498).
-            const bool few = L >= 6 && O * L * I <= 1ll << 22, mixed = ax == 1 && d6[4] * d6[5] / 2 < 64;
+            const bool few = O * L * I <= 1ll << (L < 6 ? 20 : L < 8 ? 22 : 23), mixed = ax == 1 && d6[4] * d6[5] / 2 < 64;
             if (I >= pair32_columns() && (L > 8 || few || mixed) && pair32_geometry(L, I, O, c->p32[ax])) {
                 c->pspec[ax] = spec3(CU_TENSOR_MAP_DATA_TYPE_FLOAT32, I, L, O, 4, pair32_columns(), L, 1);
                 const int n = occupancy_pair32(c->p32[ax], ax == 3);

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kConsumers + kProducer)
     const bool has_col = tid < W * P;
     for (long long k = 0; k < n_my; ++k) {
         const int st = int(k % S);
-        if (!mbar_wait_bounded(&full[st], unsigned((k / S) & 1))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[st], unsigned((k / S) & 1)))) { // (a warp leaves together)
             atomicOr(args.err, ERR_TIMEOUT);
             break;
         }
